@@ -20,16 +20,8 @@
 
 namespace ols {
 
-#ifndef OLS_PACKED_ADD
-#define OLS_PACKED_ADD 1
-#endif
-#if OLS_PACKED_ADD
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
-#else
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-#endif
 
 // a + r b and a - r b with r = -i (forward) or +i (inverse): lanes cross, scalar adds.
 template <bool INV>

@@ -46,15 +46,6 @@
 #ifndef OLS_BWD_MINB_1024
 #define OLS_BWD_MINB_1024 2
 #endif
-#ifndef OLS_BWD_L2HINTS
-#define OLS_BWD_L2HINTS 1        // streamed s and g loads evict first, the per-CTA dh spectra evict last
-#endif
-#ifndef OLS_BWD_TW_TMEM
-#define OLS_BWD_TW_TMEM OLS_FWD_TW_TMEM   // twiddles and the window's signal spectrum A in TMEM
-#endif
-#ifndef OLS_BWD_PREFETCH
-#define OLS_BWD_PREFETCH 1       // pull the next gradient window toward L2 while this one is transformed
-#endif
 
 #ifndef OLS_BWD_XCHG
 #define OLS_BWD_XCHG 0
@@ -84,16 +75,11 @@ struct L2Hints {
 };
 
 __device__ __forceinline__ float2 ld_stream(const float2 *p, const L2Hints &h) {
-#if OLS_BWD_L2HINTS
     float2 v;
     asm volatile("ld.global.nc.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;"
                  : "=f"(v.x), "=f"(v.y)
                  : "l"(p), "l"(h.stream));
     return v;
-#else
-    (void)h;
-    return __ldg(p);
-#endif
 }
 
 // *p += v without waiting for the old value (an L2 reduction).  Only one
@@ -101,27 +87,15 @@ __device__ __forceinline__ float2 ld_stream(const float2 *p, const L2Hints &h) {
 // applied in program order, so the sum is deterministic; IEEE round to
 // nearest like an FP32 add.
 __device__ __forceinline__ void red_add(float4 *p, float4 v, const L2Hints &h) {
-#if OLS_BWD_L2HINTS
     asm volatile("red.global.add.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "f"(v.x), "f"(v.y),
                  "f"(v.z), "f"(v.w), "l"(h.keep)
                  : "memory");
-#else
-    (void)h;
-    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z),
-                 "f"(v.w)
-                 : "memory");
-#endif
 }
 
 __device__ __forceinline__ void st_keep(float4 *p, float4 v, const L2Hints &h) {
-#if OLS_BWD_L2HINTS
     asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "f"(v.x), "f"(v.y),
                  "f"(v.z), "f"(v.w), "l"(h.keep)
                  : "memory");
-#else
-    (void)h;
-    *p = v;
-#endif
 }
 
 template <int LOG2N>
@@ -133,10 +107,7 @@ struct BwdGeo {
     static constexpr int BLOCK = SLOTS * G::T;
     static_assert(SLOTS <= 15 || G::T <= 32, "one named barrier per slot");
     static constexpr int HALF = G::N / 2;      // float4 entries of one spectrum
-    // exchange buffers of every slot, then each slot's signal spectrum A (in
-    // TMEM instead with OLS_BWD_TW_TMEM)
-    static constexpr size_t XBYTES = sizeof(float2) * (size_t)SLOTS * G::XBUFS * G::PADN;
-    static constexpr size_t SMEM = XBYTES + (OLS_BWD_TW_TMEM ? 0 : sizeof(float4) * (size_t)SLOTS * HALF);
+    static constexpr size_t SMEM = sizeof(float2) * (size_t)SLOTS * G::XBUFS * G::PADN;   // exchange buffers
     static constexpr uint32_t TMEM_COLS = (uint32_t)(BLOCK / 128) * 128u;   // a 128-column lane range per 128 threads
     static_assert(G::XBUFS == 2, "the product buffer is the exchange buffer not in use");
 };
@@ -155,7 +126,6 @@ ols_backward_kernel(const float2 *__restrict__ sig, long long Ns, const float2 *
     float2 *const xbase = reinterpret_cast<float2 *>(smem_raw);
     float2 *bufs = xbase + slot * G::XBUFS * G::PADN;
     const SegmentBarrier<G::T> bar{1 + slot};
-#if OLS_BWD_TW_TMEM
     // the forward kernel's TMEM layout: the thread's twiddles, then (columns
     // 96..127) the window's signal spectrum A, in its own lane
     __shared__ uint32_t tbase;
@@ -169,10 +139,6 @@ ols_backward_kernel(const float2 *__restrict__ sig, long long Ns, const float2 *
     const TwTmemT<xch> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
     tw_tmem_fill<LOG2N, xch>(twg, tw.base, t);
     const uint32_t acol = tw.base + 96;
-#else
-    float4 *Asm = reinterpret_cast<float4 *>(reinterpret_cast<char *>(smem_raw) + BG::XBYTES) + slot * BG::HALF;
-    const TwGlobal tw{twg};
-#endif
     const L2Hints l2 = L2Hints::make();
     const int lo = M - 1;
     const int Li = (int)L;
@@ -195,15 +161,8 @@ ols_backward_kernel(const float2 *__restrict__ sig, long long Ns, const float2 *
                            ? ld_stream(sig + start + k * G::T + t, l2)
                            : make_float2(0.f, 0.f);
             forward_passes<LOG2N, 0>(A, bufs, tw, t, xc, bar);
-#if OLS_BWD_TW_TMEM
             tmem::st32(acol, reinterpret_cast<const float *>(A));
             tmem::wait_st();
-#else
-            // kept in shared memory (the thread's own entries) rather than 32 registers
-#pragma unroll
-            for (int j2 = 0; j2 < 8; ++j2)
-                Asm[j2 * G::T + t] = make_float4(A[2 * j2].x, A[2 * j2].y, A[2 * j2 + 1].x, A[2 * j2 + 1].y);
-#endif
         }
         float2 D[16];
         if constexpr (WANT_DS) {
@@ -222,7 +181,6 @@ ols_backward_kernel(const float2 *__restrict__ sig, long long Ns, const float2 *
                 b[k] = (k * G::T + t < gl && in_bounds(start + k * G::T + t < Nout, status))
                            ? ld_stream(gf + k * G::T, l2)
                            : make_float2(0.f, 0.f);
-#if OLS_BWD_PREFETCH
             // a window is at most N/16 = T lines of 128 B: one line per thread
             if (f + 1 < F) {
                 if (t * 16 < gl) prefetch_l2(gf - t + Nout + t * 16);
@@ -231,7 +189,6 @@ ols_backward_kernel(const float2 *__restrict__ sig, long long Ns, const float2 *
                 if (WANT_DH && nstart < Ns) prefetch_l2(sig + nstart);
                 if (nstart < Nout) prefetch_l2(g + nstart);
             }
-#endif
             forward_passes<LOG2N, 0>(b, bufs, tw, t, xc, bar);
             if constexpr (WANT_DS) {
                 const float4 *hp = Htk + (size_t)f * BG::HALF + t;
@@ -248,7 +205,6 @@ ols_backward_kernel(const float2 *__restrict__ sig, long long Ns, const float2 *
             if constexpr (WANT_DH) {
                 // B_f conj(A) at this thread's storage positions 16 t + j (entries j2 T + t)
                 float4 q[8];
-#if OLS_BWD_TW_TMEM
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {               // A in two 16-column halves
                     float a[16];
@@ -262,15 +218,6 @@ ols_backward_kernel(const float2 *__restrict__ sig, long long Ns, const float2 *
                         q[j2] = make_float4(q0.x, q0.y, q1.x, q1.y);
                     }
                 }
-#else
-#pragma unroll
-                for (int j2 = 0; j2 < 8; ++j2) {
-                    const float4 a = Asm[j2 * G::T + t];
-                    const float2 q0 = cmulc(b[2 * j2], make_float2(a.x, a.y));
-                    const float2 q1 = cmulc(b[2 * j2 + 1], make_float2(a.z, a.w));
-                    q[j2] = make_float4(q0.x, q0.y, q1.x, q1.y);
-                }
-#endif
                 float4 *Pf = Pc + (size_t)f * BG::HALF;
                 if constexpr (BG::SLOTS == 1) {
 #pragma unroll
@@ -320,12 +267,10 @@ ols_backward_kernel(const float2 *__restrict__ sig, long long Ns, const float2 *
             }
         }
     }
-#if OLS_BWD_TW_TMEM
     tmem::fence_before_sync();
     __syncthreads();
     tmem::fence_after_sync();
     if (threadIdx.x < 32) tmem::dealloc(tbase, BG::TMEM_COLS);
-#endif
 }
 
 // ds overlaps: ds[b L + u] = head_b[u] + tail_{b-1}[u] for b in [0, nseg],
@@ -434,11 +379,7 @@ static cudaError_t prepare_bwd_one(ols_plan_s &p, int idx) {
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BG::SMEM);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    if (OLS_BWD_TW_TMEM)
-        e = resident_blocks_tmem(ols_backward_kernel<LOG2N, DS, DH>, BG::BLOCK, BG::SMEM, (int)BG::TMEM_COLS, &per_sm);
-    else
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ols_backward_kernel<LOG2N, DS, DH>, BG::BLOCK,
-                                                          BG::SMEM);
+    e = resident_blocks_tmem(ols_backward_kernel<LOG2N, DS, DH>, BG::BLOCK, BG::SMEM, (int)BG::TMEM_COLS, &per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     p.bwd_grid_cap[idx] = per_sm * p.sm_count;

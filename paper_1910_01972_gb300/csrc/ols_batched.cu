@@ -44,7 +44,6 @@ ols_batched_kernel(const BatchProblemDev *__restrict__ probs, const int2 *__rest
     const int slot = threadIdx.x / G::T;
     const int t = threadIdx.x % G::T;
     float2 *bufs = smem + slot * G::XBUFS * G::PADN;
-#if OLS_FWD_TW_TMEM
     // twiddles in TMEM: warp 0 allocates, every thread fills its own lane
     if (threadIdx.x < 32) tmem::alloc(&tbase, G::TMEM_COLS);
     tmem::fence_before_sync();
@@ -54,10 +53,6 @@ ols_batched_kernel(const BatchProblemDev *__restrict__ probs, const int2 *__rest
     constexpr bool xch = in_tx_mask<LOG2N>(OLS_BATCH_PERN_TX_MASK);
     const TwTmemT<xch> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
     tw_tmem_fill<LOG2N, xch>(twg, tw.base, t);
-#else
-    (void)tbase;
-    const TwGlobal tw{twg};
-#endif
     int xc = 0;
     for (;;) {
         __syncthreads();                       // previous item_sh readers are done
@@ -70,14 +65,12 @@ ols_batched_kernel(const BatchProblemDev *__restrict__ probs, const int2 *__rest
         const long long nseg = P.nseg;
         const long long seg = (long long)it.y * G::SEGS + slot;
         ols_segment<LOG2N>(s_ptrs[P.index], P.Ns, P.Hk, tw, y_ptrs[P.index], P.M, P.F, P.L, P.Nout, seg,
-                           seg < nseg, bufs, t, xc, 0u, CtaBarrier{}, P.status);
+                           seg < nseg, bufs, t, xc, CtaBarrier{}, P.status);
     }
-#if OLS_FWD_TW_TMEM
     tmem::fence_before_sync();
     __syncthreads();
     tmem::fence_after_sync();
     if (threadIdx.x < 32) tmem::dealloc(tbase, G::TMEM_COLS);
-#endif
 }
 
 template <int LOG2N>
@@ -87,13 +80,10 @@ static cudaError_t batched_prepare_n(int sm_count, int *grid_cap, int *segs) {
                                          (int)G::SMEM_TMEM);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    if (OLS_FWD_TW_TMEM)
-        e = resident_blocks_tmem(ols_batched_kernel<LOG2N>, G::BLOCK, G::SMEM_TMEM, (int)G::TMEM_COLS, &per_sm);
-    else
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ols_batched_kernel<LOG2N>, G::BLOCK, G::SMEM_TMEM);
+    e = resident_blocks_tmem(ols_batched_kernel<LOG2N>, G::BLOCK, G::SMEM_TMEM, (int)G::TMEM_COLS, &per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    if (OLS_FWD_TW_TMEM && per_sm > G::TMEM_MAX_CTAS) per_sm = G::TMEM_MAX_CTAS;
+    if (per_sm > G::TMEM_MAX_CTAS) per_sm = G::TMEM_MAX_CTAS;
     *grid_cap = per_sm * sm_count;
     *segs = G::SEGS;
     return cudaSuccess;
@@ -159,7 +149,6 @@ __device__ __forceinline__ void batch_one_tile(const BatchProblemDev &P, int til
         float2 *bufs = smem + slot * 2 * G::PADN;
         const long long seg = (long long)tile * SL + slot;
         const SegmentBarrier<G::T> bar{1 + slot};
-#if OLS_FWD_TW_TMEM
         // the same TMEM layout as the plain kernel (twiddles of this N, then the
         // segment spectrum), so results stay bitwise those of per-problem calls
         // (the TMEM exchange at the segment lengths of OLS_BATCH_TX_MASK); the
@@ -168,16 +157,9 @@ __device__ __forceinline__ void batch_one_tile(const BatchProblemDev &P, int til
         using TWT = TwTmemT<xch>;
         const TWT twt{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
         if (fill) tw_tmem_fill<LOG2N, xch>(tw, twt.base, t);
-        ols_segment<LOG2N, TWT, true, SegmentBarrier<G::T>>(s_ptrs[P.index], P.Ns, P.Hk, twt, y_ptrs[P.index],
+        ols_segment<LOG2N, TWT, SegmentBarrier<G::T>>(s_ptrs[P.index], P.Ns, P.Hk, twt, y_ptrs[P.index],
                                                                P.M, P.F, P.L, P.Nout, seg, seg < P.nseg, bufs, t, xc,
-                                                               0u, bar, P.status);
-#else
-        (void)tbase;
-        (void)fill;
-        ols_segment<LOG2N, TwGlobal, false, SegmentBarrier<G::T>>(s_ptrs[P.index], P.Ns, P.Hk, TwGlobal{tw},
-                                                                  y_ptrs[P.index], P.M, P.F, P.L, P.Nout, seg,
-                                                                  seg < P.nseg, bufs, t, xc, 0u, bar, P.status);
-#endif
+                                                         bar, P.status);
     }
 }
 
@@ -190,15 +172,11 @@ ols_batched_one_kernel(const BatchProblemDev *__restrict__ probs, const int4 *__
     __shared__ long long item_sh;
     __shared__ uint32_t tbase;
     float2 *smem = reinterpret_cast<float2 *>(smem_raw);
-#if OLS_FWD_TW_TMEM
     constexpr uint32_t kCols = (uint32_t)(BB / 128) * 128u;   // a 128-column lane range per 128 threads
     if (threadIdx.x < 32) tmem::alloc(&tbase, kCols);
     tmem::fence_before_sync();
     __syncthreads();
     tmem::fence_after_sync();
-#else
-    tbase = 0;
-#endif
     int xc = 0;
     // One tile per iteration.  An item's tiles run one after another (a slot
     // takes segment `slot` of each tile without synchronising with the other
@@ -234,12 +212,10 @@ ols_batched_one_kernel(const BatchProblemDev *__restrict__ probs, const int4 *__
         ++r;
         --left;
     }
-#if OLS_FWD_TW_TMEM
     tmem::fence_before_sync();
     __syncthreads();
     tmem::fence_after_sync();
     if (threadIdx.x < 32) tmem::dealloc(tbase, kCols);
-#endif
 }
 
 // two padded exchange buffers per slot; the same for every N
@@ -252,11 +228,7 @@ static cudaError_t batched_one_prepare_b(int sm_count, int *grid_cap) {
                                          (int)batch_one_smem<BB>());
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    if (OLS_FWD_TW_TMEM)
-        e = resident_blocks_tmem(ols_batched_one_kernel<BB>, BB, batch_one_smem<BB>(), (BB / 128) * 128, &per_sm);
-    else
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ols_batched_one_kernel<BB>, BB,
-                                                          batch_one_smem<BB>());
+    e = resident_blocks_tmem(ols_batched_one_kernel<BB>, BB, batch_one_smem<BB>(), (BB / 128) * 128, &per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     *grid_cap = per_sm * sm_count;

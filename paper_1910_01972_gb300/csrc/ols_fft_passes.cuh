@@ -29,23 +29,8 @@
 #ifndef OLS_PREFETCH_H
 #define OLS_PREFETCH_H 1     // load filter f+1's spectrum while filter f is transformed
 #endif
-#ifndef OLS_H_L2ONLY
-#define OLS_H_L2ONLY 0       // 1: spectra bypass L1 (__ldcg), 2: not allocated in L1, instead of __ldg
-#endif
 #ifndef OLS_XBUFS
 #define OLS_XBUFS 2          // exchange buffers per segment (2: one barrier per exchange)
-#endif
-#ifndef OLS_TW_GLOBAL
-#define OLS_TW_GLOBAL 1      // twiddles read through L1 (1) or staged in shared memory (0)
-#endif
-#ifndef OLS_FWD_TW_TMEM
-#define OLS_FWD_TW_TMEM 1    // fused kernels keep twiddles and the segment spectrum in TMEM (0: registers and L1)
-#endif
-#ifndef OLS_TW_TMEM_LATE
-#define OLS_TW_TMEM_LATE 0   // 1: TMEM twiddles of an inverse pass are read after its exchange, not before
-#endif
-#ifndef OLS_FWD_X_TMEM
-#define OLS_FWD_X_TMEM 0     // 1: the forward kernel keeps only the segment spectrum in TMEM
 #endif
 #ifndef OLS_TMEM_XCHG
 #define OLS_TMEM_XCHG 1      // N = 512..4096: the exchange between the last two passes goes through TMEM (0: shared memory)
@@ -104,23 +89,19 @@ struct Geo {
     static constexpr int TWN = tw_off(NP - 1);
     // the exchange between the last two passes goes through TMEM (kernels
     // with TMEM twiddles; columns 64..95 of the thread's block are free)
-    static constexpr bool TX = OLS_TMEM_XCHG && OLS_FWD_TW_TMEM && LOG2N >= 9 && LOG2N <= 12 &&
+    static constexpr bool TX = OLS_TMEM_XCHG && LOG2N >= 9 && LOG2N <= 12 &&
                                ((OLS_TX_MASK >> (LOG2N - 9)) & 1);
     static constexpr bool TX_NOPF = TX && ((OLS_TX_NOPF_MASK >> (LOG2N - 9)) & 1);
     // ... with pass NP-2's lanes relabelled (N = 2048)
     static constexpr bool TX_RELABEL = TX;
-    static constexpr int TWN_PAD = OLS_TW_GLOBAL ? 0 : ((TWN + 1) & ~1);   // keep buffers 16-byte aligned
     static constexpr int XBUFS = OLS_XBUFS;
-    static constexpr size_t SMEM = sizeof(float2) * (size_t)(TWN_PAD + SEGS * XBUFS * PADN);
+    static constexpr size_t SMEM = sizeof(float2) * (size_t)(SEGS * XBUFS * PADN);
     // TMEM twiddles: 128 columns per 128 threads (a thread's lane, 32 columns per pass)
     static constexpr uint32_t TMEM_COLS = (uint32_t)(BLOCK / 128) * 128u;
     static constexpr int TMEM_MAX_CTAS = 512 / (int)TMEM_COLS;
-    // segment spectrum alone in TMEM: 32 columns per 128 threads, rounded to the 32-column minimum
-    static constexpr uint32_t XT_COLS = (BLOCK / 128) * 32u < 32u ? 32u : (uint32_t)(BLOCK / 128) * 32u;
     // shared memory requested with TMEM twiddles: enough that no more CTAs fit on
     // an SM (228 KB) than TMEM can serve, so allocation never waits
-    static constexpr size_t SMEM_TMEM = !OLS_FWD_TW_TMEM ? SMEM
-                                        : (SEGS * XBUFS * PADN * sizeof(float2) > (228u * 1024u) / (TMEM_MAX_CTAS + 1))
+    static constexpr size_t SMEM_TMEM = (SEGS * XBUFS * PADN * sizeof(float2) > (228u * 1024u) / (TMEM_MAX_CTAS + 1))
                                             ? SEGS * XBUFS * PADN * sizeof(float2)
                                             : (228u * 1024u) / (TMEM_MAX_CTAS + 1) + 1024u;
 };
@@ -565,11 +546,7 @@ struct TwGlobal {
         const float2 *w = tw + G::tw_off(P) + (t % s);
 #pragma unroll
         for (int k = 1; k <= OLS_TW_LOADS; ++k) {
-#if OLS_TW_GLOBAL
             f.w[k - 1] = __ldg(w + (k - 1) * s);
-#else
-            f.w[k - 1] = w[(k - 1) * s];
-#endif
         }
     }
     template <bool INV>
@@ -698,11 +675,11 @@ __device__ __forceinline__ void inverse_passes(float2 *x, float2 *bufs, const TW
     using G = Geo<LOG2N>;
     if constexpr (P < G::NP - 1) {
         typename TW::Fetched f;
-        // in flight during the exchange, except TMEM twiddles with OLS_TW_TMEM_LATE
-        // or before the TMEM exchange (their 30 registers then are not live
-        // across the exchange: with them the kernel spills)
+        // in flight during the exchange, except TMEM twiddles before the TMEM
+        // exchange (their registers then are not live across it: with them the
+        // kernel spills)
         constexpr bool tx = G::TX && tw_xchg<TW>();
-        constexpr bool late = (OLS_TW_TMEM_LATE || (tx && P == G::NP - 2)) && is_tw_tmem<TW>::value;
+        constexpr bool late = tx && P == G::NP - 2;
         if constexpr (!late) tw.template fetch<LOG2N, P>(f, t);
         if constexpr (tx && P == G::NP - 2) {
             tx_inverse<LOG2N>(x, tw.xbase());
@@ -723,19 +700,6 @@ __device__ __forceinline__ void inverse_passes(float2 *x, float2 *bufs, const fl
     inverse_passes<LOG2N, P>(x, bufs, TwGlobal{tw}, t, xc);
 }
 
-__device__ __forceinline__ float4 load_spectrum(const float4 *p) {
-#if OLS_H_L2ONLY == 2
-    float4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "l"(p));
-    return v;
-#elif OLS_H_L2ONLY
-    return __ldcg(p);
-#else
-    return __ldg(p);
-#endif
-}
-
+__device__ __forceinline__ float4 load_spectrum(const float4 *p) { return __ldg(p); }
 
 }  // namespace ols

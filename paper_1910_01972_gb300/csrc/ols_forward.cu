@@ -49,7 +49,6 @@ ols_forward_kernel(const float2 *__restrict__ sig, long long Ns, const float4 *_
     const int slot = threadIdx.x / G::T;
     const int t = threadIdx.x % G::T;
     float2 *bufs = smem + slot * G::XBUFS * G::PADN;
-#if OLS_FWD_TW_TMEM
     // twiddles in TMEM: warp 0 allocates, every thread fills its own lane
     if (threadIdx.x < 32) tmem::alloc(&tbase, G::TMEM_COLS);
     tmem::fence_before_sync();
@@ -57,43 +56,16 @@ ols_forward_kernel(const float2 *__restrict__ sig, long long Ns, const float4 *_
     tmem::fence_after_sync();
     const TwTmem tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
     tw_tmem_fill<LOG2N>(twg, tw.base, t);
-#else
-    const TwGlobal tw{twg};
-#if OLS_FWD_X_TMEM
-    // the segment spectrum in TMEM: 32 columns per 128 threads (a thread's lane)
-    if (threadIdx.x < 32) tmem::alloc(&tbase, G::XT_COLS);
-    tmem::fence_before_sync();
-    __syncthreads();
-    tmem::fence_after_sync();
-    const uint32_t xcol_t = tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 32u;
-#else
-    (void)tbase;
-    const uint32_t xcol_t = 0;
-#endif
-#endif
     int xc = 0;
     const long long nblk = (nseg + G::SEGS - 1) / G::SEGS;
     for (long long blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
         const long long seg = blk * G::SEGS + slot;
-#if OLS_FWD_TW_TMEM
-        ols_segment<LOG2N>(sig, Ns, Hk, tw, y, M, F, L, Nout, seg, seg < nseg, bufs, t, xc, 0u, CtaBarrier{}, status);
-#else
-        ols_segment<LOG2N, TwGlobal, OLS_FWD_X_TMEM != 0>(sig, Ns, Hk, tw, y, M, F, L, Nout, seg, seg < nseg, bufs,
-                                                          t, xc, xcol_t, CtaBarrier{}, status);
-#endif
+        ols_segment<LOG2N>(sig, Ns, Hk, tw, y, M, F, L, Nout, seg, seg < nseg, bufs, t, xc, CtaBarrier{}, status);
     }
-#if OLS_FWD_X_TMEM && !OLS_FWD_TW_TMEM
-    tmem::fence_before_sync();
-    __syncthreads();
-    tmem::fence_after_sync();
-    if (threadIdx.x < 32) tmem::dealloc(tbase, G::XT_COLS);
-#endif
-#if OLS_FWD_TW_TMEM
     tmem::fence_before_sync();
     __syncthreads();
     tmem::fence_after_sync();
     if (threadIdx.x < 32) tmem::dealloc(tbase, G::TMEM_COLS);
-#endif
 }
 
 template <int LOG2N>
@@ -103,14 +75,10 @@ static cudaError_t prepare_one(ols_plan_s &p) {
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM_TMEM);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    if (OLS_FWD_TW_TMEM || OLS_FWD_X_TMEM)
-        e = resident_blocks_tmem(ols_forward_kernel<LOG2N>, G::BLOCK, G::SMEM_TMEM,
-                                 OLS_FWD_TW_TMEM ? (int)G::TMEM_COLS : (int)G::XT_COLS, &per_sm);
-    else
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ols_forward_kernel<LOG2N>, G::BLOCK, G::SMEM_TMEM);
+    e = resident_blocks_tmem(ols_forward_kernel<LOG2N>, G::BLOCK, G::SMEM_TMEM, (int)G::TMEM_COLS, &per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    if (OLS_FWD_TW_TMEM && per_sm > G::TMEM_MAX_CTAS) per_sm = G::TMEM_MAX_CTAS;
+    if (per_sm > G::TMEM_MAX_CTAS) per_sm = G::TMEM_MAX_CTAS;
     p.fwd_grid_cap = per_sm * p.sm_count;
     return cudaSuccess;
 }

@@ -46,8 +46,7 @@ struct PostGeo {
     static constexpr size_t SMEM_USED = sizeof(float2) * (size_t)(G::SEGS * SLOT);
     // requested: at least enough that no more blocks fit on an SM (228 KB)
     // than TMEM can serve, so a block's tcgen05.alloc never waits
-    static constexpr size_t SMEM = !OLS_FWD_TW_TMEM ? SMEM_USED
-                                   : (SMEM_USED > (228u * 1024u) / (G::TMEM_MAX_CTAS + 1))
+    static constexpr size_t SMEM = (SMEM_USED > (228u * 1024u) / (G::TMEM_MAX_CTAS + 1))
                                        ? SMEM_USED
                                        : (228u * 1024u) / (G::TMEM_MAX_CTAS + 1) + 1024u;
     // the derivative's epilogue holds more live values: one resident block
@@ -120,7 +119,6 @@ ols_post_kernel(const float2 *__restrict__ sig, long long Ns, const float4 *__re
     const int t = threadIdx.x % G::T;
     float2 *bufs = smem + slot * PG::SLOT;
     float2 *dbuf = bufs + G::XBUFS * G::PADN;        // DERIV: the output's neighbourhood; PEAK: warp edges
-#if OLS_FWD_TW_TMEM
     // the forward kernel's TMEM layout: twiddles, then the segment spectrum (columns 96..127)
     if (threadIdx.x < 32) tmem::alloc(&tbase, G::TMEM_COLS);
     tmem::fence_before_sync();
@@ -134,10 +132,6 @@ ols_post_kernel(const float2 *__restrict__ sig, long long Ns, const float4 *__re
     const TwTmemT<xch> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
     tw_tmem_fill<LOG2N, xch>(twg, tw.base, t);
     const uint32_t xcol = tw.base + 96;
-#else
-    (void)tbase;
-    const TwGlobal tw{twg};
-#endif
     // circular position of a segment's first output, and its input offset
     const int n0 = PG::NEIGH ? M : M - 1;
     const long long off = PG::NEIGH ? -1 : 0;
@@ -165,10 +159,8 @@ ols_post_kernel(const float2 *__restrict__ sig, long long Ns, const float4 *__re
             }
         }
         forward_passes<LOG2N, 0>(X, bufs, tw, t, xc);
-#if OLS_FWD_TW_TMEM
         tmem::st32(xcol, reinterpret_cast<const float *>(X));
         tmem::wait_st();
-#endif
 
         const long long rem = active ? (Nout - j0) : 0;
         const int span = (int)(rem < step ? rem : step);
@@ -180,13 +172,8 @@ ols_post_kernel(const float2 *__restrict__ sig, long long Ns, const float4 *__re
             if (in_bounds(j2 * G::T + t < hn_end, status)) hn[j2] = load_spectrum(Hk + j2 * G::T + t);
         for (int f = 0; f < F; ++f) {
             float2 x[16];
-#if OLS_FWD_TW_TMEM
             tmem::ld32(xcol, reinterpret_cast<float *>(x));
             tmem::wait_ld();
-#else
-#pragma unroll
-            for (int j = 0; j < 16; ++j) x[j] = X[j];
-#endif
 #pragma unroll
             for (int j2 = 0; j2 < 8; ++j2) {
                 x[2 * j2] = cmul(x[2 * j2], make_float2(hn[j2].x, hn[j2].y));
@@ -275,12 +262,10 @@ ols_post_kernel(const float2 *__restrict__ sig, long long Ns, const float4 *__re
             }
         }
     }
-#if OLS_FWD_TW_TMEM
     tmem::fence_before_sync();
     __syncthreads();
     tmem::fence_after_sync();
     if (threadIdx.x < 32) tmem::dealloc(tbase, G::TMEM_COLS);
-#endif
 }
 
 template <int LOG2N, int MODE>
@@ -291,10 +276,7 @@ static cudaError_t post_prepare_nm(ols_plan_s &p) {
                                          (int)PG::SMEM);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    if (OLS_FWD_TW_TMEM)
-        e = resident_blocks_tmem(ols_post_kernel<LOG2N, MODE>, G::BLOCK, PG::SMEM, (int)G::TMEM_COLS, &per_sm);
-    else
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ols_post_kernel<LOG2N, MODE>, G::BLOCK, PG::SMEM);
+    e = resident_blocks_tmem(ols_post_kernel<LOG2N, MODE>, G::BLOCK, PG::SMEM, (int)G::TMEM_COLS, &per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     p.post_grid_cap[MODE] = per_sm * p.sm_count;

@@ -60,7 +60,6 @@ ols_r2r_kernel(const float *__restrict__ sig, long long Ns, const float4 *__rest
     const int slot = threadIdx.x / G::T;
     const int t = threadIdx.x % G::T;
     float2 *bufs = smem + slot * G::XBUFS * G::PADN;
-#if OLS_FWD_TW_TMEM
     // the forward kernel's TMEM layout: the thread's twiddles, then (columns
     // 96..127) the segment spectrum, in its own lane
     if (threadIdx.x < 32) tmem::alloc(&tbase, G::TMEM_COLS);
@@ -72,10 +71,6 @@ ols_r2r_kernel(const float *__restrict__ sig, long long Ns, const float4 *__rest
     const TwTmemT<xch> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
     tw_tmem_fill<LOG2N, xch>(twg, tw.base, t);
     const uint32_t xcol = tw.base + 96;
-#else
-    (void)tbase;
-    const TwGlobal tw{twg};
-#endif
     const int Fc = (F + 1) / 2;
     const int lo = M - 1;                      // aliased samples per segment
     int xc = 0;
@@ -100,10 +95,8 @@ ols_r2r_kernel(const float *__restrict__ sig, long long Ns, const float4 *__rest
                     0.f);
         }
         forward_passes<LOG2N, 0>(X, bufs, tw, t, xc);
-#if OLS_FWD_TW_TMEM
         tmem::st32(xcol, reinterpret_cast<const float *>(X));
         tmem::wait_st();
-#endif
 
         const long long rem = active ? (Nout - start) : 0;
         const int span = (int)(rem < (long long)(G::N - lo) ? rem : (long long)(G::N - lo));
@@ -116,13 +109,8 @@ ols_r2r_kernel(const float *__restrict__ sig, long long Ns, const float4 *__rest
             if (in_bounds(j2 * G::T + t < hn_end, status)) hn[j2] = load_spectrum(Hk + j2 * G::T + t);
         for (int p = 0; p < Fc; ++p) {
             float2 x[16];
-#if OLS_FWD_TW_TMEM
             tmem::ld32(xcol, reinterpret_cast<float *>(x));
             tmem::wait_ld();
-#else
-#pragma unroll
-            for (int j = 0; j < 16; ++j) x[j] = X[j];
-#endif
 #pragma unroll
             for (int j2 = 0; j2 < 8; ++j2) {
                 x[2 * j2] = cmul(x[2 * j2], make_float2(hn[j2].x, hn[j2].y));
@@ -159,12 +147,10 @@ ols_r2r_kernel(const float *__restrict__ sig, long long Ns, const float4 *__rest
             }
         }
     }
-#if OLS_FWD_TW_TMEM
     tmem::fence_before_sync();
     __syncthreads();
     tmem::fence_after_sync();
     if (threadIdx.x < 32) tmem::dealloc(tbase, G::TMEM_COLS);
-#endif
 }
 
 template <int LOG2N>
@@ -174,10 +160,7 @@ static cudaError_t r2r_prepare_n(ols_plan_s &p) {
                                          (int)G::SMEM_TMEM);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    if (OLS_FWD_TW_TMEM)
-        e = resident_blocks_tmem(ols_r2r_kernel<LOG2N>, G::BLOCK, G::SMEM_TMEM, (int)G::TMEM_COLS, &per_sm);
-    else
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ols_r2r_kernel<LOG2N>, G::BLOCK, G::SMEM_TMEM);
+    e = resident_blocks_tmem(ols_r2r_kernel<LOG2N>, G::BLOCK, G::SMEM_TMEM, (int)G::TMEM_COLS, &per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     p.r2r_grid_cap = per_sm * p.sm_count;

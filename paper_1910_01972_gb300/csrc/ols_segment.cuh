@@ -1,7 +1,6 @@
 // ols_segment.cuh -- one segment of Algorithm 2, shared by the plain and the
 // batched fused kernels: load the segment (zero past Ns), forward FFT into
-// registers (kept there for all filters; with TMEM twiddles, in the thread's
-// TMEM lane instead, columns 96..127), then for every filter: point-wise
+// registers, spectrum into the thread's TMEM lane (columns 96..127), then for every filter: point-wise
 // product with its spectrum (the next filter's spectrum already in flight),
 // inverse FFT, and store of the samples not aliased (n >= M-1) that fall
 // inside the output.
@@ -13,18 +12,15 @@
 
 namespace ols {
 
-// XT: the segment spectrum waits in the thread's TMEM lane at column xcol_t
-// (32 columns) instead of registers; implied by TMEM twiddles (columns 96..127).
 // BAR: the barrier of the segment's exchanges (the whole CTA by default, or
 // only the segment's own threads).  status: the plan's status word, for the
 // bounds checks of OLS_CHECK builds (may be null).
-template <int LOG2N, class TW, bool XT = is_tw_tmem<TW>::value, class BAR = CtaBarrier>
+template <int LOG2N, class TW, class BAR = CtaBarrier>
 __device__ __forceinline__ void ols_segment(const float2 *__restrict__ sig, long long Ns,
                                             const float4 *__restrict__ Hk, const TW &tw,
                                             float2 *__restrict__ y, int M, int F, long long L,
                                             long long Nout, long long seg, bool active, float2 *bufs,
-                                            int t, int &xc, uint32_t xcol_t = 0, const BAR &bar = BAR{},
-                                            int *status = nullptr) {
+                                            int t, int &xc, const BAR &bar, int *status) {
     using G = Geo<LOG2N>;
     const int lo = M - 1;                      // aliased samples per segment
     const long long start = seg * L;
@@ -42,14 +38,9 @@ __device__ __forceinline__ void ols_segment(const float2 *__restrict__ sig, long
                        : make_float2(0.f, 0.f);
     }
     forward_passes<LOG2N, 0>(X, bufs, tw, t, xc, bar);
-    constexpr bool x_in_tmem = XT;
-    uint32_t xcol = 0;
-    if constexpr (x_in_tmem) {
-        if constexpr (is_tw_tmem<TW>::value) xcol = tw.base + 96;
-        else xcol = xcol_t;
-        tmem::st32(xcol, reinterpret_cast<const float *>(X));
-        tmem::wait_st();
-    }
+    const uint32_t xcol = tw.base + 96;
+    tmem::st32(xcol, reinterpret_cast<const float *>(X));
+    tmem::wait_st();
 
     // Valid outputs of this segment: n in [lo, lo + span), n = k T + t.
     const long long rem = active ? (Nout - start) : 0;
@@ -70,13 +61,8 @@ __device__ __forceinline__ void ols_segment(const float2 *__restrict__ sig, long
     }
     for (int f = 0; f < F; ++f) {
         float2 x[16];
-        if constexpr (x_in_tmem) {
-            tmem::ld32(xcol, reinterpret_cast<float *>(x));
-            tmem::wait_ld();
-        } else {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) x[j] = X[j];
-        }
+        tmem::ld32(xcol, reinterpret_cast<float *>(x));
+        tmem::wait_ld();
         if constexpr (!prefetch) {
             const float4 *hp = Hk + (size_t)f * (G::N / 2) + t;
 #pragma unroll
