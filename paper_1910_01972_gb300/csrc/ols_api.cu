@@ -38,9 +38,11 @@ void spectral_order(int log2N, int32_t *nu) {
     }
 }
 
-static std::vector<float2> forward_twiddles(const PassPlan &pp) {
+// The plan's twiddle table: the forward twiddles of every pass (pp.twn
+// entries), then the folded factors of the TMEM-twiddle kernels (pp.tw8n).
+static std::vector<float2> twiddle_tables(const PassPlan &pp) {
     // pass p < np-1: entry (k-1) s + n' = W_{16 s}^{n' k}, k in [1, 16), n' in [0, s)
-    std::vector<float2> tw((size_t)pp.twn);
+    std::vector<float2> tw((size_t)(pp.twn + pp.tw8n));
     for (int p = 0; p + 1 < pp.np; ++p) {
         const int s = pp.stride[p], B = 16 * s;
         for (int k = 1; k < 16; ++k)
@@ -48,6 +50,19 @@ static std::vector<float2> forward_twiddles(const PassPlan &pp) {
                 const long long e = ((long long)n * k) % B;
                 const double a = -2.0 * M_PI * (double)e / (double)B;
                 tw[(size_t)pp.tw_off[p] + (size_t)(k - 1) * s + n] =
+                    make_float2((float)std::cos(a), (float)std::sin(a));
+            }
+    }
+    // folded factors (inverse sign): w^8; w^4; w^2, w^2 e(2); w, w e(1), w e(2),
+    // w e(3) with w = exp(2 pi i n' / (16 s)), e(m) = exp(2 pi i m / 16); row i
+    // of pass p at tw8_off[p] + i s + n'
+    static const int kPow[8] = {8, 4, 2, 2, 1, 1, 1, 1}, kRot[8] = {0, 0, 0, 2, 0, 1, 2, 3};
+    for (int p = 0; p + 1 < pp.np; ++p) {
+        const int s = pp.stride[p], B = 16 * s;
+        for (int i = 0; i < 8; ++i)
+            for (int n = 0; n < s; ++n) {
+                const double a = 2.0 * M_PI * (double)(kPow[i] * n + kRot[i] * s) / (double)B;
+                tw[(size_t)pp.twn + (size_t)pp.tw8_off[p] + (size_t)i * s + n] =
                     make_float2((float)std::cos(a), (float)std::sin(a));
             }
     }
@@ -256,7 +271,7 @@ int ols_plan(ols_plan_t *out, int64_t N, int32_t M, int32_t F, uint32_t flags) {
     if (e == cudaSuccess && !r2r) e = dev_alloc(&p->Htk, sizeof(float2) * (size_t)F * (size_t)N);
     if (e == cudaSuccess && r2r) e = dev_alloc(&p->hpack, sizeof(float2) * (size_t)Fc * (size_t)M);
     if (e == cudaSuccess && r2r) e = r2r_prepare(*p);
-    if (e == cudaSuccess) e = dev_alloc(&p->tw, sizeof(float2) * (size_t)(p->pp.twn > 0 ? p->pp.twn : 1));
+    if (e == cudaSuccess) e = dev_alloc(&p->tw, sizeof(float2) * (size_t)(p->pp.twn + p->pp.tw8n));
     if (e == cudaSuccess) e = dev_alloc(&p->tw64, sizeof(double2) * (size_t)N);
     if (e == cudaSuccess) e = dev_alloc(&p->nu, sizeof(int32_t) * (size_t)N);
     if (e == cudaSuccess) e = dev_alloc(&p->d_status, sizeof(int));
@@ -278,10 +293,11 @@ int ols_plan(ols_plan_t *out, int64_t N, int32_t M, int32_t F, uint32_t flags) {
         if (e == cudaSuccess) e = tc_prepare(*p, flags == OLS_FLAG_TC_BF16SPLIT);
     }
     if (e == cudaSuccess) {
-        std::vector<float2> tw = forward_twiddles(p->pp);
+        std::vector<float2> tw = twiddle_tables(p->pp);
+        p->tw8 = p->tw + p->pp.twn;
         std::vector<int32_t> nu((size_t)N);
         spectral_order(l, nu.data());
-        if (!tw.empty()) e = cudaMemcpy(p->tw, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice);
+        e = cudaMemcpy(p->tw, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(p->nu, nu.data(), sizeof(int32_t) * nu.size(), cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess) e = launch_tw64(p->tw64, (int)N, 0);

@@ -432,7 +432,7 @@ template <int LOG2N, bool DS, bool DH>
 static void launch_bwd_one(const ols_plan_s &p, const BackwardArgs &a, cudaStream_t st) {
     using BG = BwdGeo<LOG2N>;
     ols_backward_kernel<LOG2N, DS, DH><<<a.grid, BG::BLOCK, BG::SMEM, st>>>(
-        a.s, a.Ns, a.g, a.Nout, reinterpret_cast<const float4 *>(p.Htk), p.tw, a.ds, a.edge, a.P, p.M, p.F, a.L,
+        a.s, a.Ns, a.g, a.Nout, reinterpret_cast<const float4 *>(p.Htk), p.tw8, a.ds, a.edge, a.P, p.M, p.F, a.L,
         a.nseg, p.d_status);
 }
 

@@ -87,6 +87,12 @@ struct Geo {
         return o;
     }
     static constexpr int TWN = tw_off(NP - 1);
+    // folded-twiddle table (TMEM twiddles): 8 rows of stride(p) entries per pass
+    __host__ __device__ static constexpr int tw8_off(int p) {
+        int o = 0;
+        for (int i = 0; i < p; ++i) o += 8 * stride(i);
+        return o;
+    }
     // the exchange between the last two passes goes through TMEM (kernels
     // with TMEM twiddles; columns 64..95 of the thread's block are free)
     static constexpr bool TX = OLS_TMEM_XCHG && LOG2N >= 9 && LOG2N <= 12 &&
@@ -572,8 +578,10 @@ struct TwGlobal {
     }
 };
 
-// TwTmemT: the thread's own 15 twiddles of every pass, preloaded into its
-// TMEM lane (pass P at columns 32 P .. 32 P + 29 of `base`): no L1 traffic.
+// TwTmemT: the thread's own twiddles of every pass, preloaded into its TMEM
+// lane as the eight folded factors of stage_inv / stage_fwd (pass P at columns
+// 32 P .. 32 P + 31 of `base`, four columns each): no L1 traffic.  The last
+// stage's sixteen words are loaded while the other stages run.
 // XCH: the segment FFT also uses the TMEM exchange where Geo<>::TX allows it
 // (kernels whose epilogue needs the registers opt out).
 template <bool XCH = true>
@@ -583,17 +591,36 @@ struct TwTmemT {
     // columns 64..95: the staging area of the TMEM exchange
     __device__ __forceinline__ uint32_t xbase() const { return base + 64; }
     struct Fetched {
-        float v[32];
+        float v[16];
     };
     template <int LOG2N, int P>
     __device__ __forceinline__ void fetch(Fetched &f, int) const {
-        tmem::ld32(base + 32 * P, f.v);
+        tmem::ld16(base + 32 * P, f.v);
     }
-    template <bool INV>
-    __device__ __forceinline__ void apply(float2 *x, const Fetched &f) const {
-        tmem::wait_ld();
-#pragma unroll
-        for (int k = 1; k < 16; ++k) x[k] = ctw<INV>(x[k], make_float2(f.v[2 * k - 2], f.v[2 * k - 1]));
+    // inverse: twiddle and DFT-16 (f: fetched by fetch)
+    template <int LOG2N, int P>
+    __device__ __forceinline__ void dft_inv(float2 *x, Fetched &f) const {
+        float w1[16];
+        tmem::wait_ld16(f.v);
+        tmem::ld16(base + 32 * P + 16, w1);
+        stage_inv<8, LOG2N == 8>(x, f.v);
+        stage_inv<4, LOG2N == 8>(x, f.v + 4);
+        stage_inv<2, LOG2N == 8>(x, f.v + 8);
+        tmem::wait_ld16(w1);
+        stage_inv<1, LOG2N == 8>(x, w1);
+    }
+    // forward: DFT-16 and twiddle
+    template <int LOG2N, int P>
+    __device__ __forceinline__ void dft_fwd(float2 *x) const {
+        float w1[16], w8[16];
+        tmem::ld16(base + 32 * P + 16, w1);
+        tmem::wait_ld16(w1);
+        tmem::ld16(base + 32 * P, w8);
+        stage_fwd<1>(x, w1);
+        tmem::wait_ld16(w8);
+        stage_fwd<2>(x, w8 + 8);
+        stage_fwd<4>(x, w8 + 4);
+        stage_fwd<8>(x, w8);
     }
 };
 
@@ -608,23 +635,24 @@ __device__ __forceinline__ constexpr bool tw_xchg() {
     else return false;
 }
 
-// Fill a TwTmemT<XCH> for thread t from the plan's twiddle table.
+// Fill a TwTmemT<XCH> for thread t from the plan's folded-twiddle table (pass
+// P at offset tw8_off(P): eight rows of stride(P) entries, row i at n' holding
+// factor i of w = exp(2 pi i n' / (16 stride))).
 template <int LOG2N, bool XCH = true, int P = 0>
-__device__ __forceinline__ void tw_tmem_fill(const float2 *tw, uint32_t base, int t) {
+__device__ __forceinline__ void tw_tmem_fill(const float2 *tw8, uint32_t base, int t) {
     using G = Geo<LOG2N>;
     if constexpr (P < G::NP - 1) {
         constexpr int s = G::stride(P);
-        const float2 *w = tw + G::tw_off(P) + tw_index<LOG2N, P, XCH>(t);
+        const float2 *w = tw8 + G::tw8_off(P) + tw_index<LOG2N, P, XCH>(t);
         float v[32];
 #pragma unroll
-        for (int k = 1; k < 16; ++k) {
-            const float2 wk = __ldg(w + (k - 1) * s);
-            v[2 * k - 2] = wk.x;
-            v[2 * k - 1] = wk.y;
+        for (int i = 0; i < 8; ++i) {
+            const float2 wi = __ldg(w + i * s);
+            v[4 * i] = v[4 * i + 1] = wi.x;
+            v[4 * i + 2] = v[4 * i + 3] = -wi.y;
         }
-        v[30] = v[31] = 0.f;
         tmem::st32(base + 32 * P, v);
-        tw_tmem_fill<LOG2N, XCH, P + 1>(tw, base, t);
+        tw_tmem_fill<LOG2N, XCH, P + 1>(tw8, base, t);
     } else {
         tmem::wait_st();
     }
@@ -644,10 +672,14 @@ __device__ __forceinline__ void forward_passes(float2 *x, float2 *bufs, const TW
                                                const BAR &bar = BAR{}) {
     using G = Geo<LOG2N>;
     if constexpr (P < G::NP - 1) {
-        typename TW::Fetched f;
-        tw.template fetch<LOG2N, P>(f, t);            // in flight during the DFT
-        dft_groups<G::radix(P), false>(x);
-        tw.template apply<false>(x, f);
+        if constexpr (is_tw_tmem<TW>::value) {
+            tw.template dft_fwd<LOG2N, P>(x);
+        } else {
+            typename TW::Fetched f;
+            tw.template fetch<LOG2N, P>(f, t);        // in flight during the DFT
+            dft_groups<G::radix(P), false>(x);
+            tw.template apply<false>(x, f);
+        }
         constexpr bool tx = G::TX && tw_xchg<TW>();
         if constexpr (tx && P == G::NP - 2) {
             tx_forward<LOG2N>(x, tw.xbase());
@@ -690,9 +722,15 @@ __device__ __forceinline__ void inverse_passes(float2 *x, float2 *bufs, const TW
             ++xc;
         }
         if constexpr (late) tw.template fetch<LOG2N, P>(f, t);
-        tw.template apply<true>(x, f);
+        if constexpr (is_tw_tmem<TW>::value) {
+            tw.template dft_inv<LOG2N, P>(x, f);
+        } else {
+            tw.template apply<true>(x, f);
+            dft_groups<G::radix(P), true>(x);
+        }
+    } else {
+        dft_groups<G::radix(P), true>(x);
     }
-    dft_groups<G::radix(P), true>(x);
     if constexpr (P > 0) inverse_passes<LOG2N, P - 1>(x, bufs, tw, t, xc, bar);
 }
 template <int LOG2N, int P>

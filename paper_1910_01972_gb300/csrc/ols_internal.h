@@ -26,6 +26,8 @@ struct PassPlan {
     int stride[4];
     int tw_off[4];
     int twn;     // twiddle entries of passes 0 .. np-2
+    int tw8_off[4];
+    int tw8n;    // folded-twiddle entries (8 per stride position) of those passes
 };
 PassPlan make_pass_plan(int log2N);
 
@@ -122,10 +124,10 @@ struct ols_plan_s {
     ols::PassPlan pp{};
     float2 *Hk = nullptr;        // [F][N] spectra in kernel layout (FP32)
     float2 *Htk = nullptr;       // [F][N] spectra of conj(h_f[M-1-k]) (adjoint), kernel layout
-    float2 *tw = nullptr;        // forward twiddles (FP32), pp.twn entries
+    float2 *tw = nullptr;        // forward twiddles (FP32), pp.twn entries, then the folded ones
+    const float2 *tw8 = nullptr; // folded twiddles of the TMEM-twiddle kernels: tw + pp.twn (pp.tw8n entries)
     double2 *tw64 = nullptr;     // W_N^m, m in [0, N) (FP64)
     int32_t *nu = nullptr;       // spectral order (device copy)
-    int fwd_grid_cap = 0;        // resident blocks of the forward kernel
     int bwd_grid_cap[3] = {0, 0, 0};  // backward kernel: (ds,dh), (ds), (dh)
     int last_launches = 0;
     int tc_grid_cap = 0;         // resident blocks of the tensor-core kernel
@@ -135,7 +137,6 @@ struct ols_plan_s {
     int post_grid_cap[4] = {0, 0, 0, 0};  // post-processing kernels (power, detect, derivative, peaks)
     // real-to-real plans (OLS_FLAG_R2R)
     float2 *hpack = nullptr;     // [ceil(F/2)][M] paired real filters h_{2p} + i h_{2p+1}
-    int r2r_grid_cap = 0;
     uint16_t *tc_bmat = nullptr; // split DFT-16 matrices (fwd hi, fwd lo, inv hi, inv lo), core-matrix layout
     int *d_status = nullptr;     // device status word (bounded-wait failures)
     ols::Staging stage;
@@ -164,7 +165,7 @@ struct BatchProblemDev {
     int *status;          // the problem's plan status word (bounds checks of OLS_CHECK builds)
 };
 
-// Twiddle tables of every segment length, by log2 N (single-launch batches).
+// Folded-twiddle tables of every segment length, by log2 N (single-launch batches).
 struct TwTables {
     const float2 *tw[kMaxLog2N + 1];
 };

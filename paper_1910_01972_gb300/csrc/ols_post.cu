@@ -312,7 +312,7 @@ static cudaError_t post_launch_nm(const ols_plan_s &p, const PostArgs &a, cudaSt
     const int cap = p.post_grid_cap[MODE];
     const int grid = fused_grid(LOG2N, nblk, cap);
     ols_post_kernel<LOG2N, MODE><<<grid, G::BLOCK, PG::SMEM, st>>>(
-        a.s, a.Ns, reinterpret_cast<const float4 *>(p.Hk), p.tw, a.out, p.M, p.F, a.step, a.nseg, a.Nout, a.thr,
+        a.s, a.Ns, reinterpret_cast<const float4 *>(p.Hk), p.tw8, a.out, p.M, p.F, a.step, a.nseg, a.Nout, a.thr,
         a.cand, a.count, a.cap, p.d_status);
     return cudaGetLastError();
 }

@@ -21,9 +21,8 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 
-#include "ols_fft_passes.cuh"
+#include "ols_bank.cuh"
 #include "ols_internal.h"
-#include "tmem.cuh"
 
 namespace ols {
 
@@ -46,161 +45,58 @@ cudaError_t launch_pack_real_pairs(const float *h, int M, int F, float2 *g, cuda
     return cudaGetLastError();
 }
 
-// One persistent kernel: resident blocks loop over segments (SEGS segments
-// of N/16 threads per block for small N, advancing in lock step).
-template <int LOG2N>
-__global__ void __launch_bounds__(Geo<LOG2N>::BLOCK, Geo<LOG2N>::MINB)
-ols_r2r_kernel(const float *__restrict__ sig, long long Ns, const float4 *__restrict__ Hk,
-               const float2 *__restrict__ twg, float *__restrict__ y, int M, int F, long long L, long long nseg,
-               long long Nout, int *status) {
-    using G = Geo<LOG2N>;
-    extern __shared__ float4 smem_raw[];
-    __shared__ uint32_t tbase;
-    float2 *smem = reinterpret_cast<float2 *>(smem_raw);
-    const int slot = threadIdx.x / G::T;
-    const int t = threadIdx.x % G::T;
-    float2 *bufs = smem + slot * G::XBUFS * G::PADN;
-    // the forward kernel's TMEM layout: the thread's twiddles, then (columns
-    // 96..127) the segment spectrum, in its own lane
-    if (threadIdx.x < 32) tmem::alloc(&tbase, G::TMEM_COLS);
-    tmem::fence_before_sync();
-    __syncthreads();
-    tmem::fence_after_sync();
-    // the TMEM exchange at N = 2048 only (at other N this kernel spills with it)
-    constexpr bool xch = LOG2N == 11;
-    const TwTmemT<xch> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
-    tw_tmem_fill<LOG2N, xch>(twg, tw.base, t);
-    const uint32_t xcol = tw.base + 96;
-    const int Fc = (F + 1) / 2;
-    const int lo = M - 1;                      // aliased samples per segment
-    int xc = 0;
-    const long long nblk = (nseg + G::SEGS - 1) / G::SEGS;
-    for (long long blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
-        const long long seg = blk * G::SEGS + slot;
-        const bool active = seg < nseg;
-        const long long start = seg * L;
-
-        // Segment load: real samples start + k T + t (zero past Ns) as complex values.
-        float2 X[16];
-        {
-            const long long avail = active ? (Ns - start) : 0;
-            const int lim = (int)(avail < G::N ? avail : G::N);
-            const float *src = sig + (active ? start : 0) + t;
+// Real samples in, one inverse FFT per filter pair, its real and imaginary
+// parts stored as the pair's two output rows.
+struct EpiReal {
+    static constexpr bool XCH = true;
+    template <int LOG2N>
+    static constexpr int edge() { return 0; }
+    const float *sig;
+    float *y;
+    int F;                  // real filters (F spectra of the bank kernel: pairs)
+    __device__ __forceinline__ float2 sample(long long i) const { return make_float2(__ldg(sig + i), 0.f); }
+    template <int LOG2N, class BAR>
+    __device__ __forceinline__ void store(const float2 *x, int p, int t, const BankSegment &sg, float2 *, int &,
+                                          const BAR &) const {
+        using G = Geo<LOG2N>;
+        const int v = t - sg.n0;
+        float *dre = y + (size_t)(2 * p) * (size_t)sg.Nout + (sg.j0 + v);
+        // the pair test is uniform: taken once per filter pair, so each store
+        // below is a plain predicated store
+        if (2 * p + 1 < F) {
+            float *dim = dre + sg.Nout;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                const bool ok = (unsigned)(v + k * G::T) < (unsigned)sg.span &&
+                                in_bounds(sg.j0 + v + k * G::T < sg.Nout, sg.status);
+                if (ok) __stcs(dre + k * G::T, x[k].x);
+                if (ok) __stcs(dim + k * G::T, x[k].y);
+            }
+        } else {
 #pragma unroll
             for (int k = 0; k < 16; ++k)
-                X[k] = make_float2(
-                    (k * G::T + t < lim && in_bounds((active ? start : 0) + k * G::T + t < Ns, status))
-                        ? __ldg(src + k * G::T)
-                        : 0.f,
-                    0.f);
-        }
-        forward_passes<LOG2N, 0>(X, bufs, tw, t, xc);
-        tmem::st32(xcol, reinterpret_cast<const float *>(X));
-        tmem::wait_st();
-
-        const long long rem = active ? (Nout - start) : 0;
-        const int span = (int)(rem < (long long)(G::N - lo) ? rem : (long long)(G::N - lo));
-        const long long obase = start - lo;
-
-        float4 hn[8];
-        const long long hn_end = (long long)Fc * (G::N / 2);   // float4 entries of the paired spectra
-#pragma unroll
-        for (int j2 = 0; j2 < 8; ++j2)
-            if (in_bounds(j2 * G::T + t < hn_end, status)) hn[j2] = load_spectrum(Hk + j2 * G::T + t);
-        for (int p = 0; p < Fc; ++p) {
-            float2 x[16];
-            tmem::ld32(xcol, reinterpret_cast<float *>(x));
-            tmem::wait_ld();
-#pragma unroll
-            for (int j2 = 0; j2 < 8; ++j2) {
-                x[2 * j2] = cmul(x[2 * j2], make_float2(hn[j2].x, hn[j2].y));
-                x[2 * j2 + 1] = cmul(x[2 * j2 + 1], make_float2(hn[j2].z, hn[j2].w));
-            }
-            if (p + 1 < Fc) {
-                const float4 *hp = Hk + (size_t)(p + 1) * (G::N / 2) + t;
-#pragma unroll
-                for (int j2 = 0; j2 < 8; ++j2)
-                    if (in_bounds((long long)(p + 1) * (G::N / 2) + j2 * G::T + t < hn_end, status))
-                        hn[j2] = load_spectrum(hp + j2 * G::T);
-            }
-            inverse_passes<LOG2N, G::NP - 1>(x, bufs, tw, t, xc);
-            float *dre = y + (size_t)(2 * p) * (size_t)Nout + obase;
-            float *dim = dre + Nout;
-            // the pair test is uniform: taken once per filter pair, so each
-            // store below is a plain predicated store
-            if (2 * p + 1 < F) {
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const int n = k * G::T + t;
-                    const bool ok = (unsigned)(n - lo) < (unsigned)span &&
-                                    in_bounds(obase + n >= 0 && obase + n < Nout, status);
-                    if (ok) dre[n] = x[k].x;
-                    if (ok) dim[n] = x[k].y;
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const int n = k * G::T + t;
-                    if ((unsigned)(n - lo) < (unsigned)span && in_bounds(obase + n >= 0 && obase + n < Nout, status))
-                        dre[n] = x[k].x;
-                }
-            }
+                if ((unsigned)(v + k * G::T) < (unsigned)sg.span && in_bounds(sg.j0 + v + k * G::T < sg.Nout, sg.status))
+                    __stcs(dre + k * G::T, x[k].x);
         }
     }
-    tmem::fence_before_sync();
-    __syncthreads();
-    tmem::fence_after_sync();
-    if (threadIdx.x < 32) tmem::dealloc(tbase, G::TMEM_COLS);
-}
+};
 
-template <int LOG2N>
-static cudaError_t r2r_prepare_n(ols_plan_s &p) {
-    using G = Geo<LOG2N>;
-    cudaError_t e = cudaFuncSetAttribute(ols_r2r_kernel<LOG2N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)G::SMEM_TMEM);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = resident_blocks_tmem(ols_r2r_kernel<LOG2N>, G::BLOCK, G::SMEM_TMEM, (int)G::TMEM_COLS, &per_sm);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    p.r2r_grid_cap = per_sm * p.sm_count;
-    return cudaSuccess;
-}
-
-template <int LOG2N>
-static cudaError_t r2r_launch_n(const ols_plan_s &p, const float *s, int64_t Ns, float *y, int64_t L, int64_t nseg,
-                                int64_t Nout, cudaStream_t st) {
-    using G = Geo<LOG2N>;
-    const int64_t nblk = (nseg + G::SEGS - 1) / G::SEGS;
-    const int grid = fused_grid(LOG2N, nblk, p.r2r_grid_cap);
-    ols_r2r_kernel<LOG2N><<<grid, G::BLOCK, G::SMEM_TMEM, st>>>(s, Ns, reinterpret_cast<const float4 *>(p.Hk), p.tw, y,
-                                                           p.M, p.F, L, nseg, Nout, p.d_status);
-    return cudaGetLastError();
-}
-
-cudaError_t r2r_prepare(ols_plan_s &p) {
-    switch (p.log2N) {
-        case 8: return r2r_prepare_n<8>(p);
-        case 9: return r2r_prepare_n<9>(p);
-        case 10: return r2r_prepare_n<10>(p);
-        case 11: return r2r_prepare_n<11>(p);
-        case 12: return r2r_prepare_n<12>(p);
-        case 13: return r2r_prepare_n<13>(p);
-        default: return cudaErrorInvalidValue;
-    }
-}
+cudaError_t r2r_prepare(ols_plan_s &p) { return bank_prepare_any<EpiReal>(p.log2N); }
 
 cudaError_t r2r_launch(const ols_plan_s &p, const float *s, int64_t Ns, float *y, int64_t L, int64_t nseg,
                        int64_t Nout, cudaStream_t st) {
-    switch (p.log2N) {
-        case 8: return r2r_launch_n<8>(p, s, Ns, y, L, nseg, Nout, st);
-        case 9: return r2r_launch_n<9>(p, s, Ns, y, L, nseg, Nout, st);
-        case 10: return r2r_launch_n<10>(p, s, Ns, y, L, nseg, Nout, st);
-        case 11: return r2r_launch_n<11>(p, s, Ns, y, L, nseg, Nout, st);
-        case 12: return r2r_launch_n<12>(p, s, Ns, y, L, nseg, Nout, st);
-        case 13: return r2r_launch_n<13>(p, s, Ns, y, L, nseg, Nout, st);
-        default: return cudaErrorInvalidValue;
-    }
+    BankArgs a{};
+    a.Hk = reinterpret_cast<const float4 *>(p.Hk);
+    a.tw8 = p.tw8;
+    a.F = (p.F + 1) / 2;
+    a.n0 = p.M - 1;
+    a.step = L;
+    a.off = 0;
+    a.Ns = Ns;
+    a.Nout = Nout;
+    a.nseg = nseg;
+    a.status = p.d_status;
+    return bank_launch_any(p.log2N, a, EpiReal{s, y, p.F}, p.sm_count, st);
 }
 
 }  // namespace ols

@@ -71,6 +71,17 @@ __device__ __forceinline__ void ld16(uint32_t taddr, float *v) {
                  : "memory");
 }
 
+// wait::ld that also names the registers being waited for, so that no use of
+// them can be scheduled before it.
+__device__ __forceinline__ void wait_ld16(float *v) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
+                   "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]),
+                   "+f"(v[15])
+                 :
+                 : "memory");
+}
+
 // The 16-lane shapes (lane field of taddr: quarter base, or base + 16).
 // 16x256b: thread T's register i = 4 r + 2 j + e sits at lane 8 j + T / 4,
 // column 8 r + 2 (T mod 4) + e; four repetitions (.x4) span 32 columns.
