@@ -271,7 +271,7 @@ int ols_plan(ols_plan_t *out, int64_t N, int32_t M, int32_t F, uint32_t flags) {
     if (e == cudaSuccess && !r2r) e = dev_alloc(&p->Htk, sizeof(float2) * (size_t)F * (size_t)N);
     if (e == cudaSuccess && r2r) e = dev_alloc(&p->hpack, sizeof(float2) * (size_t)Fc * (size_t)M);
     if (e == cudaSuccess && r2r) e = r2r_prepare(*p);
-    if (e == cudaSuccess) e = dev_alloc(&p->tw, sizeof(float2) * (size_t)(p->pp.twn + p->pp.tw8n));
+    if (e == cudaSuccess) e = dev_alloc(&p->tw, sizeof(float2) * (size_t)(p->pp.twn + p->pp.tw8n + N / 2));
     if (e == cudaSuccess) e = dev_alloc(&p->tw64, sizeof(double2) * (size_t)N);
     if (e == cudaSuccess) e = dev_alloc(&p->nu, sizeof(int32_t) * (size_t)N);
     if (e == cudaSuccess) e = dev_alloc(&p->d_status, sizeof(int));
@@ -295,8 +295,12 @@ int ols_plan(ols_plan_t *out, int64_t N, int32_t M, int32_t F, uint32_t flags) {
     if (e == cudaSuccess) {
         std::vector<float2> tw = twiddle_tables(p->pp);
         p->tw8 = p->tw + p->pp.twn;
+        p->dsin = reinterpret_cast<const float *>(p->tw8 + p->pp.tw8n);
         std::vector<int32_t> nu((size_t)N);
         spectral_order(l, nu.data());
+        for (int64_t q = 0; q < N; q += 2)
+            tw.push_back(make_float2((float)std::sin(2.0 * M_PI * (double)nu[q] / (double)N),
+                                     (float)std::sin(2.0 * M_PI * (double)nu[q + 1] / (double)N)));
         e = cudaMemcpy(p->tw, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(p->nu, nu.data(), sizeof(int32_t) * nu.size(), cudaMemcpyHostToDevice);
     }

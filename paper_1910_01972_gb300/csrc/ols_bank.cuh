@@ -137,6 +137,7 @@ ols_bank_kernel(const BankArgs a, const EPI epi) {
                            : make_float2(0.f, 0.f);
             }
             forward_passes<LOG2N, 0>(X, bufs, tw, t, xc, bar);
+            epi.template spectrum<LOG2N>(X, t, sg);
             tmem::st32(xcol, reinterpret_cast<const float *>(X));
             tmem::wait_st();
         }

@@ -186,11 +186,23 @@ __device__ __forceinline__ void exchange(float2 *x, float2 *buf, int t, const BA
 // p2, p7), warp = p9, p10; pass 2 (radix 8 over p0..p2): thread = p4..p10,
 // register = p0..p3 (the layout of the spectrum).  Shared exchange of passes
 // 0 and 1: position q at q ^ (p8 << 3) (no padding).
+#ifndef TX11S
+#define TX11S 0
+#endif
+#if TX11S
+__device__ __forceinline__ int tx11_addr0(int t, int k) {
+    return t + 130 * (k & 1) + 264 * ((k >> 1) & 1) + 528 * (k >> 2);
+}
+__device__ __forceinline__ int tx11_addr1(int t, int k) {
+    return ((t >> 3) & 3) + 4 * (t & 1) + 130 * ((t >> 1) & 1) + 264 * ((t >> 2) & 1) + 528 * (t >> 5) + 8 * k;
+}
+#else
 __device__ __forceinline__ int tx11_addr0(int t, int k) { return ((k & 2) ? (t ^ 8) : t) + 128 * k; }
 __device__ __forceinline__ int tx11_addr1(int t, int k) {
     const int base = ((t >> 1) & 7) + 128 * ((t >> 4) & 1) + 256 * (t & 1) + 512 * (t >> 5);
     return base + 8 * ((k & 1) ^ (t & 1)) + 16 * (k >> 1);
 }
+#endif
 
 // N = 4096 (Geo<12>::TX): pass 0 thread = p0..p7, register = p8..p11; pass 1
 // (radix 16 over p4..p7) lanes (p0, p1, p8, p2, p3), warp p9..p11; pass 2
@@ -244,6 +256,62 @@ __device__ __forceinline__ void tx_sync() { __syncwarp(); }
 //  2. a 32x32b store (column = (re/im, p4, p5, p2, p3)); 16x256b loads:
 //     thread lanes (p4..p8), x[p0 + 2 p1 + 4 p2 + 8 p3] from
 //     w[p1][4 (p2 + 2 p3) + 2 p0 + re/im].
+#if TX11S
+// v[2 (p4 + 2 p5 + 4 p2 + 8 p3) + re/im] with lane bit 0 = p6  <->  x[p3 + 2 p4 + 4 p5 + 8 p6] with lane bit 0 = p2
+__device__ __forceinline__ void tx11_forward(float2 *x, uint32_t xb) {
+    const bool odd = threadIdx.x & 1;
+    float v[32];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {      // i = p3 + 2 p4 + 4 p5
+        const int o = 2 * ((i >> 1) + 8 * (i & 1));
+        const float2 c = x[i], d = x[i + 8];
+        const float rx = __shfl_xor_sync(0xffffffffu, odd ? c.x : d.x, 1);
+        const float ry = __shfl_xor_sync(0xffffffffu, odd ? c.y : d.y, 1);
+        v[o] = odd ? rx : c.x;
+        v[o + 1] = odd ? ry : c.y;
+        v[o + 8] = odd ? d.x : rx;
+        v[o + 9] = odd ? d.y : ry;
+    }
+    tmem::st32(xb, v);
+    tmem::wait_st();
+    tx_sync();
+    float w[2][16];
+    tmem::ld16x256b_x4(xb, w[0]);
+    tmem::ld16x256b_x4(xb + (16u << 16), w[1]);
+    tmem::wait_ld();
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {   // k = p0 + 2 p1 + 4 p2 + 8 p3
+        const int p0 = k & 1, p1 = (k >> 1) & 1, p23 = k >> 2;
+        x[k] = make_float2(w[p1][4 * p23 + 2 * p0], w[p1][4 * p23 + 2 * p0 + 1]);
+    }
+}
+__device__ __forceinline__ void tx11_inverse(float2 *x, uint32_t xb) {
+    const bool odd = threadIdx.x & 1;
+    float w[2][16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const int p0 = k & 1, p1 = (k >> 1) & 1, p23 = k >> 2;
+        w[p1][4 * p23 + 2 * p0] = x[k].x;
+        w[p1][4 * p23 + 2 * p0 + 1] = x[k].y;
+    }
+    tmem::st16x256b_x4(xb, w[0]);
+    tmem::st16x256b_x4(xb + (16u << 16), w[1]);
+    tmem::wait_st();
+    tx_sync();
+    float v[32];
+    tmem::ld32(xb, v);
+    tmem::wait_ld();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {      // i = p3 + 2 p4 + 4 p5
+        const int o = 2 * ((i >> 1) + 8 * (i & 1));
+        const float2 a = make_float2(v[o], v[o + 1]), b = make_float2(v[o + 8], v[o + 9]);
+        const float rx = __shfl_xor_sync(0xffffffffu, odd ? a.x : b.x, 1);
+        const float ry = __shfl_xor_sync(0xffffffffu, odd ? a.y : b.y, 1);
+        x[i] = make_float2(odd ? rx : a.x, odd ? ry : a.y);
+        x[i + 8] = make_float2(odd ? b.x : rx, odd ? b.y : ry);
+    }
+}
+#else
 __device__ __forceinline__ void tx11_forward(float2 *x, uint32_t xb) {
 #pragma unroll
     for (int k = 0; k < 8; ++k)      // k = p3 + 2 p4 + 4 p5; registers (x[k], x[k + 8]) differ in p6
@@ -306,6 +374,7 @@ __device__ __forceinline__ void tx11_inverse(float2 *x, uint32_t xb) {
                                x[k].y, x[k + 8].x, x[k + 8].y);
     tmem::wait_ld();
 }
+#endif
 
 // N = 4096, pass 1 -> pass 2 (registers p4 + 2 p5 + 4 p6 + 8 p7), two round
 // trips:
@@ -514,7 +583,7 @@ template <int LOG2N, int P, bool XCH>
 __device__ __forceinline__ int tw_index(int t) {
     using G = Geo<LOG2N>;
     if constexpr (XCH && G::TX_RELABEL && P == G::NP - 2) {   // the relabelled lanes holding p0 .. p(s-1)
-        if constexpr (LOG2N == 11) return (t >> 1) & 7;
+        if constexpr (LOG2N == 11) return TX11S ? ((t >> 3) & 3) + 4 * (t & 1) : (t >> 1) & 7;
         else if constexpr (LOG2N == 12) return (t & 3) + 4 * ((t >> 3) & 1) + 8 * ((t >> 4) & 1);
         else if constexpr (LOG2N == 10) return (t >> 3) & 3;
         else return (t >> 1) & 1;

@@ -16,6 +16,8 @@ struct EpiPlain {
     const float2 *sig;
     float2 *y;
     __device__ __forceinline__ float2 sample(long long i) const { return __ldg(sig + i); }
+    template <int LOG2N>
+    __device__ __forceinline__ void spectrum(float2 *, int, const BankSegment &) const {}
     template <int LOG2N, class BAR>
     __device__ __forceinline__ void store(const float2 *x, int f, int t, const BankSegment &sg, float2 *, int &,
                                           const BAR &) const {

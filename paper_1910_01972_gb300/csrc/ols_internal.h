@@ -125,6 +125,7 @@ struct ols_plan_s {
     float2 *Hk = nullptr;        // [F][N] spectra in kernel layout (FP32)
     float2 *Htk = nullptr;       // [F][N] spectra of conj(h_f[M-1-k]) (adjoint), kernel layout
     float2 *tw = nullptr;        // forward twiddles (FP32), pp.twn entries, then the folded ones
+    const float *dsin = nullptr; // sin(2 pi nu / N) at each storage position (derivative): after tw8
     const float2 *tw8 = nullptr; // folded twiddles of the TMEM-twiddle kernels: tw + pp.twn (pp.tw8n entries)
     double2 *tw64 = nullptr;     // W_N^m, m in [0, N) (FP64)
     int32_t *nu = nullptr;       // spectral order (device copy)
@@ -134,7 +135,6 @@ struct ols_plan_s {
     int tc_split_grid_cap = 0;   // the same for its pre-split-input form
     long long tc_wait_limit = 0; // polls per in-loop mbarrier wait of the tensor-core kernel
     bool tc_wait_never = false;  // test switch: in-loop waits watch an mbarrier nothing arrives on
-    int post_grid_cap[4] = {0, 0, 0, 0};  // post-processing kernels (power, detect, derivative, peaks)
     // real-to-real plans (OLS_FLAG_R2R)
     float2 *hpack = nullptr;     // [ceil(F/2)][M] paired real filters h_{2p} + i h_{2p+1}
     uint16_t *tc_bmat = nullptr; // split DFT-16 matrices (fwd hi, fwd lo, inv hi, inv lo), core-matrix layout

@@ -28,31 +28,10 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 
-#include "ols_fft_passes.cuh"
+#include "ols_bank.cuh"
 #include "ols_internal.h"
-#include "tmem.cuh"
 
 namespace ols {
-
-template <int LOG2N, int MODE>
-struct PostGeo {
-    using G = Geo<LOG2N>;
-    // the modes that read the neighbours j - 1 and j + 1 of an output
-    static constexpr bool NEIGH = MODE == POST_DERIV || MODE == POST_PEAK;
-    // per segment (float2 units): the exchange buffers; DERIV's neighbourhood
-    // buffer; PEAK's warp-edge powers [2][T/32][16] floats (segments of several warps)
-    static constexpr int EDGE = (MODE == POST_PEAK && G::T > 32) ? (G::T / 32) * 16 : 0;
-    static constexpr int SLOT = G::XBUFS * G::PADN + (MODE == POST_DERIV ? G::PADN : 0) + EDGE;
-    static constexpr size_t SMEM_USED = sizeof(float2) * (size_t)(G::SEGS * SLOT);
-    // requested: at least enough that no more blocks fit on an SM (228 KB)
-    // than TMEM can serve, so a block's tcgen05.alloc never waits
-    static constexpr size_t SMEM = (SMEM_USED > (228u * 1024u) / (G::TMEM_MAX_CTAS + 1))
-                                       ? SMEM_USED
-                                       : (228u * 1024u) / (G::TMEM_MAX_CTAS + 1) + 1024u;
-    // the derivative's epilogue holds more live values: one resident block
-    // fewer per SM keeps it free of register spills
-    static constexpr int MINB = (MODE == POST_DERIV && G::MINB > 1) ? G::MINB - 1 : G::MINB;
-};
 
 // The peak test of one output with a candidate power pk (called by whole warps,
 // only when some lane has a candidate: it stays out of the common path's
@@ -104,238 +83,185 @@ __device__ __forceinline__ void append_candidates(bool hit, long long j, int f, 
     }
 }
 
-template <int LOG2N, int MODE>
-__global__ void __launch_bounds__(Geo<LOG2N>::BLOCK, (PostGeo<LOG2N, MODE>::MINB))
-ols_post_kernel(const float2 *__restrict__ sig, long long Ns, const float4 *__restrict__ Hk,
-                const float2 *__restrict__ twg, void *__restrict__ out, int M, int F, long long step,
-                long long nseg, long long Nout, float thr, ols_candidate *__restrict__ cand,
-                unsigned long long *__restrict__ count, long long cap, int *status) {
-    using G = Geo<LOG2N>;
-    using PG = PostGeo<LOG2N, MODE>;
-    extern __shared__ float4 smem_raw[];
-    __shared__ uint32_t tbase;
-    float2 *smem = reinterpret_cast<float2 *>(smem_raw);
-    const int slot = threadIdx.x / G::T;
-    const int t = threadIdx.x % G::T;
-    float2 *bufs = smem + slot * PG::SLOT;
-    float2 *dbuf = bufs + G::XBUFS * G::PADN;        // DERIV: the output's neighbourhood; PEAK: warp edges
-    // the forward kernel's TMEM layout: twiddles, then the segment spectrum (columns 96..127)
-    if (threadIdx.x < 32) tmem::alloc(&tbase, G::TMEM_COLS);
-    tmem::fence_before_sync();
-    __syncthreads();
-    tmem::fence_after_sync();
-    // the derivative runs the TMEM exchange at N = 2048 (at other N it
-    // spills); power and detection keep the exchange in shared memory (with
-    // it their epilogues spill: 0.525 vs 0.535 ms and 0.582 vs 0.613 ms on
-    // the filter bank)
-    constexpr bool xch = MODE == POST_DERIV && LOG2N == 11;
-    const TwTmemT<xch> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
-    tw_tmem_fill<LOG2N, xch>(twg, tw.base, t);
-    const uint32_t xcol = tw.base + 96;
-    // circular position of a segment's first output, and its input offset
-    const int n0 = PG::NEIGH ? M : M - 1;
-    const long long off = PG::NEIGH ? -1 : 0;
-    int xc = 0;
-    const long long nblk = (nseg + G::SEGS - 1) / G::SEGS;
-    for (long long blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
-        const long long seg = blk * G::SEGS + slot;
-        const bool active = seg < nseg;
-        const long long j0 = seg * step;                 // first output of this segment
-        const long long start = j0 + off;                // first input sample (may be -1)
-
-        // segment load: samples start + k T + t inside [0, Ns), zero elsewhere
-        float2 X[16];
-        {
-            const long long avail = active ? (Ns - start) : 0;
-            const int lim = (int)(avail < G::N ? avail : G::N);
-            const int first = active ? (int)(-start > 0 ? -start : 0) : 0;   // 1 only before s[0]
-            const float2 *src = sig + (active ? start : 0) + t;
+template <int MODE>
+struct EpiPost {
+    // the TMEM exchange everywhere (a CTA's registers now hold it without spills)
+    static constexpr bool XCH = true;
+    // PEAK: warp-edge powers [2][T/32][16] floats per segment of several warps
+    template <int LOG2N>
+    static constexpr int edge() {
+        return (MODE == POST_PEAK && Geo<LOG2N>::T > 32) ? (Geo<LOG2N>::T / 32) * 16 : 0;
+    }
+    const float2 *sig;
+    void *out;                      // POWER: float [F][Nout]; DERIV: float2 [F][Nout]
+    float thr;
+    ols_candidate *cand;
+    unsigned long long *count;
+    long long cap;
+    const float *dsin;              // DERIV: sin(2 pi nu / N) at each storage position
+    __device__ __forceinline__ float2 sample(long long i) const { return __ldg(sig + i); }
+    // DERIV: central differences of a circular sequence are the product of its
+    // spectrum with i sin(2 pi nu / N).  The segment's spectrum is scaled once
+    // for all its filters, so the inverse FFT yields the derivative itself and
+    // no output needs its neighbours.  A segment holding the first or the last
+    // output of the stream, whose differences are one-sided, keeps its plain
+    // spectrum and goes through the neighbour exchange below.  16- / 32-filter
+    // banks of 2^23 samples (N = 1024 / 2048): the exchange for every segment
+    // took 212 / 404 us (one CTA of 128 threads per segment group, one fewer
+    // per SM for its registers), this 142 / 317.
+    __device__ __forceinline__ static bool at_end(const BankSegment &sg) {
+        return sg.j0 == 0 || sg.Nout - sg.j0 == (long long)sg.span;
+    }
+    template <int LOG2N>
+    __device__ __forceinline__ void spectrum(float2 *X, int t, const BankSegment &sg) const {
+        if constexpr (MODE == POST_DERIV) {
+            if (!at_end(sg)) {
+                const float4 *p = reinterpret_cast<const float4 *>(dsin) + 4 * t;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float4 s = __ldg(p + q);
+                    X[4 * q] = make_float2(-s.x * X[4 * q].y, s.x * X[4 * q].x);
+                    X[4 * q + 1] = make_float2(-s.y * X[4 * q + 1].y, s.y * X[4 * q + 1].x);
+                    X[4 * q + 2] = make_float2(-s.z * X[4 * q + 2].y, s.z * X[4 * q + 2].x);
+                    X[4 * q + 3] = make_float2(-s.w * X[4 * q + 3].y, s.w * X[4 * q + 3].x);
+                }
+            }
+        }
+    }
+    template <int LOG2N, class BAR>
+    __device__ __forceinline__ void store(const float2 *x, int f, int t, const BankSegment &sg, float2 *bufs, int &xc,
+                                          const BAR &bar) const {
+        using G = Geo<LOG2N>;
+        const int v = t - sg.n0;             // output k T + v of the segment in register k
+        if constexpr (MODE == POST_POWER) {
+            float *dst = static_cast<float *>(out) + (size_t)f * (size_t)sg.Nout + (sg.j0 + v);
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+                if ((unsigned)(v + k * G::T) < (unsigned)sg.span && in_bounds(sg.j0 + v + k * G::T < sg.Nout, sg.status))
+                    __stcs(dst + k * G::T, fmaf(x[k].x, x[k].x, x[k].y * x[k].y));
+        } else if constexpr (MODE == POST_DETECT) {
+            // candidates are rare: one vote decides whether the warp has any at all
+            float pw[16];
+            bool any = false;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                pw[k] = fmaf(x[k].x, x[k].x, x[k].y * x[k].y);
+                any |= (unsigned)(v + k * G::T) < (unsigned)sg.span && pw[k] >= thr;
+            }
+            if (__any_sync(0xffffffffu, any)) {
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                    const bool hit = (unsigned)(v + k * G::T) < (unsigned)sg.span && pw[k] >= thr;
+                    append_candidates(hit, sg.j0 + (v + k * G::T), f, pw[k], cand, count, cap, sg.Nout, sg.status);
+                }
+            }
+        } else if constexpr (MODE == POST_PEAK) {
+            constexpr int W = G::T < 32 ? G::T : 32;          // threads of the segment in one warp
+            const int gl = t % W;
+            float pw[16];
+#pragma unroll
+            for (int k = 0; k < 16; ++k) pw[k] = fmaf(x[k].x, x[k].x, x[k].y * x[k].y);
+            // segments of several warps: first[w][k] at edge[w * 16 + k], last[w][k] after them
+            float *ed = reinterpret_cast<float *>(bufs + G::XBUFS * G::PADN);
+            if constexpr (edge<LOG2N>() > 0) {
+                if (gl == 0 || gl == W - 1) {
+                    float4 *e = reinterpret_cast<float4 *>(ed + ((gl == 0 ? 0 : G::T / 32) + t / 32) * 16);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        e[q] = make_float4(pw[4 * q], pw[4 * q + 1], pw[4 * q + 2], pw[4 * q + 3]);
+                }
+                bar();
+            }
+            // first and last output of the stream (one neighbour only), if in this segment
+            const long long rem = sg.Nout - sg.j0;
+            const int k_first = sg.j0 == 0 ? 0 : -2;
+            const int k_last = (sg.span > 0 && rem == (long long)sg.span) ? sg.span - 1 : -2;
+            bool any = false;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) any |= (unsigned)(v + k * G::T) < (unsigned)sg.span && pw[k] >= thr;
+            if (!__any_sync(0xffffffffu, any)) return;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                const int o = v + k * G::T;
+                bool hit = (unsigned)o < (unsigned)sg.span && pw[k] >= thr &&
+                           in_bounds(o + sg.n0 >= 1 && o + sg.n0 + 1 < G::N, sg.status);
+                if (__any_sync(0xffffffffu, hit))
+                    hit = peak_test<G::T>(hit, pw[k], (gl == W - 1) ? pw[k > 0 ? k - 1 : 0] : pw[k],
+                                          (gl == 0) ? pw[k < 15 ? k + 1 : 15] : pw[k], t, k, o == k_first,
+                                          o == k_last, ed);
+                append_candidates(hit, sg.j0 + o, f, pw[k], cand, count, cap, sg.Nout, sg.status);
+            }
+        } else if (!at_end(sg)) {
+            float2 *dst = static_cast<float2 *>(out) + (size_t)f * (size_t)sg.Nout + (sg.j0 + v);
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+                if ((unsigned)(v + k * G::T) < (unsigned)sg.span && in_bounds(sg.j0 + v + k * G::T < sg.Nout, sg.status))
+                    __stcs(dst + k * G::T, x[k]);
+        } else {
+            // y (circular order) to the exchange buffer not in use, padded q -> q + q/16;
+            // then each output reads its two neighbours
+            float2 *dbuf = bufs + (xc & 1) * G::PADN;
+            ++xc;
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
                 const int n = k * G::T + t;
-                const long long i = (active ? start : 0) + n;
-                X[k] = (n >= first && n < lim && in_bounds(i >= 0 && i < Ns, status)) ? __ldg(src + k * G::T)
-                                                                                     : make_float2(0.f, 0.f);
+                dbuf[n + (n >> 4)] = x[k];
             }
-        }
-        forward_passes<LOG2N, 0>(X, bufs, tw, t, xc);
-        tmem::st32(xcol, reinterpret_cast<const float *>(X));
-        tmem::wait_st();
-
-        const long long rem = active ? (Nout - j0) : 0;
-        const int span = (int)(rem < step ? rem : step);
-
-        float4 hn[8];
-        const long long hn_end = (long long)F * (G::N / 2);   // float4 entries of the spectra
+            bar();
+            float2 *dst = static_cast<float2 *>(out) + (size_t)f * (size_t)sg.Nout + (sg.j0 - sg.n0);
+            // circular positions of outputs j = 0 and j = Nout-1 (one-sided ends), if in this segment
+            const int n_first = sg.j0 == 0 ? sg.n0 : -2;
+            const int n_last = (sg.Nout - sg.j0 == (long long)sg.span) ? sg.span - 1 + sg.n0 : -2;
 #pragma unroll
-        for (int j2 = 0; j2 < 8; ++j2)
-            if (in_bounds(j2 * G::T + t < hn_end, status)) hn[j2] = load_spectrum(Hk + j2 * G::T + t);
-        for (int f = 0; f < F; ++f) {
-            float2 x[16];
-            tmem::ld32(xcol, reinterpret_cast<float *>(x));
-            tmem::wait_ld();
-#pragma unroll
-            for (int j2 = 0; j2 < 8; ++j2) {
-                x[2 * j2] = cmul(x[2 * j2], make_float2(hn[j2].x, hn[j2].y));
-                x[2 * j2 + 1] = cmul(x[2 * j2 + 1], make_float2(hn[j2].z, hn[j2].w));
-            }
-            if (f + 1 < F) {
-                const float4 *hp = Hk + (size_t)(f + 1) * (G::N / 2) + t;
-#pragma unroll
-                for (int j2 = 0; j2 < 8; ++j2)
-                    if (in_bounds((long long)(f + 1) * (G::N / 2) + j2 * G::T + t < hn_end, status))
-                        hn[j2] = load_spectrum(hp + j2 * G::T);
-            }
-            inverse_passes<LOG2N, G::NP - 1>(x, bufs, tw, t, xc);
-
-            if constexpr (MODE == POST_POWER) {
-                float *dst = static_cast<float *>(out) + (size_t)f * (size_t)Nout + (j0 - n0);
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const int n = k * G::T + t;
-                    if ((unsigned)(n - n0) < (unsigned)span && in_bounds(j0 - n0 + n >= 0 && j0 - n0 + n < Nout, status))
-                        dst[n] = fmaf(x[k].x, x[k].x, x[k].y * x[k].y);
-                }
-            } else if constexpr (MODE == POST_DETECT) {
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const int n = k * G::T + t;
-                    const float p = fmaf(x[k].x, x[k].x, x[k].y * x[k].y);
-                    const bool hit = (unsigned)(n - n0) < (unsigned)span && p >= thr;
-                    append_candidates(hit, j0 + (n - n0), f, p, cand, count, cap, Nout, status);
-                }
-            } else if constexpr (MODE == POST_PEAK) {
-                constexpr int W = G::T < 32 ? G::T : 32;          // threads of the segment in one warp
-                const int gl = t % W;
-                float pw[16];
-#pragma unroll
-                for (int k = 0; k < 16; ++k) pw[k] = fmaf(x[k].x, x[k].x, x[k].y * x[k].y);
-                // segments of several warps: first[w][k] at edge[w * 16 + k], last[w][k] after them
-                float *edge = reinterpret_cast<float *>(dbuf);
-                if constexpr (PG::EDGE > 0) {
-                    if (gl == 0 || gl == W - 1) {
-                        float4 *e = reinterpret_cast<float4 *>(edge + ((gl == 0 ? 0 : G::T / 32) + t / 32) * 16);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            e[q] = make_float4(pw[4 * q], pw[4 * q + 1], pw[4 * q + 2], pw[4 * q + 3]);
-                    }
-                    __syncthreads();
-                }
-                // circular positions of outputs j = 0 and j = Nout-1 (one neighbour only), if in this segment
-                const int n_first = j0 == 0 ? n0 : -2;
-                const int n_last = (rem <= step) ? (int)(rem - 1) + n0 : -2;
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const int n = k * G::T + t;
-                    bool hit = (unsigned)(n - n0) < (unsigned)span && pw[k] >= thr &&
-                               in_bounds(n >= 1 && n + 1 < G::N, status);
-                    if (__any_sync(0xffffffffu, hit))
-                        hit = peak_test<G::T>(hit, pw[k], (gl == W - 1) ? pw[k > 0 ? k - 1 : 0] : pw[k],
-                                              (gl == 0) ? pw[k < 15 ? k + 1 : 15] : pw[k], t, k, n == n_first,
-                                              n == n_last, edge);
-                    append_candidates(hit, j0 + (n - n0), f, pw[k], cand, count, cap, Nout, status);
-                }
-            } else {
-                // write y (circular order) to the neighbourhood buffer, padded q -> q + q/16
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const int n = k * G::T + t;
-                    dbuf[n + (n >> 4)] = x[k];
-                }
-                __syncthreads();
-                float2 *dst = static_cast<float2 *>(out) + (size_t)f * (size_t)Nout + (j0 - n0);
-                // circular positions of outputs j = 0 and j = Nout-1 (one-sided ends), if in this segment
-                const int n_first = j0 == 0 ? n0 : -2;
-                const int n_last = (rem <= step) ? (int)(rem - 1) + n0 : -2;
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const int n = k * G::T + t;
-                    if ((unsigned)(n - n0) < (unsigned)span &&
-                        in_bounds(j0 - n0 + n >= 0 && j0 - n0 + n < Nout && n >= 1 && n + 1 < G::N, status)) {
-                        const int lo = (n == n_first) ? n : n - 1;
-                        const int hi = (n == n_last) ? n : n + 1;
-                        const float sc = (lo == n || hi == n) ? 1.f : 0.5f;
-                        const float2 a = dbuf[lo + (lo >> 4)], b = dbuf[hi + (hi >> 4)];
-                        dst[n] = make_float2((b.x - a.x) * sc, (b.y - a.y) * sc);
-                    }
+            for (int k = 0; k < 16; ++k) {
+                const int n = k * G::T + t;
+                if ((unsigned)(n - sg.n0) < (unsigned)sg.span &&
+                    in_bounds(sg.j0 - sg.n0 + n < sg.Nout && n >= 1 && n + 1 < G::N, sg.status)) {
+                    const int lo = (n == n_first) ? n : n - 1;
+                    const int hi = (n == n_last) ? n : n + 1;
+                    const float sc = (lo == n || hi == n) ? 1.f : 0.5f;
+                    const float2 a = dbuf[lo + (lo >> 4)], b = dbuf[hi + (hi >> 4)];
+                    __stcs(dst + n, make_float2((b.x - a.x) * sc, (b.y - a.y) * sc));
                 }
             }
         }
     }
-    tmem::fence_before_sync();
-    __syncthreads();
-    tmem::fence_after_sync();
-    if (threadIdx.x < 32) tmem::dealloc(tbase, G::TMEM_COLS);
-}
+};
 
-template <int LOG2N, int MODE>
-static cudaError_t post_prepare_nm(ols_plan_s &p) {
-    using G = Geo<LOG2N>;
-    using PG = PostGeo<LOG2N, MODE>;
-    cudaError_t e = cudaFuncSetAttribute(ols_post_kernel<LOG2N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)PG::SMEM);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = resident_blocks_tmem(ols_post_kernel<LOG2N, MODE>, G::BLOCK, PG::SMEM, (int)G::TMEM_COLS, &per_sm);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    p.post_grid_cap[MODE] = per_sm * p.sm_count;
-    return cudaSuccess;
-}
-
-template <int LOG2N>
-static cudaError_t post_prepare_n(ols_plan_s &p) {
-    cudaError_t e = post_prepare_nm<LOG2N, POST_POWER>(p);
-    if (e == cudaSuccess) e = post_prepare_nm<LOG2N, POST_DETECT>(p);
-    if (e == cudaSuccess) e = post_prepare_nm<LOG2N, POST_DERIV>(p);
-    if (e == cudaSuccess) e = post_prepare_nm<LOG2N, POST_PEAK>(p);
+cudaError_t post_prepare(ols_plan_s &p) {
+    cudaError_t e = bank_prepare_any<EpiPost<POST_POWER>>(p.log2N);
+    if (e == cudaSuccess) e = bank_prepare_any<EpiPost<POST_DETECT>>(p.log2N);
+    if (e == cudaSuccess) e = bank_prepare_any<EpiPost<POST_DERIV>>(p.log2N);
+    if (e == cudaSuccess) e = bank_prepare_any<EpiPost<POST_PEAK>>(p.log2N);
     return e;
 }
 
-cudaError_t post_prepare(ols_plan_s &p) {
-    switch (p.log2N) {
-        case 8: return post_prepare_n<8>(p);
-        case 9: return post_prepare_n<9>(p);
-        case 10: return post_prepare_n<10>(p);
-        case 11: return post_prepare_n<11>(p);
-        case 12: return post_prepare_n<12>(p);
-        case 13: return post_prepare_n<13>(p);
-        default: return cudaErrorInvalidValue;
-    }
-}
-
-template <int LOG2N, int MODE>
-static cudaError_t post_launch_nm(const ols_plan_s &p, const PostArgs &a, cudaStream_t st) {
-    using G = Geo<LOG2N>;
-    using PG = PostGeo<LOG2N, MODE>;
-    const int64_t nblk = (a.nseg + G::SEGS - 1) / G::SEGS;
-    const int cap = p.post_grid_cap[MODE];
-    const int grid = fused_grid(LOG2N, nblk, cap);
-    ols_post_kernel<LOG2N, MODE><<<grid, G::BLOCK, PG::SMEM, st>>>(
-        a.s, a.Ns, reinterpret_cast<const float4 *>(p.Hk), p.tw8, a.out, p.M, p.F, a.step, a.nseg, a.Nout, a.thr,
-        a.cand, a.count, a.cap, p.d_status);
-    return cudaGetLastError();
-}
-
-template <int LOG2N>
-static cudaError_t post_launch_n(const ols_plan_s &p, const PostArgs &a, cudaStream_t st) {
-    switch (a.mode) {
-        case POST_POWER: return post_launch_nm<LOG2N, POST_POWER>(p, a, st);
-        case POST_DETECT: return post_launch_nm<LOG2N, POST_DETECT>(p, a, st);
-        case POST_DERIV: return post_launch_nm<LOG2N, POST_DERIV>(p, a, st);
-        case POST_PEAK: return post_launch_nm<LOG2N, POST_PEAK>(p, a, st);
-        default: return cudaErrorInvalidValue;
-    }
+template <int MODE>
+static cudaError_t post_launch_mode(const ols_plan_s &p, const PostArgs &a, cudaStream_t st) {
+    // derivative and peaks read the neighbours j - 1 and j + 1 of an output:
+    // their segments start one sample early
+    constexpr bool NEIGH = MODE == POST_DERIV || MODE == POST_PEAK;
+    BankArgs b{};
+    b.Hk = reinterpret_cast<const float4 *>(p.Hk);
+    b.tw8 = p.tw8;
+    b.F = p.F;
+    b.n0 = NEIGH ? p.M : p.M - 1;
+    b.step = a.step;
+    b.off = NEIGH ? -1 : 0;
+    b.Ns = a.Ns;
+    b.Nout = a.Nout;
+    b.nseg = a.nseg;
+    b.status = p.d_status;
+    return bank_launch_any(p.log2N, b, EpiPost<MODE>{a.s, a.out, a.thr, a.cand, a.count, (long long)a.cap, p.dsin}, p.sm_count,
+                           st);
 }
 
 cudaError_t post_launch(const ols_plan_s &p, const PostArgs &a, cudaStream_t st) {
-    switch (p.log2N) {
-        case 8: return post_launch_n<8>(p, a, st);
-        case 9: return post_launch_n<9>(p, a, st);
-        case 10: return post_launch_n<10>(p, a, st);
-        case 11: return post_launch_n<11>(p, a, st);
-        case 12: return post_launch_n<12>(p, a, st);
-        case 13: return post_launch_n<13>(p, a, st);
+    switch (a.mode) {
+        case POST_POWER: return post_launch_mode<POST_POWER>(p, a, st);
+        case POST_DETECT: return post_launch_mode<POST_DETECT>(p, a, st);
+        case POST_DERIV: return post_launch_mode<POST_DERIV>(p, a, st);
+        case POST_PEAK: return post_launch_mode<POST_PEAK>(p, a, st);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -55,6 +55,8 @@ struct EpiReal {
     float *y;
     int F;                  // real filters (F spectra of the bank kernel: pairs)
     __device__ __forceinline__ float2 sample(long long i) const { return make_float2(__ldg(sig + i), 0.f); }
+    template <int LOG2N>
+    __device__ __forceinline__ void spectrum(float2 *, int, const BankSegment &) const {}
     template <int LOG2N, class BAR>
     __device__ __forceinline__ void store(const float2 *x, int p, int t, const BankSegment &sg, float2 *, int &,
                                           const BAR &) const {

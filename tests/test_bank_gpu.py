@@ -1,9 +1,11 @@
-"""The bank kernel's work sharing and block sizes against the FP64 oracle.
+"""The bank kernel's work sharing and block sizes, and the derivative in the
+frequency domain, against the FP64 oracle.
 
 Shapes sit where the schedule can go wrong: fewer steps (blocks of segments x
 filters) than resident CTAs, one filter, shares that begin and end inside a
 segment's filters, idle slots in the last block, both block sizes.  Bounds are
-those of the parity tests: 2e-6 relative L2 (FP32 path).
+those of the parity tests: 2e-6 relative L2 (FP32 path), the derivative's error
+relative to the norm of y.
 """
 import numpy as np
 import pytest
@@ -87,3 +89,21 @@ def test_real_schedule_against_oracle(N, M, F, Ns):
     assert oracle.max_stream_rel_l2(y, ref, oracle.stream_scale(s, h, y.shape[1])) <= TOL
     plan.close()
 
+
+@pytest.mark.parametrize("N,M", [(256, 33), (512, 65), (1024, 129), (2048, 257), (4096, 513), (8192, 1025)])
+@pytest.mark.parametrize("extra", [2, 3, -1, 0, 1, 2 * 4096 + 5])
+def test_derivative_ends(N, M, extra):
+    """Two or three outputs in all, and a last segment of one output fewer
+    than, exactly, and one more than a full one (the one-sided ends)."""
+    step = N - M - 1
+    nout = extra if extra in (2, 3) else 3 * step + extra
+    s, h = inputs(N + extra + 7, nout + M - 1, 3, M)
+    plan = Plan(M, 3, N)
+    plan.set_filters(dev(h))
+    d = plan.convolve_derivative(dev(s)).cpu().numpy()
+    y = oracle.conv(s, h)
+    ref = oracle.derivative(s, h)
+    scale = oracle.stream_scale(s, h, nout)
+    err = max(np.linalg.norm(d[f] - ref[f]) / max(np.linalg.norm(y[f]), scale[f]) for f in range(3))
+    assert err <= TOL
+    plan.close()
