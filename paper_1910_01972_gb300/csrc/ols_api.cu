@@ -343,11 +343,8 @@ int ols_set_filters(ols_plan_t plan, const float *h, void *stream) {
     if (!plan || !h || !aligned8(h)) return OLS_ERR_INVALID;
     if (plan->flags == OLS_FLAG_R2R) return OLS_ERR_UNSUPPORTED;
     const float2 *hh = reinterpret_cast<const float2 *>(h);
-    cudaError_t e = launch_spectra(hh, plan->M, plan->F, plan->log2N, plan->nu, plan->tw64, plan->Hk, 0,
+    cudaError_t e = launch_spectra(hh, plan->M, plan->F, plan->log2N, plan->nu, plan->tw64, plan->Hk, plan->Htk,
                                    (cudaStream_t)stream);
-    if (e == cudaSuccess)
-        e = launch_spectra(hh, plan->M, plan->F, plan->log2N, plan->nu, plan->tw64, plan->Htk, 1,
-                           (cudaStream_t)stream);
     if (e != cudaSuccess) return status_of(e);
     plan->filters_ready = true;
     return OLS_OK;
@@ -407,7 +404,7 @@ int ols_set_filters_real(ols_plan_t plan, const float *h, void *stream) {
     const int Fc = (plan->F + 1) / 2;
     cudaError_t e = launch_pack_real_pairs(h, plan->M, plan->F, plan->hpack, (cudaStream_t)stream);
     if (e == cudaSuccess)
-        e = launch_spectra(plan->hpack, plan->M, Fc, plan->log2N, plan->nu, plan->tw64, plan->Hk, 0,
+        e = launch_spectra(plan->hpack, plan->M, Fc, plan->log2N, plan->nu, plan->tw64, plan->Hk, nullptr,
                            (cudaStream_t)stream);
     if (e != cudaSuccess) return status_of(e);
     plan->filters_ready = true;

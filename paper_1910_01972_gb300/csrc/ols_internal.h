@@ -242,11 +242,11 @@ cudaError_t prepare_backward(ols_plan_s &p);
 cudaError_t launch_backward(const ols_plan_s &p, const BackwardArgs &a, cudaStream_t st, int *launches);
 int backward_grid(const ols_plan_s &p, int64_t nseg, bool want_ds, bool want_dh);
 int backward_segs_per_block(int log2N);
-// FP64 precompute kernels.  adjoint != 0 transforms conj(h_f[M-1-k]) instead of h_f[k].
+// FP64 precompute kernels.  Htk (may be null): the spectra of conj(h_f[M-1-k]).
 cudaError_t launch_tw64(double2 *tw64, int N, cudaStream_t st);
 // Spectra in the 16-points-per-thread register layout of the kernels.
 cudaError_t launch_spectra(const float2 *h, int M, int F, int log2N, const int32_t *nu,
-                           const double2 *tw64, float2 *Hk, int adjoint, cudaStream_t st);
+                           const double2 *tw64, float2 *Hk, float2 *Htk, cudaStream_t st);
 cudaError_t launch_spectra_natural(const float2 *Hk, int F, int log2N, const int32_t *nu,
                                    float2 *H, cudaStream_t st);
 
