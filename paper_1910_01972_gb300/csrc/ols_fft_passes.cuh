@@ -112,6 +112,11 @@ struct Geo {
                                             : (228u * 1024u) / (TMEM_MAX_CTAS + 1) + 1024u;
 };
 
+// How a kernel with TMEM twiddles exchanges between the last two passes:
+// through shared memory, through TMEM where Geo<>::TX allows it, or (N = 2048;
+// else as XCHG_TMEM) through TMEM with one of the three bits by shuffles.
+enum : int { XCHG_SMEM = 0, XCHG_TMEM = 1, XCHG_SHFL = 2 };
+
 // Whether segment length 2^LOG2N is in a mask of segment lengths (bit i for
 // N = 2^(9 + i)), the form of the per-kernel TMEM-exchange choices.
 template <int LOG2N>
@@ -186,23 +191,19 @@ __device__ __forceinline__ void exchange(float2 *x, float2 *buf, int t, const BA
 // p2, p7), warp = p9, p10; pass 2 (radix 8 over p0..p2): thread = p4..p10,
 // register = p0..p3 (the layout of the spectrum).  Shared exchange of passes
 // 0 and 1: position q at q ^ (p8 << 3) (no padding).
-#ifndef TX11S
-#define TX11S 0
-#endif
-#if TX11S
-__device__ __forceinline__ int tx11_addr0(int t, int k) {
-    return t + 130 * (k & 1) + 264 * ((k >> 1) & 1) + 528 * (k >> 2);
-}
-__device__ __forceinline__ int tx11_addr1(int t, int k) {
-    return ((t >> 3) & 3) + 4 * (t & 1) + 130 * ((t >> 1) & 1) + 264 * ((t >> 2) & 1) + 528 * (t >> 5) + 8 * k;
-}
-#else
 __device__ __forceinline__ int tx11_addr0(int t, int k) { return ((k & 2) ? (t ^ 8) : t) + 128 * k; }
 __device__ __forceinline__ int tx11_addr1(int t, int k) {
     const int base = ((t >> 1) & 7) + 128 * ((t >> 4) & 1) + 256 * (t & 1) + 512 * (t >> 5);
     return base + 8 * ((k & 1) ^ (t & 1)) + 16 * (k >> 1);
 }
-#endif
+// N = 2048 with shuffles (XCHG_SHFL): pass 1 lanes (p2, p7, p8, p0, p1); position
+// q at p0..p6 + 130 p7 + 264 p8 + 528 (p9 + 2 p10).
+__device__ __forceinline__ int tx11s_addr0(int t, int k) {
+    return t + 130 * (k & 1) + 264 * ((k >> 1) & 1) + 528 * (k >> 2);
+}
+__device__ __forceinline__ int tx11s_addr1(int t, int k) {
+    return ((t >> 3) & 3) + 4 * (t & 1) + 130 * ((t >> 1) & 1) + 264 * ((t >> 2) & 1) + 528 * (t >> 5) + 8 * k;
+}
 
 // N = 4096 (Geo<12>::TX): pass 0 thread = p0..p7, register = p8..p11; pass 1
 // (radix 16 over p4..p7) lanes (p0, p1, p8, p2, p3), warp p9..p11; pass 2
@@ -226,22 +227,23 @@ __device__ __forceinline__ int tx10_addr0(int t, int k) { return t + 66 * k; }
 __device__ __forceinline__ int tx10_addr1(int t, int k) {
     return ((t >> 3) & 3) + 66 * ((t & 7) + 8 * (t >> 5)) + 4 * k;
 }
-template <int LOG2N, int P>
+template <int LOG2N, int P, int XCH>
 __device__ __forceinline__ int tx_addr(int t, int k) {
-    if constexpr (LOG2N == 10) return P == 0 ? tx10_addr0(t, k) : tx10_addr1(t, k);
+    if constexpr (LOG2N == 11 && XCH == XCHG_SHFL) return P == 0 ? tx11s_addr0(t, k) : tx11s_addr1(t, k);
+    else if constexpr (LOG2N == 10) return P == 0 ? tx10_addr0(t, k) : tx10_addr1(t, k);
     else if constexpr (LOG2N == 11) return P == 0 ? tx11_addr0(t, k) : tx11_addr1(t, k);
     else if constexpr (LOG2N == 12) return P == 0 ? tx12_addr0(t, k) : tx12_addr1(t, k);
     else return P == 0 ? tx9_addr0(t, k) : tx9_addr1(t, k);
 }
 // The shared-memory exchange of passes 0 and 1 when pass 1 is relabelled.
-template <int LOG2N, int PW, int PR, class BAR>
+template <int LOG2N, int PW, int PR, int XCH, class BAR>
 __device__ __forceinline__ void exchange_tx(float2 *x, float2 *buf, int t, const BAR &bar) {
     if constexpr (Geo<LOG2N>::XBUFS == 1) bar();
 #pragma unroll
-    for (int k = 0; k < 16; ++k) buf[tx_addr<LOG2N, PW>(t, k)] = x[k];
+    for (int k = 0; k < 16; ++k) buf[tx_addr<LOG2N, PW, XCH>(t, k)] = x[k];
     bar();
 #pragma unroll
-    for (int k = 0; k < 16; ++k) x[k] = buf[tx_addr<LOG2N, PR>(t, k)];
+    for (int k = 0; k < 16; ++k) x[k] = buf[tx_addr<LOG2N, PR, XCH>(t, k)];
 }
 
 // A warp's TMEM stores are complete (wait::st) before any lane loads them
@@ -256,62 +258,6 @@ __device__ __forceinline__ void tx_sync() { __syncwarp(); }
 //  2. a 32x32b store (column = (re/im, p4, p5, p2, p3)); 16x256b loads:
 //     thread lanes (p4..p8), x[p0 + 2 p1 + 4 p2 + 8 p3] from
 //     w[p1][4 (p2 + 2 p3) + 2 p0 + re/im].
-#if TX11S
-// v[2 (p4 + 2 p5 + 4 p2 + 8 p3) + re/im] with lane bit 0 = p6  <->  x[p3 + 2 p4 + 4 p5 + 8 p6] with lane bit 0 = p2
-__device__ __forceinline__ void tx11_forward(float2 *x, uint32_t xb) {
-    const bool odd = threadIdx.x & 1;
-    float v[32];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {      // i = p3 + 2 p4 + 4 p5
-        const int o = 2 * ((i >> 1) + 8 * (i & 1));
-        const float2 c = x[i], d = x[i + 8];
-        const float rx = __shfl_xor_sync(0xffffffffu, odd ? c.x : d.x, 1);
-        const float ry = __shfl_xor_sync(0xffffffffu, odd ? c.y : d.y, 1);
-        v[o] = odd ? rx : c.x;
-        v[o + 1] = odd ? ry : c.y;
-        v[o + 8] = odd ? d.x : rx;
-        v[o + 9] = odd ? d.y : ry;
-    }
-    tmem::st32(xb, v);
-    tmem::wait_st();
-    tx_sync();
-    float w[2][16];
-    tmem::ld16x256b_x4(xb, w[0]);
-    tmem::ld16x256b_x4(xb + (16u << 16), w[1]);
-    tmem::wait_ld();
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {   // k = p0 + 2 p1 + 4 p2 + 8 p3
-        const int p0 = k & 1, p1 = (k >> 1) & 1, p23 = k >> 2;
-        x[k] = make_float2(w[p1][4 * p23 + 2 * p0], w[p1][4 * p23 + 2 * p0 + 1]);
-    }
-}
-__device__ __forceinline__ void tx11_inverse(float2 *x, uint32_t xb) {
-    const bool odd = threadIdx.x & 1;
-    float w[2][16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        const int p0 = k & 1, p1 = (k >> 1) & 1, p23 = k >> 2;
-        w[p1][4 * p23 + 2 * p0] = x[k].x;
-        w[p1][4 * p23 + 2 * p0 + 1] = x[k].y;
-    }
-    tmem::st16x256b_x4(xb, w[0]);
-    tmem::st16x256b_x4(xb + (16u << 16), w[1]);
-    tmem::wait_st();
-    tx_sync();
-    float v[32];
-    tmem::ld32(xb, v);
-    tmem::wait_ld();
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {      // i = p3 + 2 p4 + 4 p5
-        const int o = 2 * ((i >> 1) + 8 * (i & 1));
-        const float2 a = make_float2(v[o], v[o + 1]), b = make_float2(v[o + 8], v[o + 9]);
-        const float rx = __shfl_xor_sync(0xffffffffu, odd ? a.x : b.x, 1);
-        const float ry = __shfl_xor_sync(0xffffffffu, odd ? a.y : b.y, 1);
-        x[i] = make_float2(odd ? rx : a.x, odd ? ry : a.y);
-        x[i + 8] = make_float2(odd ? b.x : rx, odd ? b.y : ry);
-    }
-}
-#else
 __device__ __forceinline__ void tx11_forward(float2 *x, uint32_t xb) {
 #pragma unroll
     for (int k = 0; k < 8; ++k)      // k = p3 + 2 p4 + 4 p5; registers (x[k], x[k + 8]) differ in p6
@@ -374,7 +320,67 @@ __device__ __forceinline__ void tx11_inverse(float2 *x, uint32_t xb) {
                                x[k].y, x[k + 8].x, x[k + 8].y);
     tmem::wait_ld();
 }
-#endif
+// The same exchange with one round trip (the form of N = 1024: registers p2..p5,
+// lanes (p6, p7, p8, p0, p1)) and the third bit traded by shuffles: each lane of
+// a pair sends half of its registers, v[2 (p4 + 2 p5 + 4 p2 + 8 p3) + re/im] with
+// lane bit 0 = p6 <-> x[p3 + 2 p4 + 4 p5 + 8 p6] with lane bit 0 = p2.  Sixteen
+// shuffles and 48 selects take the place of a round trip and its register
+// moves; which is faster depends on the epilogue (32 filters, 2^23 samples:
+// plain store 533 us against 508, real pairs 271 against 274; 16 filters:
+// power 268 against 276, derivative 326 against 316).
+__device__ __forceinline__ void tx11s_forward(float2 *x, uint32_t xb) {
+    const bool odd = threadIdx.x & 1;
+    float v[32];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {      // i = p3 + 2 p4 + 4 p5
+        const int o = 2 * ((i >> 1) + 8 * (i & 1));
+        const float2 c = x[i], d = x[i + 8];
+        const float rx = __shfl_xor_sync(0xffffffffu, odd ? c.x : d.x, 1);
+        const float ry = __shfl_xor_sync(0xffffffffu, odd ? c.y : d.y, 1);
+        v[o] = odd ? rx : c.x;
+        v[o + 1] = odd ? ry : c.y;
+        v[o + 8] = odd ? d.x : rx;
+        v[o + 9] = odd ? d.y : ry;
+    }
+    tmem::st32(xb, v);
+    tmem::wait_st();
+    tx_sync();
+    float w[2][16];
+    tmem::ld16x256b_x4(xb, w[0]);
+    tmem::ld16x256b_x4(xb + (16u << 16), w[1]);
+    tmem::wait_ld();
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {   // k = p0 + 2 p1 + 4 p2 + 8 p3
+        const int p0 = k & 1, p1 = (k >> 1) & 1, p23 = k >> 2;
+        x[k] = make_float2(w[p1][4 * p23 + 2 * p0], w[p1][4 * p23 + 2 * p0 + 1]);
+    }
+}
+__device__ __forceinline__ void tx11s_inverse(float2 *x, uint32_t xb) {
+    const bool odd = threadIdx.x & 1;
+    float w[2][16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const int p0 = k & 1, p1 = (k >> 1) & 1, p23 = k >> 2;
+        w[p1][4 * p23 + 2 * p0] = x[k].x;
+        w[p1][4 * p23 + 2 * p0 + 1] = x[k].y;
+    }
+    tmem::st16x256b_x4(xb, w[0]);
+    tmem::st16x256b_x4(xb + (16u << 16), w[1]);
+    tmem::wait_st();
+    tx_sync();
+    float v[32];
+    tmem::ld32(xb, v);
+    tmem::wait_ld();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {      // i = p3 + 2 p4 + 4 p5
+        const int o = 2 * ((i >> 1) + 8 * (i & 1));
+        const float2 a = make_float2(v[o], v[o + 1]), b = make_float2(v[o + 8], v[o + 9]);
+        const float rx = __shfl_xor_sync(0xffffffffu, odd ? a.x : b.x, 1);
+        const float ry = __shfl_xor_sync(0xffffffffu, odd ? a.y : b.y, 1);
+        x[i] = make_float2(odd ? rx : a.x, odd ? ry : a.y);
+        x[i + 8] = make_float2(odd ? b.x : rx, odd ? b.y : ry);
+    }
+}
 
 // N = 4096, pass 1 -> pass 2 (registers p4 + 2 p5 + 4 p6 + 8 p7), two round
 // trips:
@@ -562,16 +568,18 @@ __device__ __forceinline__ void tx10_inverse(float2 *x, uint32_t xb) {
     }
 }
 
-template <int LOG2N>
+template <int LOG2N, int XCH>
 __device__ __forceinline__ void tx_forward(float2 *x, uint32_t xb) {
     if constexpr (LOG2N == 12) tx12_forward(x, xb);
+    else if constexpr (LOG2N == 11 && XCH == XCHG_SHFL) tx11s_forward(x, xb);
     else if constexpr (LOG2N == 11) tx11_forward(x, xb);
     else if constexpr (LOG2N == 10) tx10_forward(x, xb);
     else tx9_forward(x, xb);
 }
-template <int LOG2N>
+template <int LOG2N, int XCH>
 __device__ __forceinline__ void tx_inverse(float2 *x, uint32_t xb) {
     if constexpr (LOG2N == 12) tx12_inverse(x, xb);
+    else if constexpr (LOG2N == 11 && XCH == XCHG_SHFL) tx11s_inverse(x, xb);
     else if constexpr (LOG2N == 11) tx11_inverse(x, xb);
     else if constexpr (LOG2N == 10) tx10_inverse(x, xb);
     else tx9_inverse(x, xb);
@@ -579,11 +587,11 @@ __device__ __forceinline__ void tx_inverse(float2 *x, uint32_t xb) {
 
 // Index n' = position mod s of pass P's twiddle W_{16 s}^{n' k} for thread t
 // (XCH: the kernel uses the TMEM exchange, which relabels pass NP-2).
-template <int LOG2N, int P, bool XCH>
+template <int LOG2N, int P, int XCH>
 __device__ __forceinline__ int tw_index(int t) {
     using G = Geo<LOG2N>;
     if constexpr (XCH && G::TX_RELABEL && P == G::NP - 2) {   // the relabelled lanes holding p0 .. p(s-1)
-        if constexpr (LOG2N == 11) return TX11S ? ((t >> 3) & 3) + 4 * (t & 1) : (t >> 1) & 7;
+        if constexpr (LOG2N == 11) return XCH == XCHG_SHFL ? ((t >> 3) & 3) + 4 * (t & 1) : (t >> 1) & 7;
         else if constexpr (LOG2N == 12) return (t & 3) + 4 * ((t >> 3) & 1) + 8 * ((t >> 4) & 1);
         else if constexpr (LOG2N == 10) return (t >> 3) & 3;
         else return (t >> 1) & 1;
@@ -653,9 +661,9 @@ struct TwGlobal {
 // stage's sixteen words are loaded while the other stages run.
 // XCH: the segment FFT also uses the TMEM exchange where Geo<>::TX allows it
 // (kernels whose epilogue needs the registers opt out).
-template <bool XCH = true>
+template <int XCH = XCHG_TMEM>
 struct TwTmemT {
-    static constexpr bool xchg = XCH;
+    static constexpr int xchg = XCH;
     uint32_t base;
     // columns 64..95: the staging area of the TMEM exchange
     __device__ __forceinline__ uint32_t xbase() const { return base + 64; }
@@ -696,18 +704,18 @@ struct TwTmemT {
 using TwTmem = TwTmemT<true>;
 template <class TW>
 struct is_tw_tmem : std::false_type {};
-template <bool X>
+template <int X>
 struct is_tw_tmem<TwTmemT<X>> : std::true_type {};
 template <class TW>
 __device__ __forceinline__ constexpr bool tw_xchg() {
-    if constexpr (is_tw_tmem<TW>::value) return TW::xchg;
+    if constexpr (is_tw_tmem<TW>::value) return TW::xchg != XCHG_SMEM;
     else return false;
 }
 
 // Fill a TwTmemT<XCH> for thread t from the plan's folded-twiddle table (pass
 // P at offset tw8_off(P): eight rows of stride(P) entries, row i at n' holding
 // factor i of w = exp(2 pi i n' / (16 stride))).
-template <int LOG2N, bool XCH = true, int P = 0>
+template <int LOG2N, int XCH = XCHG_TMEM, int P = 0>
 __device__ __forceinline__ void tw_tmem_fill(const float2 *tw8, uint32_t base, int t) {
     using G = Geo<LOG2N>;
     if constexpr (P < G::NP - 1) {
@@ -751,10 +759,10 @@ __device__ __forceinline__ void forward_passes(float2 *x, float2 *bufs, const TW
         }
         constexpr bool tx = G::TX && tw_xchg<TW>();
         if constexpr (tx && P == G::NP - 2) {
-            tx_forward<LOG2N>(x, tw.xbase());
+            tx_forward<LOG2N, TW::xchg>(x, tw.xbase());
         } else {
             float2 *buf = bufs + (G::XBUFS == 2 ? (xc & 1) * G::PADN : 0);
-            if constexpr (tx && G::TX_RELABEL && P + 1 == G::NP - 2) exchange_tx<LOG2N, P, P + 1>(x, buf, t, bar);
+            if constexpr (tx && G::TX_RELABEL && P + 1 == G::NP - 2) exchange_tx<LOG2N, P, P + 1, TW::xchg>(x, buf, t, bar);
             else exchange<LOG2N, P, P + 1>(x, buf, t, bar);
             ++xc;
         }
@@ -783,10 +791,10 @@ __device__ __forceinline__ void inverse_passes(float2 *x, float2 *bufs, const TW
         constexpr bool late = tx && P == G::NP - 2;
         if constexpr (!late) tw.template fetch<LOG2N, P>(f, t);
         if constexpr (tx && P == G::NP - 2) {
-            tx_inverse<LOG2N>(x, tw.xbase());
+            tx_inverse<LOG2N, TW::xchg>(x, tw.xbase());
         } else {
             float2 *buf = bufs + (G::XBUFS == 2 ? (xc & 1) * G::PADN : 0);
-            if constexpr (tx && G::TX_RELABEL && P + 1 == G::NP - 2) exchange_tx<LOG2N, P + 1, P>(x, buf, t, bar);
+            if constexpr (tx && G::TX_RELABEL && P + 1 == G::NP - 2) exchange_tx<LOG2N, P + 1, P, TW::xchg>(x, buf, t, bar);
             else exchange<LOG2N, P + 1, P>(x, buf, t, bar);
             ++xc;
         }

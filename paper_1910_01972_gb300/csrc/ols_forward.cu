@@ -10,7 +10,7 @@ namespace ols {
 
 // y[f][j] written once, the aliased samples dropped.
 struct EpiPlain {
-    static constexpr bool XCH = true;
+    static constexpr int XCH = XCHG_TMEM;
     template <int LOG2N>
     static constexpr int edge() { return 0; }
     const float2 *sig;

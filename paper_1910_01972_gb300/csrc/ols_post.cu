@@ -86,7 +86,7 @@ __device__ __forceinline__ void append_candidates(bool hit, long long j, int f, 
 template <int MODE>
 struct EpiPost {
     // the TMEM exchange everywhere (a CTA's registers now hold it without spills)
-    static constexpr bool XCH = true;
+    static constexpr int XCH = MODE == POST_POWER ? XCHG_SHFL : XCHG_TMEM;
     // PEAK: warp-edge powers [2][T/32][16] floats per segment of several warps
     template <int LOG2N>
     static constexpr int edge() {
