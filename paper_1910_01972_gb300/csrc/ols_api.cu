@@ -641,8 +641,8 @@ int ols_host_stage_ms(ols_plan_t plan, double *ms) {
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 static void backward_layout(const ols_plan_s &p, int64_t nseg, bool want_ds, bool want_dh, size_t *edge_bytes,
-                            size_t *part_bytes, size_t *sum_bytes, int *grid) {
-    *grid = backward_grid(p, nseg, want_ds, want_dh);
+                            size_t *part_bytes, size_t *sum_bytes, int *grid, int *block) {
+    *grid = backward_grid(p, nseg, block);
     *edge_bytes = want_ds ? align256(sizeof(float2) * (size_t)nseg * 2 * (size_t)(p.M - 1)) : 0;
     const size_t spec = sizeof(float2) * (size_t)p.F * (size_t)p.N;
     *part_bytes = want_dh ? align256(spec * (size_t)(*grid)) : 0;
@@ -655,8 +655,8 @@ int ols_backward_workspace(ols_plan_t plan, int64_t Ns, int want_ds, int want_dh
     int rc = ols_geometry(plan->N, plan->M, Ns, &L, &nseg, &Nout);
     if (rc != OLS_OK) return rc;
     size_t eb, pb, rb;
-    int grid;
-    backward_layout(*plan, nseg, want_ds != 0, want_dh != 0, &eb, &pb, &rb, &grid);
+    int grid, block;
+    backward_layout(*plan, nseg, want_ds != 0, want_dh != 0, &eb, &pb, &rb, &grid, &block);
     *bytes = eb + pb + rb;
     return OLS_OK;
 }
@@ -693,7 +693,7 @@ int ols_convolve_backward(ols_plan_t plan, const float *s, int64_t Ns, const flo
     ols_geometry(plan->N, plan->M, Ns, &L, &nseg, &Nout);
     size_t eb, pb, rb;
     BackwardArgs a{};
-    backward_layout(*plan, nseg, ds != nullptr, dh != nullptr, &eb, &pb, &rb, &a.grid);
+    backward_layout(*plan, nseg, ds != nullptr, dh != nullptr, &eb, &pb, &rb, &a.grid, &a.block);
     if (eb + pb + rb > 0 && (!workspace || workspace_bytes < eb + pb + rb || ((uintptr_t)workspace & 255u)))
         return OLS_ERR_WORKSPACE;
     a.s = reinterpret_cast<const float2 *>(s);

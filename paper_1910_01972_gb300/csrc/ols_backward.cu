@@ -20,7 +20,7 @@
 // at the end gives dh.  Per window that is F + 2 FFTs (A, the F gradient
 // windows, one inverse for ds) instead of the 2F + 2 of a per-window dh.
 //
-// Kernel shape: a CTA of BwdGeo::BLOCK threads holds BwdGeo::SLOTS windows
+// Kernel shape: a CTA of BLOCK threads holds BwdGeo::SLOTS windows
 // (one per N/16-thread slot); a slot's FFT exchanges synchronise that slot
 // only (named barrier), and once per filter the slots' products B_f conj(A)
 // are summed in shared memory in slot order and added to the CTA's P_f in
@@ -36,20 +36,6 @@
 #include "ols_fft_passes.cuh"
 #include "ols_internal.h"
 #include "tmem.cuh"
-
-#ifndef OLS_BWD_BLOCK
-#define OLS_BWD_BLOCK 512        // threads per adjoint CTA (slots of N/16 threads), one CTA per SM ...
-#endif
-#ifndef OLS_BWD_BLOCK_1024
-#define OLS_BWD_BLOCK_1024 256   // ... except for N = 1024: two CTAs of 256 per SM (measured)
-#endif
-#ifndef OLS_BWD_MINB_1024
-#define OLS_BWD_MINB_1024 2
-#endif
-
-#ifndef OLS_BWD_XCHG
-#define OLS_BWD_XCHG 0
-#endif
 
 namespace ols {
 
@@ -98,28 +84,36 @@ __device__ __forceinline__ void st_keep(float4 *p, float4 v, const L2Hints &h) {
                  : "memory");
 }
 
+// Blocks of 512 threads, one per SM (two of 256 at N = 1024: 235 against 244
+// us for 16 filters of 2^22 samples), or of max(128, N/16) for short signals.
 template <int LOG2N>
+constexpr int bwd_block() { return LOG2N == 10 ? 256 : 512; }
+template <int LOG2N>
+constexpr int bwd_small_block() { return Geo<LOG2N>::T > 128 ? Geo<LOG2N>::T : 128; }
+
+template <int LOG2N, int BLOCK>
 struct BwdGeo {
     using G = Geo<LOG2N>;
-    static constexpr int TARGET = G::T == 64 ? OLS_BWD_BLOCK_1024 : OLS_BWD_BLOCK;
-    static constexpr int MINB = G::T == 64 ? OLS_BWD_MINB_1024 : 1;   // CTAs per SM for the register budget
-    static constexpr int SLOTS = TARGET / G::T > 1 ? TARGET / G::T : 1;
-    static constexpr int BLOCK = SLOTS * G::T;
-    static_assert(SLOTS <= 15 || G::T <= 32, "one named barrier per slot");
+    static constexpr int MINB = 512 / BLOCK;   // CTAs per SM for the register budget
+    static constexpr int SLOTS = BLOCK / G::T;
+    static_assert(SLOTS >= 1 && (SLOTS <= 15 || G::T <= 32), "one named barrier per slot");
     static constexpr int HALF = G::N / 2;      // float4 entries of one spectrum
-    static constexpr size_t SMEM = sizeof(float2) * (size_t)SLOTS * G::XBUFS * G::PADN;   // exchange buffers
+    static constexpr size_t USED = sizeof(float2) * (size_t)SLOTS * G::XBUFS * G::PADN;   // exchange buffers
+    // requested: enough that no more CTAs fit on an SM (228 KB) than tensor memory can serve
+    static constexpr size_t CLAIM = (228u * 1024u) / (MINB + 1) + 1024u;
+    static constexpr size_t SMEM = USED > CLAIM ? USED : CLAIM;
     static constexpr uint32_t TMEM_COLS = (uint32_t)(BLOCK / 128) * 128u;   // a 128-column lane range per 128 threads
     static_assert(G::XBUFS == 2, "the product buffer is the exchange buffer not in use");
 };
 
-template <int LOG2N, bool WANT_DS, bool WANT_DH>
-__global__ void __launch_bounds__(BwdGeo<LOG2N>::BLOCK, BwdGeo<LOG2N>::MINB)
+template <int LOG2N, int BLOCK, bool WANT_DS, bool WANT_DH>
+__global__ void __launch_bounds__(BLOCK, (BwdGeo<LOG2N, BLOCK>::MINB))
 ols_backward_kernel(const float2 *__restrict__ sig, long long Ns, const float2 *__restrict__ g,
                     long long Nout, const float4 *__restrict__ Htk, const float2 *__restrict__ twg,
                     float2 *__restrict__ ds, float2 *__restrict__ edge, float4 *__restrict__ P,
                     int M, int F, long long L, long long nseg, int *status) {
     using G = Geo<LOG2N>;
-    using BG = BwdGeo<LOG2N>;
+    using BG = BwdGeo<LOG2N, BLOCK>;
     extern __shared__ float4 smem_raw[];
     const int slot = threadIdx.x / G::T;
     const int t = threadIdx.x % G::T;
@@ -133,11 +127,8 @@ ols_backward_kernel(const float2 *__restrict__ sig, long long Ns, const float2 *
     tmem::fence_before_sync();
     __syncthreads();
     tmem::fence_after_sync();
-    // without the TMEM exchange: with it the N = 1024 adjoint takes 0.248 ms
-    // instead of 0.239 ms (72 bytes of spills), and the N = 2048 one spills more
-    constexpr bool xch = OLS_BWD_XCHG && LOG2N == 10;
-    const TwTmemT<xch> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
-    tw_tmem_fill<LOG2N, xch>(twg, tw.base, t);
+    const TwPlain tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
+    tw_plain_fill<LOG2N>(twg, tw.base, t);
     const uint32_t acol = tw.base + 96;
     const L2Hints l2 = L2Hints::make();
     const int lo = M - 1;
@@ -237,7 +228,7 @@ ols_backward_kernel(const float2 *__restrict__ sig, long long Ns, const float2 *
 #pragma unroll
                     for (int j2 = 0; j2 < 8; ++j2) prod[slot * SSTRIDE + j2 * G::T + t] = q[j2];
                     __syncthreads();
-                    for (int e = threadIdx.x; e < BG::HALF; e += BG::BLOCK) {
+                    for (int e = threadIdx.x; e < BG::HALF; e += BLOCK) {
                         float4 acc = prod[e];
 #pragma unroll
                         for (int s2 = 1; s2 < BG::SLOTS; ++s2) acc = f4add(acc, prod[s2 * SSTRIDE + e]);
@@ -372,25 +363,26 @@ ols_backward_dh_kernel(const float4 *__restrict__ Pr, const float2 *__restrict__
     }
 }
 
-template <int LOG2N, bool DS, bool DH>
-static cudaError_t prepare_bwd_one(ols_plan_s &p, int idx) {
-    using BG = BwdGeo<LOG2N>;
-    cudaError_t e = cudaFuncSetAttribute(ols_backward_kernel<LOG2N, DS, DH>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BG::SMEM);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = resident_blocks_tmem(ols_backward_kernel<LOG2N, DS, DH>, BG::BLOCK, BG::SMEM, (int)BG::TMEM_COLS, &per_sm);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    p.bwd_grid_cap[idx] = per_sm * p.sm_count;
-    return cudaSuccess;
+template <int LOG2N, int BLOCK>
+static cudaError_t prepare_bwd_block() {
+    const int smem = (int)BwdGeo<LOG2N, BLOCK>::SMEM;
+    cudaError_t e = cudaFuncSetAttribute(ols_backward_kernel<LOG2N, BLOCK, true, true>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(ols_backward_kernel<LOG2N, BLOCK, true, false>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(ols_backward_kernel<LOG2N, BLOCK, false, true>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    return e;
 }
 
 template <int LOG2N>
 static cudaError_t prepare_bwd_n(ols_plan_s &p) {
-    cudaError_t e = prepare_bwd_one<LOG2N, true, true>(p, 0);
-    if (e == cudaSuccess) e = prepare_bwd_one<LOG2N, true, false>(p, 1);
-    if (e == cudaSuccess) e = prepare_bwd_one<LOG2N, false, true>(p, 2);
+    cudaError_t e = prepare_bwd_block<LOG2N, bwd_block<LOG2N>()>();
+    if constexpr (bwd_small_block<LOG2N>() < bwd_block<LOG2N>()) {
+        if (e == cudaSuccess) e = prepare_bwd_block<LOG2N, bwd_small_block<LOG2N>()>();
+    }
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(ols_backward_dh_kernel<LOG2N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)Geo<LOG2N>::SMEM);
@@ -409,38 +401,49 @@ cudaError_t prepare_backward(ols_plan_s &p) {
     }
 }
 
-int backward_segs_per_block(int log2N) {
-    switch (log2N) {
-        case 8: return BwdGeo<8>::SLOTS;
-        case 9: return BwdGeo<9>::SLOTS;
-        case 10: return BwdGeo<10>::SLOTS;
-        case 11: return BwdGeo<11>::SLOTS;
-        case 12: return BwdGeo<12>::SLOTS;
-        case 13: return BwdGeo<13>::SLOTS;
-        default: return 1;
+// Small blocks while all of them are resident at once and their dh spectra
+// stay within 16 MB: a block runs its windows' F + 2 transforms in a row, so
+// more blocks of fewer windows finish sooner (F = 8: 45 windows of N = 512 in
+// 12 blocks instead of 3 43 -> 27 us, 37 of N = 1024 in 19 instead of 10 31 ->
+// 27 us).  The bound on the spectra keeps the whole workspace of such a call
+// below OLS_NOALLOC_SCRATCH_BYTES (16 MB of spectra, at most 8 MB for their
+// sum, at most 10 MB of edges, and not all at once), so the rule, which looks
+// neither at the gradients wanted nor at the entry point, makes no call too
+// large for the scratch that large blocks would have fitted.
+int backward_grid(const ols_plan_s &p, int64_t nseg, int *block) {
+    const int T = p.pp.T, large = p.log2N == 10 ? 256 : 512, small = T > 128 ? T : 128;
+    const int64_t gs = (nseg + small / T - 1) / (small / T), gl = (nseg + large / T - 1) / (large / T);
+    const int64_t spec = (int64_t)sizeof(float2) * p.F * p.N;
+    if (small < large && gs > gl && gs <= (int64_t)(512 / small) * p.sm_count && gs * spec <= (int64_t)16 << 20) {
+        *block = small;
+        return (int)gs;
     }
+    const int64_t cap = (int64_t)(512 / large) * p.sm_count;
+    *block = large;
+    return (int)(gl < cap ? gl : cap);
 }
 
-int backward_grid(const ols_plan_s &p, int64_t nseg, bool want_ds, bool want_dh) {
-    const int idx = want_ds ? (want_dh ? 0 : 1) : 2;
-    const int segs = backward_segs_per_block(p.log2N);
-    const int64_t nblk = (nseg + segs - 1) / segs;
-    return (int)(nblk < p.bwd_grid_cap[idx] ? nblk : p.bwd_grid_cap[idx]);
-}
-
-template <int LOG2N, bool DS, bool DH>
+template <int LOG2N, int BLOCK, bool DS, bool DH>
 static void launch_bwd_one(const ols_plan_s &p, const BackwardArgs &a, cudaStream_t st) {
-    using BG = BwdGeo<LOG2N>;
-    ols_backward_kernel<LOG2N, DS, DH><<<a.grid, BG::BLOCK, BG::SMEM, st>>>(
-        a.s, a.Ns, a.g, a.Nout, reinterpret_cast<const float4 *>(p.Htk), p.tw8, a.ds, a.edge, a.P, p.M, p.F, a.L,
+    using BG = BwdGeo<LOG2N, BLOCK>;
+    ols_backward_kernel<LOG2N, BLOCK, DS, DH><<<a.grid, BLOCK, BG::SMEM, st>>>(
+        a.s, a.Ns, a.g, a.Nout, reinterpret_cast<const float4 *>(p.Htk), p.tw, a.ds, a.edge, a.P, p.M, p.F, a.L,
         a.nseg, p.d_status);
+}
+
+template <int LOG2N, int BLOCK>
+static void launch_bwd_block(const ols_plan_s &p, const BackwardArgs &a, cudaStream_t st) {
+    if (a.ds && a.dh) launch_bwd_one<LOG2N, BLOCK, true, true>(p, a, st);
+    else if (a.ds) launch_bwd_one<LOG2N, BLOCK, true, false>(p, a, st);
+    else launch_bwd_one<LOG2N, BLOCK, false, true>(p, a, st);
 }
 
 template <int LOG2N>
 static void launch_bwd_n(const ols_plan_s &p, const BackwardArgs &a, cudaStream_t st) {
-    if (a.ds && a.dh) launch_bwd_one<LOG2N, true, true>(p, a, st);
-    else if (a.ds) launch_bwd_one<LOG2N, true, false>(p, a, st);
-    else launch_bwd_one<LOG2N, false, true>(p, a, st);
+    if constexpr (bwd_small_block<LOG2N>() < bwd_block<LOG2N>()) {
+        if (a.block == bwd_small_block<LOG2N>()) return launch_bwd_block<LOG2N, bwd_small_block<LOG2N>()>(p, a, st);
+    }
+    launch_bwd_block<LOG2N, bwd_block<LOG2N>()>(p, a, st);
 }
 
 template <int LOG2N>

@@ -701,6 +701,51 @@ struct TwTmemT {
     }
 };
 
+// TwPlain: the thread's 15 twiddles of every pass in its TMEM lane (pass P at
+// columns 32 P .. 32 P + 29), applied by complex multiplies around a plain
+// DFT.  The adjoint's form: it transforms forward, where folding saves nothing
+// (a butterfly of (a - b) W is no multiply-add; folded 239 / 209 us for both
+// gradients / dh alone at N = 1024, plain 235 / 195; decimation in time with
+// folded butterflies 235 / 206, and it spills at N = 4096: 320 against 305).
+struct TwPlain {
+    uint32_t base;
+    struct Fetched {
+        float v[32];
+    };
+    template <int LOG2N, int P>
+    __device__ __forceinline__ void fetch(Fetched &f, int) const {
+        tmem::ld32(base + 32 * P, f.v);
+    }
+    template <bool INV>
+    __device__ __forceinline__ void apply(float2 *x, const Fetched &f) const {
+        tmem::wait_ld();
+#pragma unroll
+        for (int k = 1; k < 16; ++k) x[k] = ctw<INV>(x[k], make_float2(f.v[2 * k - 2], f.v[2 * k - 1]));
+    }
+};
+
+// Fill a TwPlain for thread t from the plan's twiddle table.
+template <int LOG2N, int P = 0>
+__device__ __forceinline__ void tw_plain_fill(const float2 *tw, uint32_t base, int t) {
+    using G = Geo<LOG2N>;
+    if constexpr (P < G::NP - 1) {
+        constexpr int s = G::stride(P);
+        const float2 *w = tw + G::tw_off(P) + t % s;
+        float v[32];
+#pragma unroll
+        for (int k = 1; k < 16; ++k) {
+            const float2 wk = __ldg(w + (k - 1) * s);
+            v[2 * k - 2] = wk.x;
+            v[2 * k - 1] = wk.y;
+        }
+        v[30] = v[31] = 0.f;
+        tmem::st32(base + 32 * P, v);
+        tw_plain_fill<LOG2N, P + 1>(tw, base, t);
+    } else {
+        tmem::wait_st();
+    }
+}
+
 using TwTmem = TwTmemT<true>;
 template <class TW>
 struct is_tw_tmem : std::false_type {};

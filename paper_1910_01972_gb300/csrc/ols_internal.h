@@ -129,7 +129,6 @@ struct ols_plan_s {
     const float2 *tw8 = nullptr; // folded twiddles of the TMEM-twiddle kernels: tw + pp.twn (pp.tw8n entries)
     double2 *tw64 = nullptr;     // W_N^m, m in [0, N) (FP64)
     int32_t *nu = nullptr;       // spectral order (device copy)
-    int bwd_grid_cap[3] = {0, 0, 0};  // backward kernel: (ds,dh), (ds), (dh)
     int last_launches = 0;
     int tc_grid_cap = 0;         // resident blocks of the tensor-core kernel
     int tc_split_grid_cap = 0;   // the same for its pre-split-input form
@@ -152,7 +151,7 @@ struct BackwardArgs {
     float2 *ds, *dh;
     float2 *edge;             // workspace: ds overlap edges (nseg x 2 x (M-1))
     float4 *P, *Pr;           // workspace: per-CTA dh spectra (grid x F x N/2), their sum (F x N/2)
-    int grid;
+    int grid, block;
 };
 
 // One problem of a batch, as the batched kernel reads it.
@@ -240,8 +239,8 @@ int backward_validate(ols_plan_t plan, const float *s, int64_t Ns, const float *
 // kernel; `launches` receives the number of kernels enqueued.
 cudaError_t prepare_backward(ols_plan_s &p);
 cudaError_t launch_backward(const ols_plan_s &p, const BackwardArgs &a, cudaStream_t st, int *launches);
-int backward_grid(const ols_plan_s &p, int64_t nseg, bool want_ds, bool want_dh);
-int backward_segs_per_block(int log2N);
+// Block size and grid of the adjoints window kernel for nseg windows.
+int backward_grid(const ols_plan_s &p, int64_t nseg, int *block);
 // FP64 precompute kernels.  Htk (may be null): the spectra of conj(h_f[M-1-k]).
 cudaError_t launch_tw64(double2 *tw64, int N, cudaStream_t st);
 // Spectra in the 16-points-per-thread register layout of the kernels.

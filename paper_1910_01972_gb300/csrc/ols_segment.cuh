@@ -90,7 +90,7 @@ __device__ __forceinline__ void ols_segment(const float2 *__restrict__ sig, long
         for (int k = 0; k < 16; ++k) {
             const int n = k * G::T + t;
             if ((unsigned)(n - lo) < (unsigned)span && in_bounds(obase + n >= 0 && obase + n < Nout, status))
-                dst[obase + n] = x[k];
+                __stcs(dst + obase + n, x[k]);
         }
     }
 }
