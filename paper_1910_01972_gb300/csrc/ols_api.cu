@@ -105,6 +105,44 @@ static std::vector<uint16_t> tc_dft16_tables(bool bf16) {
     return out;
 }
 
+// Tables of ols_tc64.cu: the inverse DFT-64 as the real 128 x 128 matrix [[C, S],
+// [-S, C]] (rows: Re, Im of the input; columns: Re, Im of the output), split in
+// 16-bit hi and lo parts (element (k, n) at byte (k/8) 2048 + (n/8) 128 + (n%8) 16
+// + (k%8) 2), then the twiddles e(n2 nu1 / 4096) / 8 as float2, points (n2 = 16 q +
+// 2 i, + 1) of row nu1 at float4 index i 256 + 64 q + nu1.
+static std::vector<uint16_t> tc64_tables(bool bf16) {
+    std::vector<uint16_t> out(2 * 128 * 128 + 4096 * 4);
+    for (int k = 0; k < 128; ++k)
+        for (int n = 0; n < 128; ++n) {
+            const double th = 2.0 * M_PI * (double)(((k % 64) * (n % 64)) % 64) / 64.0;
+            const double cs = std::cos(th), sn = std::sin(th);
+            const double v = (k < 64) == (n < 64) ? cs : (k < 64 ? sn : -sn);
+            uint16_t hi, lo;
+            if (bf16) {
+                const __nv_bfloat16 h = __double2bfloat16(v);
+                const __nv_bfloat16 l = __double2bfloat16(v - (double)__bfloat162float(h));
+                hi = *reinterpret_cast<const uint16_t *>(&h);
+                lo = *reinterpret_cast<const uint16_t *>(&l);
+            } else {
+                const __half h = __double2half(v);
+                const __half l = __double2half(v - (double)__half2float(h));
+                hi = *reinterpret_cast<const uint16_t *>(&h);
+                lo = *reinterpret_cast<const uint16_t *>(&l);
+            }
+            const int e = ((k / 8) * 2048 + (n / 8) * 128 + (n % 8) * 16 + (k % 8) * 2) / 2;
+            out[e] = hi;
+            out[128 * 128 + e] = lo;
+        }
+    for (int n2 = 0; n2 < 64; ++n2)
+        for (int nu1 = 0; nu1 < 64; ++nu1) {
+            const double th = 2.0 * M_PI * (double)(n2 * nu1) / 4096.0;
+            const float w[2] = {(float)(std::cos(th) / 8.0), (float)(std::sin(th) / 8.0)};
+            const int q = n2 / 16, i = (n2 % 16) / 2;
+            std::memcpy(&out[2 * 128 * 128 + ((i * 256 + 64 * q + nu1) * 4 + 2 * (n2 & 1)) * 2], w, sizeof(w));
+        }
+    return out;
+}
+
 static thread_local int t_alloc_depth = 0;
 static thread_local int t_alloc_seq = 0;
 
@@ -287,10 +325,12 @@ int ols_plan(ols_plan_t *out, int64_t N, int32_t M, int32_t F, uint32_t flags) {
     }
     if (const char *wn = std::getenv("OLS_TC_WAIT_NEVER")) p->tc_wait_never = wn[0] == '1';
     if (e == cudaSuccess && flags != OLS_FLAG_FP32 && flags != OLS_FLAG_R2R) {
-        const std::vector<uint16_t> b = tc_dft16_tables(flags == OLS_FLAG_TC_BF16SPLIT);
+        const bool bf16 = flags == OLS_FLAG_TC_BF16SPLIT;
+        p->rows64 = l == 12;
+        const std::vector<uint16_t> b = p->rows64 ? tc64_tables(bf16) : tc_dft16_tables(bf16);
         e = dev_alloc(&p->tc_bmat, sizeof(uint16_t) * b.size());
         if (e == cudaSuccess) e = cudaMemcpy(p->tc_bmat, b.data(), sizeof(uint16_t) * b.size(), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = tc_prepare(*p, flags == OLS_FLAG_TC_BF16SPLIT);
+        if (e == cudaSuccess) e = tc_prepare(*p, bf16);
     }
     if (e == cudaSuccess) {
         std::vector<float2> tw = twiddle_tables(p->pp);
@@ -298,6 +338,8 @@ int ols_plan(ols_plan_t *out, int64_t N, int32_t M, int32_t F, uint32_t flags) {
         p->dsin = reinterpret_cast<const float *>(p->tw8 + p->pp.tw8n);
         std::vector<int32_t> nu((size_t)N);
         spectral_order(l, nu.data());
+        if (p->rows64)
+            for (int q = 0; q < 4096; ++q) nu[(size_t)q] = ((q >> 4) & 63) + 64 * (16 * (q >> 10) + (q & 15));
         for (int64_t q = 0; q < N; q += 2)
             tw.push_back(make_float2((float)std::sin(2.0 * M_PI * (double)nu[q] / (double)N),
                                      (float)std::sin(2.0 * M_PI * (double)nu[q + 1] / (double)N)));
@@ -344,7 +386,7 @@ int ols_set_filters(ols_plan_t plan, const float *h, void *stream) {
     if (plan->flags == OLS_FLAG_R2R) return OLS_ERR_UNSUPPORTED;
     const float2 *hh = reinterpret_cast<const float2 *>(h);
     cudaError_t e = launch_spectra(hh, plan->M, plan->F, plan->log2N, plan->nu, plan->tw64, plan->Hk, plan->Htk,
-                                   (cudaStream_t)stream);
+                                   plan->rows64, (cudaStream_t)stream);
     if (e != cudaSuccess) return status_of(e);
     plan->filters_ready = true;
     return OLS_OK;
@@ -405,7 +447,7 @@ int ols_set_filters_real(ols_plan_t plan, const float *h, void *stream) {
     cudaError_t e = launch_pack_real_pairs(h, plan->M, plan->F, plan->hpack, (cudaStream_t)stream);
     if (e == cudaSuccess)
         e = launch_spectra(plan->hpack, plan->M, Fc, plan->log2N, plan->nu, plan->tw64, plan->Hk, nullptr,
-                           (cudaStream_t)stream);
+                           false, (cudaStream_t)stream);
     if (e != cudaSuccess) return status_of(e);
     plan->filters_ready = true;
     return OLS_OK;

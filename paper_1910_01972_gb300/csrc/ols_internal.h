@@ -137,6 +137,8 @@ struct ols_plan_s {
     // real-to-real plans (OLS_FLAG_R2R)
     float2 *hpack = nullptr;     // [ceil(F/2)][M] paired real filters h_{2p} + i h_{2p+1}
     uint16_t *tc_bmat = nullptr; // split DFT-16 matrices (fwd hi, fwd lo, inv hi, inv lo), core-matrix layout
+                                 // (N = 4096: split DFT-64 matrix and twiddles, see tc64_tables)
+    bool rows64 = false;         // spectra in the order of ols_tc64.cu
     int *d_status = nullptr;     // device status word (bounded-wait failures)
     ols::Staging stage;
 };
@@ -220,6 +222,10 @@ struct TcSignal {
 cudaError_t tc_prepare(ols_plan_s &p, bool bf16);
 cudaError_t tc_launch(const ols_plan_s &p, const TcSignal &sg, int64_t Ns, float2 *y, int64_t L, int64_t nseg,
                       int64_t Nout, cudaStream_t st);
+// ... at N = 4096 (ols_tc64.cu)
+cudaError_t tc64_prepare(bool bf16);
+cudaError_t tc64_launch(const ols_plan_s &p, const TcSignal &sg, int64_t Ns, float2 *y, int64_t L, int64_t nseg,
+                        int64_t Nout, cudaStream_t st);
 cudaError_t launch_split_signal(const float2 *s, int64_t Ns, bool bf16, uint32_t *hi, uint32_t *lo, int sm_count,
                                 cudaStream_t st);
 
@@ -245,7 +251,7 @@ int backward_grid(const ols_plan_s &p, int64_t nseg, int *block);
 cudaError_t launch_tw64(double2 *tw64, int N, cudaStream_t st);
 // Spectra in the 16-points-per-thread register layout of the kernels.
 cudaError_t launch_spectra(const float2 *h, int M, int F, int log2N, const int32_t *nu,
-                           const double2 *tw64, float2 *Hk, float2 *Htk, cudaStream_t st);
+                           const double2 *tw64, float2 *Hk, float2 *Htk, bool rows64, cudaStream_t st);
 cudaError_t launch_spectra_natural(const float2 *Hk, int F, int log2N, const int32_t *nu,
                                    float2 *H, cudaStream_t st);
 

@@ -39,7 +39,8 @@ __global__ void tw64_kernel(double2 *tw64, int N) {
 // after: F = 8, M = 65, N = 512 62 -> 9 us; 16, 129, 1024 116 -> 9; 32, 257, 2048
 // 435 -> 13; 64, 512, 4096 2962 -> 33; 24, 1025, 8192 5098 -> 31 us.
 __global__ void spectra_kernel(const float2 *__restrict__ h, int M, int log2N, const int32_t *__restrict__ nu_tab,
-                               const double2 *__restrict__ tw64, float2 *__restrict__ Hk, float2 *__restrict__ Htk) {
+                               const double2 *__restrict__ tw64, float2 *__restrict__ Hk, float2 *__restrict__ Htk,
+                               bool rows64) {
     extern __shared__ double2 smem64[];
     const int N = 1 << log2N, P = N / 16, lp = log2N - 4, TR = P / 2;
     const int grp = threadIdx.x / TR, i = threadIdx.x % TR;      // residue group of the block, its butterfly
@@ -77,10 +78,17 @@ __global__ void spectra_kernel(const float2 *__restrict__ h, int M, int log2N, c
     const int T = N / 16;
     for (int e = i; e < P; e += TR) {                            // e: (j, t) with t fastest
         const int tl = e & (P / 16 - 1), j = e / (P / 16);
-        const int t = r * (P / 16) + tl, q = 16 * t + j;
-        const int nu = nu_tab[q], k = nu >> 4;
+        int t = r * (P / 16) + tl, jj = j, nu;
+        if (rows64) {                                            // ols_tc64.cu: nu = nu1 + 64 (16 c + j), t = 64 c + nu1
+            nu = r + 16 * e;
+            t = ((nu >> 10) << 6) + (nu & 63);
+            jj = (nu >> 6) & 15;
+        } else {
+            nu = nu_tab[16 * t + j];
+        }
+        const int k = nu >> 4;
         const double2 v = u[__brev((unsigned)k) >> (32 - lp)];
-        const size_t idx = (size_t)f * N + (size_t)(j >> 1) * (2 * T) + 2 * t + (j & 1);
+        const size_t idx = (size_t)f * N + (size_t)(jj >> 1) * (2 * T) + 2 * t + (jj & 1);
         Hk[idx] = make_float2((float)(v.x * inv), (float)(v.y * inv));
         if (Htk) {
             const double2 w = tw64[((long long)nu * (M - 1)) & (N - 1)];
@@ -109,13 +117,13 @@ cudaError_t launch_tw64(double2 *tw64, int N, cudaStream_t st) {
 }
 
 cudaError_t launch_spectra(const float2 *h, int M, int F, int log2N, const int32_t *nu,
-                           const double2 *tw64, float2 *Hk, float2 *Htk, cudaStream_t st) {
+                           const double2 *tw64, float2 *Hk, float2 *Htk, bool rows64, cudaStream_t st) {
     const int P = (1 << log2N) / 16, block = P / 2 > 32 ? P / 2 : 32;
     const int per_block = block / (P / 2);
     const long long grid = (long long)F * (16 / per_block);
     if (grid > 0x7fffffffll) return cudaErrorInvalidValue;
     spectra_kernel<<<(unsigned)grid, block, sizeof(double2) * (size_t)(P * per_block), st>>>(h, M, log2N, nu, tw64, Hk,
-                                                                                            Htk);
+                                                                                            Htk, rows64);
     return cudaGetLastError();
 }
 

@@ -44,6 +44,7 @@
 
 #include "ols_internal.h"
 #include "ols_fft_passes.cuh"
+#include "ols_tc_split.cuh"
 
 namespace ols {
 
@@ -51,27 +52,7 @@ namespace tc {
 
 constexpr int kCols = 128;           // TMEM columns per 128-row tile: two groups of A_hi 16, A_lo 16, D 32
 constexpr int kBytesB = 32 * 32 * 2; // one 32x32 16-bit matrix
-constexpr long long kWaitLimit = 1ll << 20;   // polls; also the drain limit before tcgen05.dealloc
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// 16-bit split of an FP32 pair into packed hi and lo words.
-template <bool BF16>
-__device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t &lo) {
-    if constexpr (BF16) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-        const float2 hf = __bfloat1622float2(h);
-        const __nv_bfloat162 l = __floats2bfloat162_rn(a - hf.x, b - hf.y);
-        hi = *reinterpret_cast<const uint32_t *>(&h);
-        lo = *reinterpret_cast<const uint32_t *>(&l);
-    } else {
-        const __half2 h = __floats2half2_rn(a, b);
-        const float2 hf = __half22float2(h);
-        const __half2 l = __floats2half2_rn(a - hf.x, b - hf.y);
-        hi = *reinterpret_cast<const uint32_t *>(&h);
-        lo = *reinterpret_cast<const uint32_t *>(&l);
-    }
-}
 
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t *v) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
@@ -183,18 +164,6 @@ __device__ __forceinline__ void issue(Ctx &c, int g) {
                      : "memory");
         c.pending[g] = true;
     }
-}
-
-// Bounded poll of mbarrier `bar` for parity `phase`; true once it completed.
-__device__ __forceinline__ bool poll(uint32_t bar, uint32_t phase, long long limit) {
-    uint32_t done = 0;
-    for (long long it = 0; it < limit && !done; ++it) {
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(done)
-                     : "r"(bar), "r"(phase)
-                     : "memory");
-    }
-    return done != 0;
 }
 
 // Wait (bounded) for group g's MMAs and read this thread's row of D into x.
@@ -488,7 +457,7 @@ cudaError_t tc_prepare(ols_plan_s &p, bool bf16) {
         case 9: return bf16 ? tc_prepare_one<9, true>(p) : tc_prepare_one<9, false>(p);
         case 10: return bf16 ? tc_prepare_one<10, true>(p) : tc_prepare_one<10, false>(p);
         case 11: return bf16 ? tc_prepare_one<11, true>(p) : tc_prepare_one<11, false>(p);
-        case 12: return bf16 ? tc_prepare_one<12, true>(p) : tc_prepare_one<12, false>(p);
+        case 12: return tc64_prepare(bf16);
         case 13: return bf16 ? tc_prepare_one<13, true>(p) : tc_prepare_one<13, false>(p);
         default: return cudaErrorInvalidValue;
     }
@@ -525,7 +494,7 @@ cudaError_t tc_launch(const ols_plan_s &p, const TcSignal &sg, int64_t Ns, float
         case 9: return tc_launch_n<9>(p, sg, Ns, y, L, nseg, Nout, st);
         case 10: return tc_launch_n<10>(p, sg, Ns, y, L, nseg, Nout, st);
         case 11: return tc_launch_n<11>(p, sg, Ns, y, L, nseg, Nout, st);
-        case 12: return tc_launch_n<12>(p, sg, Ns, y, L, nseg, Nout, st);
+        case 12: return tc64_launch(p, sg, Ns, y, L, nseg, Nout, st);
         case 13: return tc_launch_n<13>(p, sg, Ns, y, L, nseg, Nout, st);
         default: return cudaErrorInvalidValue;
     }

@@ -1,0 +1,44 @@
+"""The N = 4096 tensor-core form (two radix-64 stages) where its schedule and
+layout can go wrong: one filter, an odd number of segments (an idle half tile),
+shares that begin inside a segment pair's filters, the shortest signal, every
+output position of one segment; against the FP64 oracle.  Bounds as in
+test_tc_gpu: 2e-6 (FP16), 3e-5 (BF16)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+from paper_1910_01972_gb300 import Plan, _native
+from paper_1910_01972_gb300 import build as _build
+
+pytestmark = pytest.mark.gpu
+BOUND = {_native.OLS_FLAG_TC_FP16SPLIT: 2e-6, _native.OLS_FLAG_TC_BF16SPLIT: 3e-5}
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+@pytest.mark.parametrize("flag", list(BOUND))
+@pytest.mark.parametrize("M,F,Ns", [(512, 1, 512), (512, 1, 4096), (100, 2, 4097), (1, 3, 4096), (513, 1, 60_000),
+                                    (513, 61, 11_000), (4096, 3, 4100), (257, 200, 8_000)])
+def test_parity(flag, M, F, Ns):
+    _build.build()
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    g = np.random.Generator(np.random.PCG64(M + F + flag))
+    s, h = synth.signal(g, Ns), synth.filters(g, F, M)
+    p = Plan(M, F, 4096, flags=flag)
+    p.set_filters(dev(h))
+    y = p.convolve(dev(s))
+    assert p.status() == 0
+    ref = oracle.conv(s, h)
+    assert oracle.max_stream_rel_l2(y.cpu().numpy(), ref, oracle.stream_scale(s, h, ref.shape[1])) <= BOUND[flag]
+    # the spectra read back in natural order, and the stored-split input bit for bit
+    H = p.spectra().cpu().numpy()
+    Href = np.fft.fft(h.astype(np.complex128), 4096, axis=1) / 4096
+    assert np.max(np.abs(H - Href)) <= 6e-8 * np.max(np.abs(Href))
+    hi, lo = p.split_signal(dev(s))
+    assert torch.equal(p.convolve_split(hi, lo), y)
+    p.close()
