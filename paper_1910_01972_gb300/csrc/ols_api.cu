@@ -53,19 +53,26 @@ static std::vector<float2> twiddle_tables(const PassPlan &pp) {
                     make_float2((float)std::cos(a), (float)std::sin(a));
             }
     }
+    // N = 8192 runs as two 4096-point transforms (and one twiddle, below)
+    const PassPlan fp = pp.log2N == 13 ? make_pass_plan(12) : pp;
     // folded factors (inverse sign): w^8; w^4; w^2, w^2 e(2); w, w e(1), w e(2),
     // w e(3) with w = exp(2 pi i n' / (16 s)), e(m) = exp(2 pi i m / 16); row i
     // of pass p at tw8_off[p] + i s + n'
     static const int kPow[8] = {8, 4, 2, 2, 1, 1, 1, 1}, kRot[8] = {0, 0, 0, 2, 0, 1, 2, 3};
-    for (int p = 0; p + 1 < pp.np; ++p) {
-        const int s = pp.stride[p], B = 16 * s;
+    for (int p = 0; p + 1 < fp.np; ++p) {
+        const int s = fp.stride[p], B = 16 * s;
         for (int i = 0; i < 8; ++i)
             for (int n = 0; n < s; ++n) {
                 const double a = 2.0 * M_PI * (double)(kPow[i] * n + kRot[i] * s) / (double)B;
-                tw[(size_t)pp.twn + (size_t)pp.tw8_off[p] + (size_t)i * s + n] =
+                tw[(size_t)pp.twn + (size_t)fp.tw8_off[p] + (size_t)i * s + n] =
                     make_float2((float)std::cos(a), (float)std::sin(a));
             }
     }
+    if (pp.log2N == 13)
+        for (int t = 0; t < 256; ++t) {
+            const double a = 2.0 * M_PI * (double)t / 8192.0;
+            tw[(size_t)(pp.twn + fp.tw8n + t)] = make_float2((float)std::cos(a), (float)std::sin(a));
+        }
     return tw;
 }
 
@@ -304,6 +311,7 @@ int ols_plan(ols_plan_t *out, int64_t N, int32_t M, int32_t F, uint32_t flags) {
     cudaError_t e = cudaGetDevice(&p->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, p->device);
     const bool r2r = flags == OLS_FLAG_R2R;
+    if (l == 13 && (r2r || flags == OLS_FLAG_FP32)) p->layout = LAYOUT_HALVES;
     const int32_t Fc = r2r ? (F + 1) / 2 : F;       // complex spectra held: paired filters for R2R
     if (e == cudaSuccess) e = dev_alloc(&p->Hk, sizeof(float2) * (size_t)Fc * (size_t)N);
     if (e == cudaSuccess && !r2r) e = dev_alloc(&p->Htk, sizeof(float2) * (size_t)F * (size_t)N);
@@ -326,8 +334,8 @@ int ols_plan(ols_plan_t *out, int64_t N, int32_t M, int32_t F, uint32_t flags) {
     if (const char *wn = std::getenv("OLS_TC_WAIT_NEVER")) p->tc_wait_never = wn[0] == '1';
     if (e == cudaSuccess && flags != OLS_FLAG_FP32 && flags != OLS_FLAG_R2R) {
         const bool bf16 = flags == OLS_FLAG_TC_BF16SPLIT;
-        p->rows64 = l == 12;
-        const std::vector<uint16_t> b = p->rows64 ? tc64_tables(bf16) : tc_dft16_tables(bf16);
+        if (l == 12) p->layout = LAYOUT_ROWS64;
+        const std::vector<uint16_t> b = l == 12 ? tc64_tables(bf16) : tc_dft16_tables(bf16);
         e = dev_alloc(&p->tc_bmat, sizeof(uint16_t) * b.size());
         if (e == cudaSuccess) e = cudaMemcpy(p->tc_bmat, b.data(), sizeof(uint16_t) * b.size(), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = tc_prepare(*p, bf16);
@@ -338,11 +346,11 @@ int ols_plan(ols_plan_t *out, int64_t N, int32_t M, int32_t F, uint32_t flags) {
         p->dsin = reinterpret_cast<const float *>(p->tw8 + p->pp.tw8n);
         std::vector<int32_t> nu((size_t)N);
         spectral_order(l, nu.data());
-        if (p->rows64)
-            for (int q = 0; q < 4096; ++q) nu[(size_t)q] = ((q >> 4) & 63) + 64 * (16 * (q >> 10) + (q & 15));
-        for (int64_t q = 0; q < N; q += 2)
-            tw.push_back(make_float2((float)std::sin(2.0 * M_PI * (double)nu[q] / (double)N),
-                                     (float)std::sin(2.0 * M_PI * (double)nu[q + 1] / (double)N)));
+        auto dsin = [&](int64_t q) {
+            const int f = p->layout == LAYOUT_STD ? nu[(size_t)q] : layout_freq(p->layout, (int)q);
+            return (float)std::sin(2.0 * M_PI * (double)f / (double)N);
+        };
+        for (int64_t q = 0; q < N; q += 2) tw.push_back(make_float2(dsin(q), dsin(q + 1)));
         e = cudaMemcpy(p->tw, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(p->nu, nu.data(), sizeof(int32_t) * nu.size(), cudaMemcpyHostToDevice);
     }
@@ -386,7 +394,7 @@ int ols_set_filters(ols_plan_t plan, const float *h, void *stream) {
     if (plan->flags == OLS_FLAG_R2R) return OLS_ERR_UNSUPPORTED;
     const float2 *hh = reinterpret_cast<const float2 *>(h);
     cudaError_t e = launch_spectra(hh, plan->M, plan->F, plan->log2N, plan->nu, plan->tw64, plan->Hk, plan->Htk,
-                                   plan->rows64, (cudaStream_t)stream);
+                                   plan->layout, (cudaStream_t)stream);
     if (e != cudaSuccess) return status_of(e);
     plan->filters_ready = true;
     return OLS_OK;
@@ -397,7 +405,7 @@ int ols_get_spectra(ols_plan_t plan, float *H, void *stream) {
     if (!plan->filters_ready) return OLS_ERR_NOT_READY;
     const int Fc = plan->flags == OLS_FLAG_R2R ? (plan->F + 1) / 2 : plan->F;
     return status_of(launch_spectra_natural(plan->Hk, Fc, plan->log2N, plan->nu,
-                                            reinterpret_cast<float2 *>(H), (cudaStream_t)stream));
+                                            reinterpret_cast<float2 *>(H), plan->layout, (cudaStream_t)stream));
 }
 
 int ols_convolve(ols_plan_t plan, const float *s, int64_t Ns, float *y, void *stream) {
@@ -447,7 +455,7 @@ int ols_set_filters_real(ols_plan_t plan, const float *h, void *stream) {
     cudaError_t e = launch_pack_real_pairs(h, plan->M, plan->F, plan->hpack, (cudaStream_t)stream);
     if (e == cudaSuccess)
         e = launch_spectra(plan->hpack, plan->M, Fc, plan->log2N, plan->nu, plan->tw64, plan->Hk, nullptr,
-                           false, (cudaStream_t)stream);
+                           plan->layout, (cudaStream_t)stream);
     if (e != cudaSuccess) return status_of(e);
     plan->filters_ready = true;
     return OLS_OK;

@@ -93,7 +93,7 @@ ols_bank_kernel(const BankArgs a, const EPI epi) {
     tmem::fence_before_sync();
     __syncthreads();
     tmem::fence_after_sync();
-    const TwTmemT<EPI::XCH> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
+    const TwTmemT<EPI::XCH> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(a.tw8, t)};
     tw_tmem_fill<LOG2N, EPI::XCH>(a.tw8, tw.base, t);
     const uint32_t xcol = tw.base + 96;
 
@@ -123,7 +123,7 @@ ols_bank_kernel(const BankArgs a, const EPI epi) {
         sg.Nout = a.Nout;
         sg.status = a.status;
         {
-            // samples start + k T + t inside [0, Ns), zero elsewhere
+            // samples start + base(t) + off(k) inside [0, Ns), zero elsewhere
             float2 X[16];
             const long long start = sg.j0 + a.off;
             const long long avail = active ? a.Ns - start : 0;
@@ -131,7 +131,7 @@ ols_bank_kernel(const BankArgs a, const EPI epi) {
             const int first = start < 0 ? (int)-start : 0;
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
-                const int n = k * G::T + t;
+                const int n = G::base(t) + G::off(k);
                 X[k] = (n >= first && n < lim && in_bounds(start + n >= 0 && start + n < a.Ns, a.status))
                            ? epi.sample(start + n)
                            : make_float2(0.f, 0.f);

@@ -50,8 +50,8 @@ ols_batched_kernel(const BatchProblemDev *__restrict__ probs, const int2 *__rest
     __syncthreads();
     tmem::fence_after_sync();
     // the TMEM exchange at the segment lengths of OLS_BATCH_PERN_TX_MASK
-    constexpr bool xch = in_tx_mask<LOG2N>(OLS_BATCH_PERN_TX_MASK);
-    const TwTmemT<xch> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
+    constexpr int xch = (LOG2N == 13 || in_tx_mask<LOG2N>(OLS_BATCH_PERN_TX_MASK)) ? XCHG_TMEM : XCHG_SMEM;
+    const TwTmemT<xch> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(twg, t)};
     tw_tmem_fill<LOG2N, xch>(twg, tw.base, t);
     int xc = 0;
     for (;;) {
@@ -153,9 +153,9 @@ __device__ __forceinline__ void batch_one_tile(const BatchProblemDev &P, int til
         // segment spectrum), so results stay bitwise those of per-problem calls
         // (the TMEM exchange at the segment lengths of OLS_BATCH_TX_MASK); the
         // twiddles are written on an item's first tile only
-        constexpr bool xch = in_tx_mask<LOG2N>(OLS_BATCH_TX_MASK);
+        constexpr int xch = (LOG2N == 13 || in_tx_mask<LOG2N>(OLS_BATCH_TX_MASK)) ? XCHG_TMEM : XCHG_SMEM;
         using TWT = TwTmemT<xch>;
-        const TWT twt{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
+        const TWT twt{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(tw, t)};
         if (fill) tw_tmem_fill<LOG2N, xch>(tw, twt.base, t);
         ols_segment<LOG2N, TWT, SegmentBarrier<G::T>>(s_ptrs[P.index], P.Ns, P.Hk, twt, y_ptrs[P.index],
                                                                P.M, P.F, P.L, P.Nout, seg, seg < P.nseg, bufs, t, xc,

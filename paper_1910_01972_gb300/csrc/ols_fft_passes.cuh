@@ -87,6 +87,12 @@ struct Geo {
         return o;
     }
     static constexpr int TWN = tw_off(NP - 1);
+    // sample n of the segment that register k of thread t holds in the time
+    // domain: base(t) + off(k) (N = 8192: see halves13 below)
+    __host__ __device__ static constexpr int base(int t) { return LOG2N == 13 ? 2048 * (t >> 8) + (t & 255) : t; }
+    __host__ __device__ static constexpr int off(int k) {
+        return LOG2N == 13 ? 256 * (k & 7) + 4096 * (k >> 3) : k * T;
+    }
     // folded-twiddle table (TMEM twiddles): 8 rows of stride(p) entries per pass
     __host__ __device__ static constexpr int tw8_off(int p) {
         int o = 0;
@@ -665,6 +671,7 @@ template <int XCH = XCHG_TMEM>
 struct TwTmemT {
     static constexpr int xchg = XCH;
     uint32_t base;
+    float2 odd = {0.f, 0.f};         // N = 8192: exp(2 pi i (t mod 256) / 8192)
     // columns 64..95: the staging area of the TMEM exchange
     __device__ __forceinline__ uint32_t xbase() const { return base + 64; }
     struct Fetched {
@@ -763,7 +770,9 @@ __device__ __forceinline__ constexpr bool tw_xchg() {
 template <int LOG2N, int XCH = XCHG_TMEM, int P = 0>
 __device__ __forceinline__ void tw_tmem_fill(const float2 *tw8, uint32_t base, int t) {
     using G = Geo<LOG2N>;
-    if constexpr (P < G::NP - 1) {
+    if constexpr (LOG2N == 13) {
+        tw_tmem_fill<12, XCH>(tw8, base, t & 255);      // two 4096-point transforms
+    } else if constexpr (P < G::NP - 1) {
         constexpr int s = G::stride(P);
         const float2 *w = tw8 + G::tw8_off(P) + tw_index<LOG2N, P, XCH>(t);
         float v[32];
@@ -780,6 +789,14 @@ __device__ __forceinline__ void tw_tmem_fill(const float2 *tw8, uint32_t base, i
     }
 }
 
+// The twiddle that a thread keeps in registers (N = 8192; after the 4096-point
+// table of tw8).
+template <int LOG2N>
+__device__ __forceinline__ float2 tw_odd(const float2 *tw8, int t) {
+    if constexpr (LOG2N == 13) return __ldg(tw8 + Geo<12>::tw8_off(2) + (t & 255));
+    else return make_float2(0.f, 0.f);
+}
+
 // One global-table twiddle step (fetch and apply back to back).
 template <int LOG2N, int P, bool INV>
 __device__ __forceinline__ void twiddle(float2 *x, const float2 *tw, int t) {
@@ -789,11 +806,111 @@ __device__ __forceinline__ void twiddle(float2 *x, const float2 *tw, int t) {
     g.template apply<INV>(x, f);
 }
 
+// N = 8192 as two 4096-point transforms, by the parity of the frequency: the
+// even ones transform x[n] + x[n + 4096], the odd ones (x[n] - x[n + 4096])
+// W_8192^n, n < 4096.  Threads 0..255 do the even half, 256..511 the odd one
+// (groups with barriers of their own), each with three radix-16 passes and the
+// TMEM exchange of N = 4096; four passes with three exchanges over 512 threads
+// took 358 us where this takes 319 (24 filters, 2^22 samples).  In the time domain a thread of group g holds
+// n and n + 4096 for eight n = 256 (8 g + k) + t mod 256, so the butterfly is its
+// own, and half of its values go to the other group (swap_halves).
+// Shared memory: group g owns 8704 float2 at bufs + 8704 g: 4352 for the passes'
+// exchange, then two of 2048 for the halves, used in turn.  The passes' exchange
+// is a transform's only one in its buffer; the next one's write comes after the
+// halves' barrier of all 512 threads (the forward transform, whose halves come
+// first, ends with a barrier instead).
+template <class BAR>
+__device__ __forceinline__ void swap_halves(float2 *v, float2 *bufs, int t, int &xc, const BAR &bar) {
+    const int g = t >> 8, tl = t & 255;
+    float2 *hx = bufs + 4352 + 2048 * (xc & 1);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) hx[8704 * g + 256 * k + tl] = v[k];
+    bar();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = hx[8704 * (g ^ 1) + 256 * k + tl];
+    ++xc;
+}
+// x[j] *= (w e^{2 pi i j / 32})^(-1 forward, +1 inverse)
+template <bool INV>
+__device__ __forceinline__ void odd_twiddle(float2 *x, float2 w) {
+    constexpr float c32[9] = {1.f, 0.98078528040323044f, 0.92387953251128674f, 0.83146961230254524f,
+                              0.70710678118654752f, 0.55557023301960218f, 0.38268343236508977f,
+                              0.19509032201612825f, 0.f};
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {       // (each factor formed by itself: sharing those of j and j + 8 took 358 us
+        // where this takes 319, a longer live range each)
+        const float c = j <= 8 ? c32[j] : -c32[16 - j], s = j <= 8 ? c32[8 - j] : c32[j - 8];
+        const float2 wj = make_float2(fmaf(w.x, c, -w.y * s), fmaf(w.x, s, w.y * c));
+        x[j] = INV ? cmul(x[j], wj) : cmulc(x[j], wj);
+    }
+}
 template <int LOG2N, int P, class TW, class BAR = CtaBarrier>
 __device__ __forceinline__ void forward_passes(float2 *x, float2 *bufs, const TW &tw, int t, int &xc,
-                                               const BAR &bar = BAR{}) {
+                                               const BAR &bar = BAR{});
+template <int LOG2N, int P, class TW, class BAR = CtaBarrier>
+__device__ __forceinline__ void inverse_passes(float2 *x, float2 *bufs, const TW &tw, int t, int &xc,
+                                               const BAR &bar = BAR{});
+template <class TW, class BAR>
+__device__ __forceinline__ void forward13(float2 *x, float2 *bufs, const TW &tw, int t, int &xc, const BAR &bar) {
+    const int g = t >> 8;
+    float2 v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const float2 s = cadd(x[k], x[k + 8]), d = csub(x[k], x[k + 8]);
+        x[k] = g ? d : s;                    // kept
+        v[k] = g ? s : d;                    // the other group's
+    }
+    swap_halves(v, bufs, t, xc, bar);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const float2 own = x[k];
+        x[k] = g ? v[k] : own;
+        x[k + 8] = g ? own : v[k];
+    }
+    if (g) odd_twiddle<false>(x, tw.odd);
+    int one = 0;
+    forward_passes<12, 0>(x, bufs + 8704 * g, tw, t & 255, one, SegmentBarrier<256>{2 + g});
+    bar();
+}
+template <class TW, class BAR>
+__device__ __forceinline__ void inverse13(float2 *x, float2 *bufs, const TW &tw, int t, int &xc, const BAR &bar) {
+    const int g = t >> 8;
+    int one = 0;
+    inverse_passes<12, 2>(x, bufs + 8704 * g, tw, t & 255, one, SegmentBarrier<256>{2 + g});
+    float2 v[8];
+    if (g) {
+        odd_twiddle<true>(x, tw.odd);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = x[k];
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = x[k + 8];
+    }
+    swap_halves(v, bufs, t, xc, bar);
+    if (g) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float2 o = x[k + 8];
+            x[k] = cadd(v[k], o);
+            x[k + 8] = csub(v[k], o);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float2 e = x[k];
+            x[k] = cadd(e, v[k]);
+            x[k + 8] = csub(e, v[k]);
+        }
+    }
+}
+
+template <int LOG2N, int P, class TW, class BAR>
+__device__ __forceinline__ void forward_passes(float2 *x, float2 *bufs, const TW &tw, int t, int &xc,
+                                               const BAR &bar) {
     using G = Geo<LOG2N>;
-    if constexpr (P < G::NP - 1) {
+    if constexpr (LOG2N == 13 && is_tw_tmem<TW>::value) {
+        forward13(x, bufs, tw, t, xc, bar);
+    } else if constexpr (P < G::NP - 1) {
         if constexpr (is_tw_tmem<TW>::value) {
             tw.template dft_fwd<LOG2N, P>(x);
         } else {
@@ -823,11 +940,14 @@ __device__ __forceinline__ void forward_passes(float2 *x, float2 *bufs, const fl
 
 // x holds pass P+1's layout (or pass NP-1's when P == NP-1); runs the
 // inverse of passes P, P-1, ..., 0.
-template <int LOG2N, int P, class TW, class BAR = CtaBarrier>
+template <int LOG2N, int P, class TW, class BAR>
 __device__ __forceinline__ void inverse_passes(float2 *x, float2 *bufs, const TW &tw, int t, int &xc,
-                                               const BAR &bar = BAR{}) {
+                                               const BAR &bar) {
     using G = Geo<LOG2N>;
-    if constexpr (P < G::NP - 1) {
+    if constexpr (LOG2N == 13 && is_tw_tmem<TW>::value) {
+        inverse13(x, bufs, tw, t, xc, bar);
+        return;
+    } else if constexpr (P < G::NP - 1) {
         typename TW::Fetched f;
         // in flight during the exchange, except TMEM twiddles before the TMEM
         // exchange (their registers then are not live across it: with them the
@@ -853,7 +973,7 @@ __device__ __forceinline__ void inverse_passes(float2 *x, float2 *bufs, const TW
     } else {
         dft_groups<G::radix(P), true>(x);
     }
-    if constexpr (P > 0) inverse_passes<LOG2N, P - 1>(x, bufs, tw, t, xc, bar);
+    if constexpr (P > 0 && !(LOG2N == 13 && is_tw_tmem<TW>::value)) inverse_passes<LOG2N, P - 1>(x, bufs, tw, t, xc, bar);
 }
 template <int LOG2N, int P>
 __device__ __forceinline__ void inverse_passes(float2 *x, float2 *bufs, const float2 *tw, int t, int &xc) {

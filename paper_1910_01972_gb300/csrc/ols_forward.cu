@@ -22,17 +22,17 @@ struct EpiPlain {
     __device__ __forceinline__ void store(const float2 *x, int f, int t, const BankSegment &sg, float2 *, int &,
                                           const BAR &) const {
         using G = Geo<LOG2N>;
-        const int v = t - sg.n0;                 // output k T + v of the segment in register k
+        const int v = G::base(t) - sg.n0;                 // output v + off(k) of the segment in register k
         float2 *dst = y + (size_t)f * (size_t)sg.Nout + (sg.j0 + v);
         if (sg.span == G::N - sg.n0) {           // a full segment: only the aliased samples are dropped
 #pragma unroll
             for (int k = 0; k < 16; ++k)
-                if (v >= -k * G::T && in_bounds(sg.j0 + v + k * G::T < sg.Nout, sg.status)) __stcs(dst + k * G::T, x[k]);
+                if (v >= -G::off(k) && in_bounds(sg.j0 + v + G::off(k) < sg.Nout, sg.status)) __stcs(dst + G::off(k), x[k]);
         } else {
 #pragma unroll
             for (int k = 0; k < 16; ++k)
-                if ((unsigned)(v + k * G::T) < (unsigned)sg.span && in_bounds(sg.j0 + v + k * G::T < sg.Nout, sg.status))
-                    __stcs(dst + k * G::T, x[k]);
+                if ((unsigned)(v + G::off(k)) < (unsigned)sg.span && in_bounds(sg.j0 + v + G::off(k) < sg.Nout, sg.status))
+                    __stcs(dst + G::off(k), x[k]);
         }
     }
 };
@@ -76,7 +76,7 @@ PassPlan make_pass_plan(int log2N) {
         }
     }
     pp.twn = off;
-    pp.tw8n = off8;
+    pp.tw8n = log2N == 13 ? 8 * (256 + 16) + 256 : off8;   // N = 8192: two 4096-point transforms
     return pp;
 }
 

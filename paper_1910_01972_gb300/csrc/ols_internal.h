@@ -34,6 +34,23 @@ PassPlan make_pass_plan(int log2N);
 // Frequency index held at each storage position of the forward FFT output.
 void spectral_order(int log2N, int32_t *nu);
 
+// Storage order of a plan's spectra Hk: the frequency at storage position q
+// (register q % 16 of thread q / 16), and its inverse.
+enum SpectrumLayout : int {
+    LAYOUT_STD = 0,     // the digit-reversed order of the forward passes (spectral_order)
+    LAYOUT_ROWS64 = 1,  // N = 4096, ols_tc64.cu: thread 64 c + nu1, register j: nu1 + 64 (16 c + j)
+    LAYOUT_HALVES = 2   // N = 8192 in FP32: frequencies of parity g in threads 256 g .., 4096-point order
+};
+__host__ __device__ inline int layout_freq(int layout, int q) {
+    if (layout == LAYOUT_ROWS64) return ((q >> 4) & 63) + 64 * (16 * (q >> 10) + (q & 15));
+    return 2 * (((q >> 8) & 15) + 16 * ((q >> 4) & 15) + 256 * (q & 15)) + (q >> 12);
+}
+__host__ __device__ inline int layout_pos(int layout, int nu) {
+    if (layout == LAYOUT_ROWS64) return 16 * (((nu >> 10) << 6) + (nu & 63)) + ((nu >> 6) & 15);
+    const int m = nu >> 1;
+    return ((nu & 1) << 12) | ((m & 15) << 8) | (((m >> 4) & 15) << 4) | (m >> 8);
+}
+
 // Model-based segment length (no measurement): minimises (N / L)(log2 N + c).
 int64_t choose_segment_length(int32_t M);
 
@@ -138,7 +155,7 @@ struct ols_plan_s {
     float2 *hpack = nullptr;     // [ceil(F/2)][M] paired real filters h_{2p} + i h_{2p+1}
     uint16_t *tc_bmat = nullptr; // split DFT-16 matrices (fwd hi, fwd lo, inv hi, inv lo), core-matrix layout
                                  // (N = 4096: split DFT-64 matrix and twiddles, see tc64_tables)
-    bool rows64 = false;         // spectra in the order of ols_tc64.cu
+    int layout = 0;              // SpectrumLayout of Hk
     int *d_status = nullptr;     // device status word (bounded-wait failures)
     ols::Staging stage;
 };
@@ -247,12 +264,13 @@ cudaError_t prepare_backward(ols_plan_s &p);
 cudaError_t launch_backward(const ols_plan_s &p, const BackwardArgs &a, cudaStream_t st, int *launches);
 // Block size and grid of the adjoints window kernel for nseg windows.
 int backward_grid(const ols_plan_s &p, int64_t nseg, int *block);
-// FP64 precompute kernels.  Htk (may be null): the spectra of conj(h_f[M-1-k]).
+// FP64 precompute kernels.  Htk (may be null): the spectra of conj(h_f[M-1-k]),
+// always in the standard layout.
 cudaError_t launch_tw64(double2 *tw64, int N, cudaStream_t st);
 // Spectra in the 16-points-per-thread register layout of the kernels.
 cudaError_t launch_spectra(const float2 *h, int M, int F, int log2N, const int32_t *nu,
-                           const double2 *tw64, float2 *Hk, float2 *Htk, bool rows64, cudaStream_t st);
+                           const double2 *tw64, float2 *Hk, float2 *Htk, int layout, cudaStream_t st);
 cudaError_t launch_spectra_natural(const float2 *Hk, int F, int log2N, const int32_t *nu,
-                                   float2 *H, cudaStream_t st);
+                                   float2 *H, int layout, cudaStream_t st);
 
 }  // namespace ols

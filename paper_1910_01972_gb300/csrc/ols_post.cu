@@ -33,6 +33,17 @@
 
 namespace ols {
 
+// Thread and register that hold sample n of a segment in the time domain (the inverse of
+// Geo<>::base and off).
+template <class G>
+__device__ __forceinline__ int thread_of(int n) {
+    return G::N == 8192 ? ((n >> 11) & 1) * 256 + (n & 255) : n % G::T;
+}
+template <class G>
+__device__ __forceinline__ int reg_of(int n) {
+    return G::N == 8192 ? ((n >> 8) & 7) + 8 * (n >> 12) : n / G::T;
+}
+
 // The peak test of one output with a candidate power pk (called by whole warps,
 // only when some lane has a candidate: it stays out of the common path's
 // register allocation).  Neighbours n - 1 and n + 1 of output n = k T + t are
@@ -49,9 +60,17 @@ __device__ __noinline__ bool peak_test(bool hit, float pk, float up, float dn, i
     float prv = __shfl_sync(0xffffffffu, up, gl == 0 ? W - 1 : gl - 1, W);
     float nxt = __shfl_sync(0xffffffffu, dn, gl == W - 1 ? 0 : gl + 1, W);
     if constexpr (T > 32) {
-        const int w = t / 32, nw = T / 32;
-        if (gl == 0) prv = w > 0 ? edge[(nw + w - 1) * 16 + k] : edge[(2 * nw - 1) * 16 + (k > 0 ? k - 1 : 0)];
-        if (gl == W - 1) nxt = w < nw - 1 ? edge[(w + 1) * 16 + k] : edge[k < 15 ? k + 1 : 15];
+        constexpr int nw = T / 32;
+        using G = Geo<(T == 512 ? 13 : T == 256 ? 12 : T == 128 ? 11 : 10)>;
+        const int n = G::base(t) + G::off(k);
+        if (gl == 0) {
+            const int m = n > 0 ? n - 1 : 0;
+            prv = edge[(nw + thread_of<G>(m) / 32) * 16 + reg_of<G>(m)];
+        }
+        if (gl == W - 1) {
+            const int m = n < G::N - 1 ? n + 1 : n;
+            nxt = edge[thread_of<G>(m) / 32 * 16 + reg_of<G>(m)];
+        }
     }
     if (hit && !first) hit = pk > prv;
     if (hit && !last) hit = pk >= nxt;
@@ -132,13 +151,13 @@ struct EpiPost {
     __device__ __forceinline__ void store(const float2 *x, int f, int t, const BankSegment &sg, float2 *bufs, int &xc,
                                           const BAR &bar) const {
         using G = Geo<LOG2N>;
-        const int v = t - sg.n0;             // output k T + v of the segment in register k
+        const int v = G::base(t) - sg.n0;             // output v + off(k) of the segment in register k
         if constexpr (MODE == POST_POWER) {
             float *dst = static_cast<float *>(out) + (size_t)f * (size_t)sg.Nout + (sg.j0 + v);
 #pragma unroll
             for (int k = 0; k < 16; ++k)
-                if ((unsigned)(v + k * G::T) < (unsigned)sg.span && in_bounds(sg.j0 + v + k * G::T < sg.Nout, sg.status))
-                    __stcs(dst + k * G::T, fmaf(x[k].x, x[k].x, x[k].y * x[k].y));
+                if ((unsigned)(v + G::off(k)) < (unsigned)sg.span && in_bounds(sg.j0 + v + G::off(k) < sg.Nout, sg.status))
+                    __stcs(dst + G::off(k), fmaf(x[k].x, x[k].x, x[k].y * x[k].y));
         } else if constexpr (MODE == POST_DETECT) {
             // candidates are rare: one vote decides whether the warp has any at all
             float pw[16];
@@ -146,13 +165,13 @@ struct EpiPost {
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
                 pw[k] = fmaf(x[k].x, x[k].x, x[k].y * x[k].y);
-                any |= (unsigned)(v + k * G::T) < (unsigned)sg.span && pw[k] >= thr;
+                any |= (unsigned)(v + G::off(k)) < (unsigned)sg.span && pw[k] >= thr;
             }
             if (__any_sync(0xffffffffu, any)) {
 #pragma unroll
                 for (int k = 0; k < 16; ++k) {
-                    const bool hit = (unsigned)(v + k * G::T) < (unsigned)sg.span && pw[k] >= thr;
-                    append_candidates(hit, sg.j0 + (v + k * G::T), f, pw[k], cand, count, cap, sg.Nout, sg.status);
+                    const bool hit = (unsigned)(v + G::off(k)) < (unsigned)sg.span && pw[k] >= thr;
+                    append_candidates(hit, sg.j0 + (v + G::off(k)), f, pw[k], cand, count, cap, sg.Nout, sg.status);
                 }
             }
         } else if constexpr (MODE == POST_PEAK) {
@@ -178,11 +197,11 @@ struct EpiPost {
             const int k_last = (sg.span > 0 && rem == (long long)sg.span) ? sg.span - 1 : -2;
             bool any = false;
 #pragma unroll
-            for (int k = 0; k < 16; ++k) any |= (unsigned)(v + k * G::T) < (unsigned)sg.span && pw[k] >= thr;
+            for (int k = 0; k < 16; ++k) any |= (unsigned)(v + G::off(k)) < (unsigned)sg.span && pw[k] >= thr;
             if (!__any_sync(0xffffffffu, any)) return;
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
-                const int o = v + k * G::T;
+                const int o = v + G::off(k);
                 bool hit = (unsigned)o < (unsigned)sg.span && pw[k] >= thr &&
                            in_bounds(o + sg.n0 >= 1 && o + sg.n0 + 1 < G::N, sg.status);
                 if (__any_sync(0xffffffffu, hit))
@@ -195,16 +214,18 @@ struct EpiPost {
             float2 *dst = static_cast<float2 *>(out) + (size_t)f * (size_t)sg.Nout + (sg.j0 + v);
 #pragma unroll
             for (int k = 0; k < 16; ++k)
-                if ((unsigned)(v + k * G::T) < (unsigned)sg.span && in_bounds(sg.j0 + v + k * G::T < sg.Nout, sg.status))
-                    __stcs(dst + k * G::T, x[k]);
+                if ((unsigned)(v + G::off(k)) < (unsigned)sg.span && in_bounds(sg.j0 + v + G::off(k) < sg.Nout, sg.status))
+                    __stcs(dst + G::off(k), x[k]);
         } else {
             // y (circular order) to the exchange buffer not in use, padded q -> q + q/16;
             // then each output reads its two neighbours
-            float2 *dbuf = bufs + (xc & 1) * G::PADN;
-            ++xc;
+            // (N = 8192: the buffers of both halves, free between two barriers)
+            float2 *dbuf = LOG2N == 13 ? bufs : bufs + (xc & 1) * G::PADN;
+            if constexpr (LOG2N == 13) bar();
+            else ++xc;
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
-                const int n = k * G::T + t;
+                const int n = G::base(t) + G::off(k);
                 dbuf[n + (n >> 4)] = x[k];
             }
             bar();
@@ -214,7 +235,7 @@ struct EpiPost {
             const int n_last = (sg.Nout - sg.j0 == (long long)sg.span) ? sg.span - 1 + sg.n0 : -2;
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
-                const int n = k * G::T + t;
+                const int n = G::base(t) + G::off(k);
                 if ((unsigned)(n - sg.n0) < (unsigned)sg.span &&
                     in_bounds(sg.j0 - sg.n0 + n < sg.Nout && n >= 1 && n + 1 < G::N, sg.status)) {
                     const int lo = (n == n_first) ? n : n - 1;
@@ -224,6 +245,7 @@ struct EpiPost {
                     __stcs(dst + n, make_float2((b.x - a.x) * sc, (b.y - a.y) * sc));
                 }
             }
+            if constexpr (LOG2N == 13) bar();
         }
     }
 };

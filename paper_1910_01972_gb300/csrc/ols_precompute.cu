@@ -40,7 +40,7 @@ __global__ void tw64_kernel(double2 *tw64, int N) {
 // 435 -> 13; 64, 512, 4096 2962 -> 33; 24, 1025, 8192 5098 -> 31 us.
 __global__ void spectra_kernel(const float2 *__restrict__ h, int M, int log2N, const int32_t *__restrict__ nu_tab,
                                const double2 *__restrict__ tw64, float2 *__restrict__ Hk, float2 *__restrict__ Htk,
-                               bool rows64) {
+                               int layout) {
     extern __shared__ double2 smem64[];
     const int N = 1 << log2N, P = N / 16, lp = log2N - 4, TR = P / 2;
     const int grp = threadIdx.x / TR, i = threadIdx.x % TR;      // residue group of the block, its butterfly
@@ -78,18 +78,16 @@ __global__ void spectra_kernel(const float2 *__restrict__ h, int M, int log2N, c
     const int T = N / 16;
     for (int e = i; e < P; e += TR) {                            // e: (j, t) with t fastest
         const int tl = e & (P / 16 - 1), j = e / (P / 16);
-        int t = r * (P / 16) + tl, jj = j, nu;
-        if (rows64) {                                            // ols_tc64.cu: nu = nu1 + 64 (16 c + j), t = 64 c + nu1
-            nu = r + 16 * e;
-            t = ((nu >> 10) << 6) + (nu & 63);
-            jj = (nu >> 6) & 15;
-        } else {
-            nu = nu_tab[16 * t + j];
-        }
-        const int k = nu >> 4;
+        const int t = r * (P / 16) + tl;
+        const int nu = nu_tab[16 * t + j], k = nu >> 4;
         const double2 v = u[__brev((unsigned)k) >> (32 - lp)];
-        const size_t idx = (size_t)f * N + (size_t)(jj >> 1) * (2 * T) + 2 * t + (jj & 1);
-        Hk[idx] = make_float2((float)(v.x * inv), (float)(v.y * inv));
+        const size_t idx = (size_t)f * N + (size_t)(j >> 1) * (2 * T) + 2 * t + (j & 1);
+        size_t hidx = idx;
+        if (layout != LAYOUT_STD) {
+            const int q = layout_pos(layout, nu);
+            hidx = (size_t)f * N + (size_t)((q & 15) >> 1) * (2 * T) + 2 * (q >> 4) + (q & 1);
+        }
+        Hk[hidx] = make_float2((float)(v.x * inv), (float)(v.y * inv));
         if (Htk) {
             const double2 w = tw64[((long long)nu * (M - 1)) & (N - 1)];
             const double cr = fma(w.x, v.x, w.y * v.y), ci = fma(w.y, v.x, -w.x * v.y);   // w conj(v)
@@ -100,7 +98,7 @@ __global__ void spectra_kernel(const float2 *__restrict__ h, int M, int log2N, c
 
 // Natural-order copy of the plan's spectra: H[f][nu_tab[q]] = Hk[f][layout(q)].
 __global__ void spectra_natural_kernel(const float2 *__restrict__ Hk, int F, int log2N,
-                                       const int32_t *__restrict__ nu_tab, float2 *__restrict__ H) {
+                                       const int32_t *__restrict__ nu_tab, float2 *__restrict__ H, int layout) {
     const int N = 1 << log2N;
     const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= (long long)F * N) return;
@@ -108,7 +106,7 @@ __global__ void spectra_natural_kernel(const float2 *__restrict__ Hk, int F, int
     const int q = (int)(gid & (N - 1));
     const int T = N / 16, t = q >> 4, j = q & 15;
     const size_t idx = (size_t)f * N + (size_t)(j >> 1) * (2 * T) + 2 * t + (j & 1);
-    H[(size_t)f * N + nu_tab[q]] = Hk[idx];
+    H[(size_t)f * N + (layout == LAYOUT_STD ? nu_tab[q] : layout_freq(layout, q))] = Hk[idx];
 }
 
 cudaError_t launch_tw64(double2 *tw64, int N, cudaStream_t st) {
@@ -117,20 +115,20 @@ cudaError_t launch_tw64(double2 *tw64, int N, cudaStream_t st) {
 }
 
 cudaError_t launch_spectra(const float2 *h, int M, int F, int log2N, const int32_t *nu,
-                           const double2 *tw64, float2 *Hk, float2 *Htk, bool rows64, cudaStream_t st) {
+                           const double2 *tw64, float2 *Hk, float2 *Htk, int layout, cudaStream_t st) {
     const int P = (1 << log2N) / 16, block = P / 2 > 32 ? P / 2 : 32;
     const int per_block = block / (P / 2);
     const long long grid = (long long)F * (16 / per_block);
     if (grid > 0x7fffffffll) return cudaErrorInvalidValue;
     spectra_kernel<<<(unsigned)grid, block, sizeof(double2) * (size_t)(P * per_block), st>>>(h, M, log2N, nu, tw64, Hk,
-                                                                                            Htk, rows64);
+                                                                                            Htk, layout);
     return cudaGetLastError();
 }
 
 cudaError_t launch_spectra_natural(const float2 *Hk, int F, int log2N, const int32_t *nu, float2 *H,
-                                   cudaStream_t st) {
+                                   int layout, cudaStream_t st) {
     const long long total = (long long)F << log2N;
-    spectra_natural_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(Hk, F, log2N, nu, H);
+    spectra_natural_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(Hk, F, log2N, nu, H, layout);
     return cudaGetLastError();
 }
 

@@ -61,7 +61,7 @@ struct EpiReal {
     __device__ __forceinline__ void store(const float2 *x, int p, int t, const BankSegment &sg, float2 *, int &,
                                           const BAR &) const {
         using G = Geo<LOG2N>;
-        const int v = t - sg.n0;
+        const int v = G::base(t) - sg.n0;
         float *dre = y + (size_t)(2 * p) * (size_t)sg.Nout + (sg.j0 + v);
         // the pair test is uniform: taken once per filter pair, so each store
         // below is a plain predicated store
@@ -69,16 +69,16 @@ struct EpiReal {
             float *dim = dre + sg.Nout;
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
-                const bool ok = (unsigned)(v + k * G::T) < (unsigned)sg.span &&
-                                in_bounds(sg.j0 + v + k * G::T < sg.Nout, sg.status);
-                if (ok) __stcs(dre + k * G::T, x[k].x);
-                if (ok) __stcs(dim + k * G::T, x[k].y);
+                const bool ok = (unsigned)(v + G::off(k)) < (unsigned)sg.span &&
+                                in_bounds(sg.j0 + v + G::off(k) < sg.Nout, sg.status);
+                if (ok) __stcs(dre + G::off(k), x[k].x);
+                if (ok) __stcs(dim + G::off(k), x[k].y);
             }
         } else {
 #pragma unroll
             for (int k = 0; k < 16; ++k)
-                if ((unsigned)(v + k * G::T) < (unsigned)sg.span && in_bounds(sg.j0 + v + k * G::T < sg.Nout, sg.status))
-                    __stcs(dre + k * G::T, x[k].x);
+                if ((unsigned)(v + G::off(k)) < (unsigned)sg.span && in_bounds(sg.j0 + v + G::off(k) < sg.Nout, sg.status))
+                    __stcs(dre + G::off(k), x[k].x);
         }
     }
 };

@@ -30,11 +30,11 @@ __device__ __forceinline__ void ols_segment(const float2 *__restrict__ sig, long
     {
         const long long avail = active ? (Ns - start) : 0;
         const int lim = (int)(avail < G::N ? avail : G::N);
-        const float2 *src = sig + (active ? start : 0) + t;
+        const float2 *src = sig + (active ? start : 0) + G::base(t);
 #pragma unroll
         for (int k = 0; k < 16; ++k)
-            X[k] = (k * G::T + t < lim && in_bounds((active ? start : 0) + k * G::T + t < Ns, status))
-                       ? __ldg(src + k * G::T)
+            X[k] = (G::base(t) + G::off(k) < lim && in_bounds((active ? start : 0) + G::base(t) + G::off(k) < Ns, status))
+                       ? __ldg(src + G::off(k))
                        : make_float2(0.f, 0.f);
     }
     forward_passes<LOG2N, 0>(X, bufs, tw, t, xc, bar);
@@ -51,7 +51,7 @@ __device__ __forceinline__ void ols_segment(const float2 *__restrict__ sig, long
     // spectrum prefetch: its 32 registers make them spill (filter banks of 32
     // filters, Ns = 2^23: N = 512 0.479 against 0.531 ms, N = 1024 0.153
     // against 0.166 ms at Ns = 2^22, N = 4096 0.664 against 0.714 ms)
-    constexpr bool prefetch = OLS_PREFETCH_H && !(G::TX_NOPF && tw_xchg<TW>());
+    constexpr bool prefetch = OLS_PREFETCH_H && LOG2N != 13 && !(G::TX_NOPF && tw_xchg<TW>());
     float4 hn[8];
     const long long hn_end = (long long)F * (G::N / 2);   // float4 entries of the spectra
     if constexpr (prefetch) {
@@ -88,7 +88,7 @@ __device__ __forceinline__ void ols_segment(const float2 *__restrict__ sig, long
         float2 *dst = y + (size_t)f * (size_t)Nout;
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
-            const int n = k * G::T + t;
+            const int n = G::base(t) + G::off(k);
             if ((unsigned)(n - lo) < (unsigned)span && in_bounds(obase + n >= 0 && obase + n < Nout, status))
                 __stcs(dst + obase + n, x[k]);
         }
