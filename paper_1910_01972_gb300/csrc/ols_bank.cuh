@@ -76,6 +76,35 @@ struct BankSegment {
     int *status;
 };
 
+// y[f][j] written once, the aliased samples dropped.
+struct EpiPlain {
+    static constexpr int XCH = XCHG_TMEM;
+    template <int LOG2N>
+    static constexpr int edge() { return 0; }
+    const float2 *sig;
+    float2 *y;
+    __device__ __forceinline__ float2 sample(long long i) const { return __ldg(sig + i); }
+    template <int LOG2N>
+    __device__ __forceinline__ void spectrum(float2 *, int, const BankSegment &) const {}
+    template <int LOG2N, class BAR>
+    __device__ __forceinline__ void store(const float2 *x, int f, int t, const BankSegment &sg, float2 *, int &,
+                                          const BAR &) const {
+        using G = Geo<LOG2N>;
+        const int v = G::base(t) - sg.n0;                 // output v + off(k) of the segment in register k
+        float2 *dst = y + (size_t)f * (size_t)sg.Nout + (sg.j0 + v);
+        if (sg.span == G::N - sg.n0) {           // a full segment: only the aliased samples are dropped
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+                if (v >= -G::off(k) && in_bounds(sg.j0 + v + G::off(k) < sg.Nout, sg.status)) __stcs(dst + G::off(k), x[k]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+                if ((unsigned)(v + G::off(k)) < (unsigned)sg.span && in_bounds(sg.j0 + v + G::off(k) < sg.Nout, sg.status))
+                    __stcs(dst + G::off(k), x[k]);
+        }
+    }
+};
+
 template <int LOG2N, int BLOCK, class EPI>
 __global__ void __launch_bounds__(BLOCK, (BankGeo<LOG2N, BLOCK, EPI>::MINB))
 ols_bank_kernel(const BankArgs a, const EPI epi) {

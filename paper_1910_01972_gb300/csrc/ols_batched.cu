@@ -15,20 +15,6 @@
 #include "ols_internal.h"
 #include "ols_segment.cuh"
 
-// Segment lengths whose batch items use the TMEM exchange (bit i: N = 2^(9 + i)):
-// N = 2048 only.  The single-launch kernel holds every segment length's body,
-// so it runs at the register budget of the hungriest one: with the exchange
-// also at N = 1024 the batch took 9.10 instead of 8.87 ms, at 512 and 4096
-// 10.6-11.1 ms.
-#ifndef OLS_BATCH_TX_MASK
-#define OLS_BATCH_TX_MASK 0x4
-#endif
-// ... and for the kernels of the per-segment-length mode (one segment length
-// each): N = 2048 only as well (at every length: 8.90 against 8.86 ms)
-#ifndef OLS_BATCH_PERN_TX_MASK
-#define OLS_BATCH_PERN_TX_MASK 0x4
-#endif
-
 namespace ols {
 
 template <int LOG2N>
@@ -49,10 +35,8 @@ ols_batched_kernel(const BatchProblemDev *__restrict__ probs, const int2 *__rest
     tmem::fence_before_sync();
     __syncthreads();
     tmem::fence_after_sync();
-    // the TMEM exchange at the segment lengths of OLS_BATCH_PERN_TX_MASK
-    constexpr int xch = (LOG2N == 13 || in_tx_mask<LOG2N>(OLS_BATCH_PERN_TX_MASK)) ? XCHG_TMEM : XCHG_SMEM;
-    const TwTmemT<xch> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(twg, t)};
-    tw_tmem_fill<LOG2N, xch>(twg, tw.base, t);
+    const TwTmem tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(twg, t)};
+    tw_tmem_fill<LOG2N>(twg, tw.base, t);
     int xc = 0;
     for (;;) {
         __syncthreads();                       // previous item_sh readers are done
@@ -62,10 +46,8 @@ ols_batched_kernel(const BatchProblemDev *__restrict__ probs, const int2 *__rest
         if (item >= nitems) break;
         const int2 it = items[item];           // (problem, tile)
         const BatchProblemDev P = probs[it.x];
-        const long long nseg = P.nseg;
         const long long seg = (long long)it.y * G::SEGS + slot;
-        ols_segment<LOG2N>(s_ptrs[P.index], P.Ns, P.Hk, tw, y_ptrs[P.index], P.M, P.F, P.L, P.Nout, seg,
-                           seg < nseg, bufs, t, xc, CtaBarrier{}, P.status);
+        ols_segment<LOG2N>(P, s_ptrs[P.index], y_ptrs[P.index], tw, seg, bufs, t, xc, CtaBarrier{});
     }
     tmem::fence_before_sync();
     __syncthreads();
@@ -136,31 +118,32 @@ cudaError_t batched_launch(const BatchGroup &g, const float2 *const *s_ptrs, flo
 // twiddles once for the whole run.  Each segment is
 // processed exactly as by the plain kernel, so results are bitwise those of
 // per-problem calls.
+// A tile's body per segment length is a function of its own: inlined into one
+// kernel, the six bodies shared a register allocation and a choice that helped one
+// (the TMEM exchange, the spectrum prefetch) made another spill.  Returns xc.
 template <int BB, int LOG2N>
-__device__ __forceinline__ void batch_one_tile(const BatchProblemDev &P, int tile, bool fill,
-                                               const float2 *const *s_ptrs, float2 *const *y_ptrs, const float2 *tw,
-                                               float2 *smem, int &xc, uint32_t tbase) {
+__device__ __noinline__ int batch_one_tile(const BatchProblemDev *__restrict__ prob, int tile, bool fill,
+                                           const float2 *const *s_ptrs, float2 *const *y_ptrs, const float2 *tw,
+                                           int xc, uint32_t tbase) {
     using G = Geo<LOG2N>;
     if constexpr (G::T <= BB) {
+        extern __shared__ float4 smem_raw[];
         constexpr int SL = BB / G::T;
         static_assert(SL <= 15 || G::T <= 32, "one named barrier per slot");
+        const BatchProblemDev P = *prob;
         const int slot = threadIdx.x / G::T;
         const int t = threadIdx.x % G::T;
-        float2 *bufs = smem + slot * 2 * G::PADN;
+        float2 *bufs = reinterpret_cast<float2 *>(smem_raw) + slot * 2 * G::PADN;
         const long long seg = (long long)tile * SL + slot;
         const SegmentBarrier<G::T> bar{1 + slot};
-        // the same TMEM layout as the plain kernel (twiddles of this N, then the
-        // segment spectrum), so results stay bitwise those of per-problem calls
-        // (the TMEM exchange at the segment lengths of OLS_BATCH_TX_MASK); the
-        // twiddles are written on an item's first tile only
-        constexpr int xch = (LOG2N == 13 || in_tx_mask<LOG2N>(OLS_BATCH_TX_MASK)) ? XCHG_TMEM : XCHG_SMEM;
-        using TWT = TwTmemT<xch>;
-        const TWT twt{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(tw, t)};
-        if (fill) tw_tmem_fill<LOG2N, xch>(tw, twt.base, t);
-        ols_segment<LOG2N, TWT, SegmentBarrier<G::T>>(s_ptrs[P.index], P.Ns, P.Hk, twt, y_ptrs[P.index],
-                                                               P.M, P.F, P.L, P.Nout, seg, seg < P.nseg, bufs, t, xc,
-                                                         bar, P.status);
+        // the TMEM layout and exchange of the plain kernel, so results stay bitwise
+        // those of per-problem calls; the twiddles are written on an item's first
+        // tile only
+        const TwTmem twt{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(tw, t)};
+        if (fill) tw_tmem_fill<LOG2N>(tw, twt.base, t);
+        ols_segment<LOG2N>(P, s_ptrs[P.index], y_ptrs[P.index], twt, seg, bufs, t, xc, bar);
     }
+    return xc;
 }
 
 template <int BB>
@@ -168,10 +151,8 @@ __global__ void __launch_bounds__(BB, kBatchOneBlock / BB)
 ols_batched_one_kernel(const BatchProblemDev *__restrict__ probs, const int4 *__restrict__ items, long long nitems,
                        const float2 *const *__restrict__ s_ptrs, float2 *const *__restrict__ y_ptrs,
                        unsigned long long *__restrict__ ticket, TwTables tw) {
-    extern __shared__ float4 smem_raw[];
     __shared__ long long item_sh;
     __shared__ uint32_t tbase;
-    float2 *smem = reinterpret_cast<float2 *>(smem_raw);
     constexpr uint32_t kCols = (uint32_t)(BB / 128) * 128u;   // a 128-column lane range per 128 threads
     if (threadIdx.x < 32) tmem::alloc(&tbase, kCols);
     tmem::fence_before_sync();
@@ -198,15 +179,15 @@ ols_batched_one_kernel(const BatchProblemDev *__restrict__ probs, const int4 *__
             xc = 0;                            // buffers restart with every item
         }
         const int4 it = items[item];           // (problem, first tile, tiles)
-        const BatchProblemDev P = probs[it.x];
+        const BatchProblemDev *P = probs + it.x;
         const int tile = it.y + r;
-        switch (P.log2N) {
-            case 8: batch_one_tile<BB, 8>(P, tile, r == 0, s_ptrs, y_ptrs, tw.tw[8], smem, xc, tbase); break;
-            case 9: batch_one_tile<BB, 9>(P, tile, r == 0, s_ptrs, y_ptrs, tw.tw[9], smem, xc, tbase); break;
-            case 10: batch_one_tile<BB, 10>(P, tile, r == 0, s_ptrs, y_ptrs, tw.tw[10], smem, xc, tbase); break;
-            case 11: batch_one_tile<BB, 11>(P, tile, r == 0, s_ptrs, y_ptrs, tw.tw[11], smem, xc, tbase); break;
-            case 12: batch_one_tile<BB, 12>(P, tile, r == 0, s_ptrs, y_ptrs, tw.tw[12], smem, xc, tbase); break;
-            case 13: batch_one_tile<BB, 13>(P, tile, r == 0, s_ptrs, y_ptrs, tw.tw[13], smem, xc, tbase); break;
+        switch (P->log2N) {
+            case 8: xc = batch_one_tile<BB, 8>(P, tile, r == 0, s_ptrs, y_ptrs, tw.tw[8], xc, tbase); break;
+            case 9: xc = batch_one_tile<BB, 9>(P, tile, r == 0, s_ptrs, y_ptrs, tw.tw[9], xc, tbase); break;
+            case 10: xc = batch_one_tile<BB, 10>(P, tile, r == 0, s_ptrs, y_ptrs, tw.tw[10], xc, tbase); break;
+            case 11: xc = batch_one_tile<BB, 11>(P, tile, r == 0, s_ptrs, y_ptrs, tw.tw[11], xc, tbase); break;
+            case 12: xc = batch_one_tile<BB, 12>(P, tile, r == 0, s_ptrs, y_ptrs, tw.tw[12], xc, tbase); break;
+            case 13: xc = batch_one_tile<BB, 13>(P, tile, r == 0, s_ptrs, y_ptrs, tw.tw[13], xc, tbase); break;
             default: break;
         }
         ++r;

@@ -26,9 +26,6 @@
 #include "tmem.cuh"
 
 // Tuning knobs (compile-time; defaults are the measured best on GB300).
-#ifndef OLS_PREFETCH_H
-#define OLS_PREFETCH_H 1     // load filter f+1's spectrum while filter f is transformed
-#endif
 #ifndef OLS_XBUFS
 #define OLS_XBUFS 2          // exchange buffers per segment (2: one barrier per exchange)
 #endif
@@ -37,9 +34,6 @@
 #endif
 #ifndef OLS_TX_MASK
 #define OLS_TX_MASK 0xF      // segment lengths with the TMEM exchange: bit i for N = 2^(9 + i)
-#endif
-#ifndef OLS_TX_NOPF_MASK
-#define OLS_TX_NOPF_MASK 0xB // ... and among them those run without the spectrum prefetch (512, 1024, 4096)
 #endif
 #ifndef OLS_WARPS_PER_SM
 #define OLS_WARPS_PER_SM 16  // resident warps per SM the register budget must allow
@@ -103,7 +97,6 @@ struct Geo {
     // with TMEM twiddles; columns 64..95 of the thread's block are free)
     static constexpr bool TX = OLS_TMEM_XCHG && LOG2N >= 9 && LOG2N <= 12 &&
                                ((OLS_TX_MASK >> (LOG2N - 9)) & 1);
-    static constexpr bool TX_NOPF = TX && ((OLS_TX_NOPF_MASK >> (LOG2N - 9)) & 1);
     // ... with pass NP-2's lanes relabelled (N = 2048)
     static constexpr bool TX_RELABEL = TX;
     static constexpr int XBUFS = OLS_XBUFS;
@@ -122,13 +115,6 @@ struct Geo {
 // through shared memory, through TMEM where Geo<>::TX allows it, or (N = 2048;
 // else as XCHG_TMEM) through TMEM with one of the three bits by shuffles.
 enum : int { XCHG_SMEM = 0, XCHG_TMEM = 1, XCHG_SHFL = 2 };
-
-// Whether segment length 2^LOG2N is in a mask of segment lengths (bit i for
-// N = 2^(9 + i)), the form of the per-kernel TMEM-exchange choices.
-template <int LOG2N>
-__host__ __device__ constexpr bool in_tx_mask(unsigned mask) {
-    return LOG2N >= 9 && LOG2N <= 12 && ((mask >> (LOG2N - 9)) & 1u);
-}
 
 // Padded shared-memory base of thread t in the layout of pass P:
 // positions (t / s) * 16 s + (t % s) + k s, padded q -> q + q / 16.
