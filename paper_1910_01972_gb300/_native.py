@@ -92,6 +92,8 @@ class OLSError(RuntimeError):
 def lib():
     """The loaded library (raises if it has not been built)."""
     global _lib
+    if _lib is not None:        # set once, under the lock below
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib

@@ -25,9 +25,8 @@ _lock = threading.Lock()
 
 def _plan(M: int, F: int, N: int, device: torch.device):
     """(plan, lock) for the current stream of `device`."""
-    from . import Plan
-    stream = torch.cuda.current_stream(device).cuda_stream
-    key = (M, F, N, device.index, stream)
+    from . import Plan, _stream_ptr
+    key = (M, F, N, device.index, _stream_ptr(device))
     with _lock:
         entry = _plans.get(key)
         if entry is None:
@@ -39,7 +38,9 @@ def _plan(M: int, F: int, N: int, device: torch.device):
 
 def _values(t: torch.Tensor) -> torch.Tensor:
     # lazy conjugate / negative views carry a flag, not the values, in memory
-    return t.resolve_conj().resolve_neg().contiguous()
+    if t.is_conj() or t.is_neg():
+        t = t.resolve_conj().resolve_neg()
+    return t if t.is_contiguous() else t.contiguous()
 
 
 class OLSConvFunction(torch.autograd.Function):
