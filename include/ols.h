@@ -78,8 +78,8 @@ typedef struct ols_batch_s *ols_batch_t;
 
 /* Plan flags (arithmetic of the convolution). */
 #define OLS_FLAG_FP32 0u
-/* Every radix-16 FFT stage as a tensor-core (tcgen05) matrix product on
- * 16-bit split operands x = x_hi + x_lo and DFT matrices W = W_hi + W_lo,
+/* Every radix-16 FFT stage (N = 4096: two radix-64 stages) as a tensor-core
+ * (tcgen05) matrix product on 16-bit split operands x = x_hi + x_lo and DFT matrices W = W_hi + W_lo,
  * D = x_hi W_hi + x_hi W_lo + x_lo W_hi with FP32 accumulation; twiddles,
  * the point-wise product and the exchanges stay FP32.  FP16 split: ~22
  * significant bits per operand; BF16 split: ~16 bits.  Input range: the
@@ -121,6 +121,9 @@ OLS_API int ols_geometry(int64_t N, int32_t M, int64_t Ns, int64_t *L, int64_t *
  * transform consumes it, so the forward FFT skips the reordering step.  This
  * returns, for each storage position q in [0, N), the frequency index
  * nu[q] held there (a permutation of [0, N)).  nu: host array of N int32.
+ * (Two kernels hold the spectrum in orders of their own -- N = 8192 in FP32, by
+ * the parity of the frequency, and the tensor-core form at N = 4096;
+ * ols_get_spectra returns natural order for every plan.)
  */
 OLS_API int ols_spectrum_order(int64_t N, int32_t *nu);
 

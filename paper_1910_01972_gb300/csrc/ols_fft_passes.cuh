@@ -29,12 +29,6 @@
 #ifndef OLS_XBUFS
 #define OLS_XBUFS 2          // exchange buffers per segment (2: one barrier per exchange)
 #endif
-#ifndef OLS_TMEM_XCHG
-#define OLS_TMEM_XCHG 1      // N = 512..4096: the exchange between the last two passes goes through TMEM (0: shared memory)
-#endif
-#ifndef OLS_TX_MASK
-#define OLS_TX_MASK 0xF      // segment lengths with the TMEM exchange: bit i for N = 2^(9 + i)
-#endif
 #ifndef OLS_WARPS_PER_SM
 #define OLS_WARPS_PER_SM 16  // resident warps per SM the register budget must allow
 #endif
@@ -95,10 +89,7 @@ struct Geo {
     }
     // the exchange between the last two passes goes through TMEM (kernels
     // with TMEM twiddles; columns 64..95 of the thread's block are free)
-    static constexpr bool TX = OLS_TMEM_XCHG && LOG2N >= 9 && LOG2N <= 12 &&
-                               ((OLS_TX_MASK >> (LOG2N - 9)) & 1);
-    // ... with pass NP-2's lanes relabelled (N = 2048)
-    static constexpr bool TX_RELABEL = TX;
+    static constexpr bool TX = LOG2N >= 9 && LOG2N <= 12;
     static constexpr int XBUFS = OLS_XBUFS;
     static constexpr size_t SMEM = sizeof(float2) * (size_t)(SEGS * XBUFS * PADN);
     // TMEM twiddles: 128 columns per 128 threads (a thread's lane, 32 columns per pass)
@@ -582,7 +573,7 @@ __device__ __forceinline__ void tx_inverse(float2 *x, uint32_t xb) {
 template <int LOG2N, int P, int XCH>
 __device__ __forceinline__ int tw_index(int t) {
     using G = Geo<LOG2N>;
-    if constexpr (XCH && G::TX_RELABEL && P == G::NP - 2) {   // the relabelled lanes holding p0 .. p(s-1)
+    if constexpr (XCH && G::TX && P == G::NP - 2) {   // the relabelled lanes holding p0 .. p(s-1)
         if constexpr (LOG2N == 11) return XCH == XCHG_SHFL ? ((t >> 3) & 3) + 4 * (t & 1) : (t >> 1) & 7;
         else if constexpr (LOG2N == 12) return (t & 3) + 4 * ((t >> 3) & 1) + 8 * ((t >> 4) & 1);
         else if constexpr (LOG2N == 10) return (t >> 3) & 3;
@@ -910,7 +901,7 @@ __device__ __forceinline__ void forward_passes(float2 *x, float2 *bufs, const TW
             tx_forward<LOG2N, TW::xchg>(x, tw.xbase());
         } else {
             float2 *buf = bufs + (G::XBUFS == 2 ? (xc & 1) * G::PADN : 0);
-            if constexpr (tx && G::TX_RELABEL && P + 1 == G::NP - 2) exchange_tx<LOG2N, P, P + 1, TW::xchg>(x, buf, t, bar);
+            if constexpr (tx && P + 1 == G::NP - 2) exchange_tx<LOG2N, P, P + 1, TW::xchg>(x, buf, t, bar);
             else exchange<LOG2N, P, P + 1>(x, buf, t, bar);
             ++xc;
         }
@@ -945,7 +936,7 @@ __device__ __forceinline__ void inverse_passes(float2 *x, float2 *bufs, const TW
             tx_inverse<LOG2N, TW::xchg>(x, tw.xbase());
         } else {
             float2 *buf = bufs + (G::XBUFS == 2 ? (xc & 1) * G::PADN : 0);
-            if constexpr (tx && G::TX_RELABEL && P + 1 == G::NP - 2) exchange_tx<LOG2N, P + 1, P, TW::xchg>(x, buf, t, bar);
+            if constexpr (tx && P + 1 == G::NP - 2) exchange_tx<LOG2N, P + 1, P, TW::xchg>(x, buf, t, bar);
             else exchange<LOG2N, P + 1, P>(x, buf, t, bar);
             ++xc;
         }
