@@ -405,16 +405,18 @@ cudaError_t prepare_backward(ols_plan_s &p) {
 // stay within 16 MB: a block runs its windows' F + 2 transforms in a row, so
 // more blocks of fewer windows finish sooner (F = 8: 45 windows of N = 512 in
 // 12 blocks instead of 3 43 -> 27 us, 37 of N = 1024 in 19 instead of 10 31 ->
-// 27 us).  The bound on the spectra keeps the whole workspace of such a call
-// below OLS_NOALLOC_SCRATCH_BYTES (16 MB of spectra, at most 8 MB for their
-// sum, at most 10 MB of edges, and not all at once), so the rule, which looks
-// neither at the gradients wanted nor at the entry point, makes no call too
-// large for the scratch that large blocks would have fitted.
+// 27 us).  A small-block call whose whole workspace (both gradients) would not
+// fit OLS_NOALLOC_SCRATCH_BYTES keeps the large blocks (filters nearly as long
+// as the segment have edges of up to 20 MB): the rule makes no call too large for
+// that scratch.  It looks neither at the gradients wanted nor at the entry point.
 int backward_grid(const ols_plan_s &p, int64_t nseg, int *block) {
     const int T = p.pp.T, large = p.log2N == 10 ? 256 : 512, small = T > 128 ? T : 128;
     const int64_t gs = (nseg + small / T - 1) / (small / T), gl = (nseg + large / T - 1) / (large / T);
     const int64_t spec = (int64_t)sizeof(float2) * p.F * p.N;
-    if (small < large && gs > gl && gs <= (int64_t)(512 / small) * p.sm_count && gs * spec <= (int64_t)16 << 20) {
+    const int64_t edges = (int64_t)sizeof(float2) * nseg * 2 * (p.M - 1);
+    const int64_t need = edges + (gs + 1) * spec + 3 * 256;       // each part rounded up to 256 bytes
+    if (small < large && gs > gl && gs <= (int64_t)(512 / small) * p.sm_count && gs * spec <= (int64_t)16 << 20 &&
+        need <= (int64_t)OLS_NOALLOC_SCRATCH_BYTES) {
         *block = small;
         return (int)gs;
     }

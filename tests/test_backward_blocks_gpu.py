@@ -33,3 +33,15 @@ def test_few_windows_against_oracle(N, M, F, windows):
     assert oracle.rel_l2(ds.cpu().numpy(), ds_ref) <= 2e-6
     assert oracle.max_stream_rel_l2(dh.cpu().numpy(), dh_ref) <= 1e-5
     plan.close()
+
+
+@pytest.mark.parametrize("N,M,F,windows", [(2048, 2048, 2, 512), (512, 511, 6, 2432), (256, 255, 13, 4864)])
+def test_scratch_still_takes_long_filters(N, M, F, windows):
+    # edges (16 windows (M - 1) bytes) beside the spectra of every small block would exceed the
+    # scratch; those of the large blocks fit it
+    _build.build()
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    plan = Plan(M, F, N)
+    assert plan.backward_workspace(windows * (N - M + 1) + M - 1) <= _native.OLS_NOALLOC_SCRATCH_BYTES
+    plan.close()
