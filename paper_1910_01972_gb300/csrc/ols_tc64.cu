@@ -33,9 +33,11 @@
 // store, wait and exchange three times, and their threads' work bounds them:
 // 64 filters, 2^22 samples 1156 us there, 733 here (FP16; the FP32 kernel 620).
 // Spectra prefetched a filter ahead 761 us: their registers spill.
-// Scales (exact powers of two) keep the split's low parts normal and every
-// 16-bit operand in range for |s| <= 1.42 and unit-L2 filters: spectra of the
-// segment x 512 (|Y| <= 91 for M <= N), stage 2's operand x 64 (|Z| <= 724).
+// Scales (exact powers of two): spectra of the segment x 16 (|Y| <= 2.9 for |s| <=
+// 1.42, unit-L2 filters and M <= N), stage 2's operand x 2 (|Z| <= 23).  They give
+// FP16 operands the range of ols_tc.cu: a tone of |s| = 64 in its matched filter
+// comes through (x 512 it overflowed from |s| = 4 on, with the same error at
+// |s| <= 1.42: 6.8e-7).
 // Waits are bounded as in ols_tc.cu.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -341,11 +343,11 @@ ols_tc64_kernel(const float2 *__restrict__ sig, const uint32_t *__restrict__ sig
                 ok = wait_done(bars, 1, phase, wait_limit, status);
                 if (!ok) break;
                 load_d(X, lane, 1, q);
-                // conjugate back; x 8 undoes the twiddles' 1/8, x 512 is the spectrum's scale
+                // conjugate back; x 8 undoes the twiddles' 1/8, x 16 is the spectrum's scale
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
-                    xs[512 * i] = make_float4(X[2 * i].x * 4096.f, X[2 * i].y * -4096.f, X[2 * i + 1].x * 4096.f,
-                                              X[2 * i + 1].y * -4096.f);
+                    xs[512 * i] = make_float4(X[2 * i].x * 128.f, X[2 * i].y * -128.f, X[2 * i + 1].x * 128.f,
+                                              X[2 * i + 1].y * -128.f);
             }
             const long long rem = active ? Nout - start : 0;
             const int span = (int)(rem < L ? rem : L);
@@ -396,7 +398,7 @@ ols_tc64_kernel(const float2 *__restrict__ sig, const uint32_t *__restrict__ sig
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
                         if ((unsigned)(v0 + 64 * j) < (unsigned)span && in_bounds(start + v0 + 64 * j < Nout, status))
-                            __stcs(dst + 64 * j, make_float2(z[j].x * (1.f / 64.f), z[j].y * (1.f / 64.f)));
+                            __stcs(dst + 64 * j, make_float2(z[j].x * 0.5f, z[j].y * 0.5f));
                 }
             }
         }

@@ -42,3 +42,21 @@ def test_parity(flag, M, F, Ns):
     hi, lo = p.split_signal(dev(s))
     assert torch.equal(p.convolve_split(hi, lo), y)
     p.close()
+
+
+@pytest.mark.parametrize("M,amplitude", [(512, 64.0), (4000, 64.0), (512, 2.0 ** -6), (4000, 2.0 ** -6)])
+def test_range_of_a_matched_tone(M, amplitude):
+    # a tone in its matched filter gathers a segment's energy in one bin: the largest 16-bit operands
+    # an amplitude can give.  The range is the radix-16 form's, FP16 split, bound as above.
+    _build.build()
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    Ns, w = 20_000, 2.0 * np.pi * 37 / 4096
+    s = (amplitude * np.exp(1j * w * np.arange(Ns))).astype(np.complex64)
+    h = (np.exp(1j * w * np.arange(M)) / np.sqrt(M)).astype(np.complex64)[None]
+    p = Plan(M, 1, 4096, flags=_native.OLS_FLAG_TC_FP16SPLIT)
+    p.set_filters(dev(h))
+    y = p.convolve(dev(s)).cpu().numpy()
+    assert p.status() == 0
+    assert oracle.rel_l2(y, oracle.conv(s, h)) <= BOUND[_native.OLS_FLAG_TC_FP16SPLIT]
+    p.close()
