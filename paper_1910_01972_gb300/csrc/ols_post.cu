@@ -3,9 +3,9 @@
 // "optional post-processing" step; Sec. 4.3: per-element and non-local
 // post-processing; Sec. 4.4: reducing the output before it leaves the GPU).
 //
-// Four epilogues on the same segment body as ols_forward.cu (segment FFT
-// kept in registers for all filters; per filter the point-wise product, the
-// inverse FFT and the discard of aliased samples):
+// Four epilogues of the bank kernel (ols_bank.cuh: the segment's spectrum kept in
+// tensor memory for all filters; per filter the point-wise product, the inverse
+// FFT and the discard of aliased samples):
 // * POWER   (per element)   p_f[j] = |y_f[j]|^2, written as FP32 (half the
 //   output bytes of y);
 // * DETECT  (per element + selection) the candidates (f, j) whose power
@@ -15,8 +15,9 @@
 //   differences (y[j+1] - y[j-1]) / 2 inside, one-sided differences at j = 0
 //   and j = Nout-1.  Each segment advances by L-2 instead of L and starts one
 //   output early, so every derivative it writes has both neighbours among
-//   its own unaliased samples (the "immediate neighbourhood" of Sec. 4.3);
-//   the neighbours are exchanged through a shared-memory buffer of their own.
+//   its own unaliased samples (the "immediate neighbourhood" of Sec. 4.3).
+//   Inside the stream the difference is taken on the segment's spectrum; the
+//   segments at its two ends exchange neighbours through shared memory.
 // * PEAK    (non-local + selection) the peaks of the power (Sec. 4.4's peak
 //   finding): (f, j) whose power reaches the threshold, is above the power of
 //   j - 1 and at least that of j + 1 (no neighbour at the two ends of the
@@ -104,7 +105,7 @@ __device__ __forceinline__ void append_candidates(bool hit, long long j, int f, 
 
 template <int MODE>
 struct EpiPost {
-    // the TMEM exchange everywhere (a CTA's registers now hold it without spills)
+    // POWER: one of the exchange's three bits by shuffles (as the real form)
     static constexpr int XCH = MODE == POST_POWER ? XCHG_SHFL : XCHG_TMEM;
     // PEAK: warp-edge powers [2][T/32][16] floats per segment of several warps
     template <int LOG2N>
