@@ -215,7 +215,10 @@ cudaError_t bank_launch_block(BankArgs a, const EPI &epi, int sm_count, cudaStre
 // blocks of 512 / 256: N = 256 94 / 97 us, 1024 113 / 120, 2048 133 / 141); with fewer
 // than four steps per SM two CTAs of 256 start and end sooner (32 filters,
 // 2^15 samples, N = 2048: 12.5 / 11.0 us; from 2^17 samples on the two are
-// equal).  At N = 4096 a 512-thread CTA holds only two segments and 256
+// equal).  While CTAs of 128 threads, four per SM, leave at most one step each,
+// they set up sooner and reach more SMs (one filter, 2^16 samples, 256 / 128:
+// N = 256 6.4 / 5.2 us, 512 6.6 / 5.2, 2048 6.6 / 5.4; 32 filters, 2^15 samples, N = 512
+// 9.7 / 8.6, 1024 9.8 / 8.6).  At N = 4096 a 512-thread CTA holds only two segments and 256
 // threads, one segment, were faster throughout (166 / 159 us; one filter, 2^23
 // samples: 52 / 48 us).  N = 8192 needs 512 threads for its one segment.
 template <int LOG2N, class EPI>
@@ -224,6 +227,9 @@ cudaError_t bank_prepare() {
     if constexpr (LOG2N != 12) e = bank_prepare_block<LOG2N, 512, EPI>();
     if constexpr (LOG2N != 13) {
         if (e == cudaSuccess) e = bank_prepare_block<LOG2N, 256, EPI>();
+    }
+    if constexpr (LOG2N < 12) {
+        if (e == cudaSuccess) e = bank_prepare_block<LOG2N, 128, EPI>();
     }
     return e;
 }
@@ -236,6 +242,8 @@ cudaError_t bank_launch(const BankArgs &a, const EPI &epi, int sm_count, cudaStr
     } else {
         constexpr int SL = 512 / Geo<LOG2N>::T;
         const long long steps = (a.nseg + SL - 1) / SL * a.F;
+        constexpr int SL1 = 128 / Geo<LOG2N>::T;
+        if ((a.nseg + SL1 - 1) / SL1 * a.F <= 4ll * sm_count) return bank_launch_block<LOG2N, 128>(a, epi, sm_count, st);
         if (steps < 4ll * sm_count) return bank_launch_block<LOG2N, 256>(a, epi, sm_count, st);
         return bank_launch_block<LOG2N, 512>(a, epi, sm_count, st);
     }

@@ -107,3 +107,25 @@ def test_derivative_ends(N, M, extra):
     err = max(np.linalg.norm(d[f] - ref[f]) / max(np.linalg.norm(y[f]), scale[f]) for f in range(3))
     assert err <= TOL
     plan.close()
+
+
+@pytest.mark.parametrize("N,M", [(256, 33), (512, 65), (1024, 129), (2048, 257)])
+def test_smallest_blocks(N, M):
+    """128-thread CTAs (at most one step each on 148 SMs or more) against the oracle, and bit for bit
+    the head of a signal past that rule (256-thread CTAs), in each form."""
+    F, L, per = 9, N - M + 1, 2048 // N                 # `per` segments to a 128-thread CTA
+    s, h = inputs(N + 7, 60 * per * L + M - 1 - 5, F, M)          # 540 steps; the last segment ragged
+    tail = inputs(N + 8, 20 * per * L, F, M)[0]                   # 720 in all
+    plan = Plan(M, F, N)
+    plan.set_filters(dev(h))
+    a, b = plan.convolve(dev(s)), plan.convolve(dev(np.concatenate([s, tail])))
+    whole = (60 * per - 1) * L
+    assert torch.equal(a[:, :whole], b[:, :whole])
+    y = a.cpu().numpy()
+    assert oracle.max_stream_rel_l2(y, oracle.conv(s, h), oracle.stream_scale(s, h, y.shape[1])) <= TOL
+    p, q = plan.convolve_power(dev(s)), plan.convolve_power(dev(np.concatenate([s, tail])))
+    assert torch.equal(p[:, :whole], q[:, :whole])
+    d, e = plan.convolve_derivative(dev(s)), plan.convolve_derivative(dev(np.concatenate([s, tail])))
+    inner = (whole // (L - 2) - 1) * (L - 2)            # whole segments of the derivative in both signals
+    assert torch.equal(d[:, :inner], e[:, :inner])
+    plan.close()
