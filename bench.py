@@ -79,6 +79,12 @@ def tc_flops(N, F, nseg):
     return nseg * (lg // 4) * (F + 1) * (N // 16) * 6 * 2 * 32 * 16
 
 
+def tc64_flops(F, nseg):
+    """The same of the N = 4096 form (two radix-64 stages): 48 MMAs of 128 x 128 x
+    16 per pair of segments and transform (F inverse ones and the forward one)."""
+    return (nseg + 1) // 2 * (F + 1) * 48 * 2 * 128 * 128 * 16
+
+
 def tc_peak():
     """Dense 16-bit tensor peak in TFLOP/s: the measured bf16 burst figure (FP16
     and BF16 run at the same kind::f16 rate), or the nominal 2250."""
@@ -484,7 +490,7 @@ def _tensor_core(res, samples, peak, ns=0):
                        "hbm_frac": tb / (ms * 1e-3) / 1e9 / peak, "status": q.status()}
         if flag:
             nseg = q.query(cfg.Ns)["nseg"]
-            fl = tc_flops(cfg.N, cfg.F, nseg)
+            fl = tc64_flops(cfg.F, nseg) if cfg.N == 4096 else tc_flops(cfg.N, cfg.F, nseg)
             tp, tk = tc_peak()
             tcres[name].update({"tensor_tflops": fl / (ms * 1e-3) / 1e12, "tensor_frac": fl / (ms * 1e-3) / 1e12 / tp,
                                 "tensor_flops_per_launch": fl, "tensor_peak": tp, "tensor_peak_kind": tk})
