@@ -106,6 +106,33 @@ struct EpiPlain {
     }
 };
 
+// A segment's filters f .. fend - 1 of F, its spectrum in the thread's tensor-memory
+// lane and filter f's in h: product, inverse FFT, epilogue (the loop of the bank
+// and of the batch kernels).  At N = 256 a warp holds two segments, whose epilogues
+// may take different branches (a full segment beside a ragged or idle one), while
+// the tensor-memory accesses of the next filter, or of the next segment, are
+// warp-wide: the warp meets again after each epilogue.
+template <int LOG2N, class EPI, class TW, class LOADH, class BAR>
+__device__ __forceinline__ void segment_filters(const EPI &epi, const TW &tw, float4 *h, const LOADH &load_h, int f,
+                                                int fend, int F, const BankSegment &sg, float2 *bufs, int t, int &xc,
+                                                const BAR &bar) {
+    using G = Geo<LOG2N>;
+    for (; f < fend; ++f) {
+        float2 x[16];
+        tmem::ld32(tw.base + 96, reinterpret_cast<float *>(x));
+        tmem::wait_ld();
+#pragma unroll
+        for (int j2 = 0; j2 < 8; ++j2) {
+            x[2 * j2] = cmul(x[2 * j2], make_float2(h[j2].x, h[j2].y));
+            x[2 * j2 + 1] = cmul(x[2 * j2 + 1], make_float2(h[j2].z, h[j2].w));
+        }
+        load_h(f + 1 == F ? 0 : f + 1);          // of this segment, or the first of the next
+        inverse_passes<LOG2N, G::NP - 1>(x, bufs, tw, t, xc, bar);
+        epi.template store<LOG2N>(x, f, t, sg, bufs, xc, bar);
+        if constexpr (G::T < 32) __syncwarp();
+    }
+}
+
 template <int LOG2N, int BLOCK, class EPI>
 __global__ void __launch_bounds__(BLOCK, (BankGeo<LOG2N, BLOCK, EPI>::MINB))
 ols_bank_kernel(const BankArgs a, const EPI epi) {
@@ -173,20 +200,7 @@ ols_bank_kernel(const BankArgs a, const EPI epi) {
         }
         const int fend = a.F - f < todo ? a.F : f + (int)todo;
         todo -= fend - f;
-        for (; f < fend; ++f) {
-            float2 x[16];
-            tmem::ld32(xcol, reinterpret_cast<float *>(x));
-            tmem::wait_ld();
-#pragma unroll
-            for (int j2 = 0; j2 < 8; ++j2) {
-                x[2 * j2] = cmul(x[2 * j2], make_float2(h[j2].x, h[j2].y));
-                x[2 * j2 + 1] = cmul(x[2 * j2 + 1], make_float2(h[j2].z, h[j2].w));
-            }
-            load_h(f + 1 == a.F ? 0 : f + 1);        // of this segment, or the first of the next
-            inverse_passes<LOG2N, G::NP - 1>(x, bufs, tw, t, xc, bar);
-            epi.template store<LOG2N>(x, f, t, sg, bufs, xc, bar);
-            if constexpr (G::T < 32) __syncwarp();   // two slots of a warp may have taken different paths
-        }
+        segment_filters<LOG2N>(epi, tw, h, load_h, f, fend, a.F, sg, bufs, t, xc, bar);
     }
     tmem::fence_before_sync();
     __syncthreads();

@@ -51,19 +51,7 @@ __device__ __forceinline__ void ols_segment(const BatchProblemDev &P, const floa
             if (in_bounds(ff < F, sg.status)) h[j2] = load_spectrum(hp + j2 * G::T);
     };
     load_h(0);
-    for (int f = 0; f < F; ++f) {
-        float2 x[16];
-        tmem::ld32(xcol, reinterpret_cast<float *>(x));
-        tmem::wait_ld();
-#pragma unroll
-        for (int j2 = 0; j2 < 8; ++j2) {
-            x[2 * j2] = cmul(x[2 * j2], make_float2(h[j2].x, h[j2].y));
-            x[2 * j2 + 1] = cmul(x[2 * j2 + 1], make_float2(h[j2].z, h[j2].w));
-        }
-        load_h(f + 1 == F ? 0 : f + 1);
-        inverse_passes<LOG2N, G::NP - 1>(x, bufs, tw, t, xc, bar);
-        epi.template store<LOG2N>(x, f, t, sg, bufs, xc, bar);
-    }
+    segment_filters<LOG2N>(epi, tw, h, load_h, 0, F, F, sg, bufs, t, xc, bar);
 }
 
 }  // namespace ols
