@@ -195,6 +195,7 @@ ols_bank_kernel(const BankArgs a, const EPI epi) {
             }
             forward_passes<LOG2N, 0>(X, bufs, tw, t, xc, bar);
             epi.template spectrum<LOG2N>(X, t, sg);
+            if constexpr (G::T < 32) __syncwarp();   // the warp's two segments may have branched apart
             tmem::st32(xcol, reinterpret_cast<const float *>(X));
             tmem::wait_st();
         }

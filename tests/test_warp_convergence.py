@@ -34,7 +34,7 @@ def statements_after(call):
     return out
 
 
-@pytest.mark.parametrize("call", ["store"])
+@pytest.mark.parametrize("call", ["store", "spectrum"])
 def test_warp_meets_after_per_segment_code(call):
     found = statements_after(call)
     assert found
@@ -62,3 +62,20 @@ def test_batch_with_mixed_warps(per_n, nout):
     for s, h, y in zip(ss, hs, b.convolve([dev(s) for s in ss])):
         assert oracle.max_stream_rel_l2(y.cpu().numpy(), oracle.conv(s, h), oracle.stream_scale(s, h, y.shape[1])) <= 2e-6
     b.close()
+
+
+# inner segments beside the first, the last (full or ragged) and an idle one
+@pytest.mark.gpu
+@pytest.mark.parametrize("nout", [2, L, 2 * (L - 2), 5 * (L - 2), 6 * (L - 2) + 1, 7 * (L - 2) - 1])
+def test_derivative_with_mixed_warps(nout):
+    _build.build()
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    g = np.random.Generator(np.random.PCG64(nout))
+    s, h = synth.signal(g, nout + M - 1), synth.filters(g, F, M)
+    p = Plan(M, F, N)
+    p.set_filters(dev(h))
+    d = p.convolve_derivative(dev(s)).cpu().numpy()
+    y, ref, scale = oracle.conv(s, h), oracle.derivative(s, h), oracle.stream_scale(s, h, nout)
+    assert max(np.linalg.norm(d[f] - ref[f]) / max(np.linalg.norm(y[f]), scale[f]) for f in range(F)) <= 2e-6
+    p.close()
