@@ -100,6 +100,7 @@ __device__ __forceinline__ void append_candidates(bool hit, long long j, int f, 
                 cand[i] = c;
             }
         }
+        __syncwarp();       // the next filter's tensor-memory load is warp-wide
     }
 }
 

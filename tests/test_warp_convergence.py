@@ -42,6 +42,13 @@ def test_warp_meets_after_per_segment_code(call):
         assert nxt == "if constexpr (G::T < 32) __syncwarp();", (name, nxt)
 
 
+def test_warp_meets_after_candidate_records():
+    """Only the lanes with a candidate write a record."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(_build.CSRC, "ols_post.cu")).read())
+    record = re.search(r"cand\[i\] = c;([\s}]*)(\w+\(\);)?", text)
+    assert record and record.group(2) == "__syncwarp();"
+
+
 def dev(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
