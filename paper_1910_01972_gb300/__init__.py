@@ -410,9 +410,15 @@ class BatchPlan:
     def handle(self) -> int:
         return self._h
 
+    def _one_each(self, tensors, what):
+        # the library reads B pointers from each table, whatever the list's length
+        if len(tensors) != self.B:
+            raise ValueError("%d %s for a batch of %d problems" % (len(tensors), what, self.B))
+        return tensors
+
     def set_filters(self, hs) -> None:
         """hs: list of B device tensors [F[b]][M[b]] complex64."""
-        hs = [_input(h, "h[%d]" % b, self.device) for b, h in enumerate(hs)]
+        hs = self._one_each([_input(h, "h[%d]" % b, self.device) for b, h in enumerate(hs)], "filter banks")
         for b, h in enumerate(hs):
             if tuple(h.shape) != (self.F[b], self.M[b]):
                 raise ValueError("h[%d] must have shape [%d][%d]" % (b, self.F[b], self.M[b]))
@@ -436,12 +442,13 @@ class BatchPlan:
 
     def convolve(self, ss, ys=None):
         """ss: list of B device tensors [Ns[b]]; returns the list of outputs."""
-        ss = [_input(s, "s[%d]" % b, self.device) for b, s in enumerate(ss)]
+        ss = self._one_each([_input(s, "s[%d]" % b, self.device) for b, s in enumerate(ss)], "signals")
         for b, s in enumerate(ss):
             if s.shape != (self.Ns[b],):
                 raise ValueError("s[%d] must have %d samples" % (b, self.Ns[b]))
         if ys is None:
             ys = self.outputs()
+        self._one_each(ys, "outputs")
         for b, y in enumerate(ys):
             _output(y, "y[%d]" % b, self.device)
             if tuple(y.shape) != (self.F[b], self.Nout[b]):
