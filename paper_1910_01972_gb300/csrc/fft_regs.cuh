@@ -167,93 +167,6 @@ __device__ __forceinline__ void dft16(C *x) {
     for (int k = 0; k < 16; ++k) x[k] = y[k];
 }
 
-// The 16-point DFT of a twiddled pass with the pass's twiddle folded into the
-// butterflies.  A twiddled inverse DFT is the polynomial P(t) = sum_j x_j t^j
-// at t = w e^(2 pi i k / 16), k < 16 (w: the thread's twiddle), and splitting
-// P into even and odd powers four times gives radix-2 butterflies
-//   s = a + W b,  d = a - W b = 2 a - s,   W = w^h e^(2 pi i h k / 16), h = 8, 4, 2, 1,
-// with W = w^8; w^4 (and i w^4); w^2, w^2 e(2) (and i times them); w e(0..3)
-// (and i times them), e(m) = e^(2 pi i m / 16): eight distinct values per
-// pass, each held as (re, re, -im, -im) so that one packed multiply-add takes
-// re (or, for the rotated i W, im) for both components; two scalar ones add
-// the crossed terms.  Against a plain DFT-16 after 15 complex multiplies this
-// is 192 FP32 lane operations instead of 220 and 16 live twiddle registers
-// instead of 30.  PACKED: the difference as one packed multiply-add (128
-// instructions per DFT, plain form 172) or as two scalar ones (160), which
-// do not hold the packed pipe for two cycles: on 32- and 16-filter banks
-// scalar / packed measured 507 / 536 us at N = 2048, 224 / 230 at 1024,
-// 314 / 321 at 4096, 228 / 226 at 512 and 148 / 141 at 256, so only N = 256
-// packs.  d = 2 a - s shares the rounding error of s: the error of an inverse
-// FFT grows by about 10% (1.15e-7 to 1.27e-7 at N = 2048 in an FP32
-// simulation), that of a whole convolution by about 5%.
-template <bool ROT, bool PACKED>
-__device__ __forceinline__ void bfly_inv(float2 &a, float2 &b, const float *w) {
-    float2 s;
-    if constexpr (!ROT) {
-        const float2 u = __ffma2_rn(make_float2(w[0], w[1]), b, a);
-        s = make_float2(fmaf(w[2], b.y, u.x), fmaf(-w[2], b.x, u.y));
-    } else {        // W -> i W
-        const float2 u = __ffma2_rn(make_float2(w[2], w[3]), b, a);
-        s = make_float2(fmaf(-w[0], b.y, u.x), fmaf(w[0], b.x, u.y));
-    }
-    if constexpr (PACKED) b = __ffma2_rn(make_float2(2.f, 2.f), a, make_float2(-s.x, -s.y));
-    else b = make_float2(fmaf(2.f, a.x, -s.x), fmaf(2.f, a.y, -s.y));
-    a = s;
-}
-// The transposed butterfly of the forward pass: a + b and (a - b) conj(W).
-template <bool ROT>
-__device__ __forceinline__ void bfly_fwd(float2 &a, float2 &b, const float *w) {
-    const float2 d = csub(a, b);
-    a = cadd(a, b);
-    if constexpr (!ROT) {
-        const float2 u = __fmul2_rn(make_float2(w[0], w[1]), d);
-        b = make_float2(fmaf(-w[2], d.y, u.x), fmaf(w[2], d.x, u.y));
-    } else {        // conj(i W) = -i conj(W)
-        const float2 u = __fmul2_rn(make_float2(w[2], w[3]), d);
-        b = make_float2(fmaf(w[0], d.y, u.x), fmaf(-w[0], d.x, u.y));
-    }
-}
-
-// Stage h of the folded DFT-16 on x[0..15]; w: its distinct W, four words
-// each (h = 8 and 4: one, h = 2: two, h = 1: four).  Between the stages
-// register j * (16 / h) + k holds the partial sum of residue j at the k-th
-// of 16 / h points; the last inverse stage leaves output k in register k, and
-// the forward DFT is the same graph from the outputs back to the inputs.
-template <int H, bool PACKED>
-__device__ __forceinline__ void stage_inv(float2 *x, const float *w) {
-    constexpr int K = 8 / H;                 // points per residue before the stage
-    float2 y[16];
-#pragma unroll
-    for (int j = 0; j < H; ++j)
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            float2 a = x[j * K + k], b = x[(j + H) * K + k];
-            if (H * k >= 4) bfly_inv<true, PACKED>(a, b, w + 4 * (k - 4 / H));
-            else bfly_inv<false, PACKED>(a, b, w + 4 * k);
-            y[j * 2 * K + k] = a;
-            y[j * 2 * K + k + K] = b;
-        }
-#pragma unroll
-    for (int k = 0; k < 16; ++k) x[k] = y[k];
-}
-template <int H>
-__device__ __forceinline__ void stage_fwd(float2 *x, const float *w) {
-    constexpr int K = 8 / H;
-    float2 y[16];
-#pragma unroll
-    for (int j = 0; j < H; ++j)
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            float2 a = x[j * 2 * K + k], b = x[j * 2 * K + k + K];
-            if (H * k >= 4) bfly_fwd<true>(a, b, w + 4 * (k - 4 / H));
-            else bfly_fwd<false>(a, b, w + 4 * k);
-            y[j * K + k] = a;
-            y[(j + H) * K + k] = b;
-        }
-#pragma unroll
-    for (int k = 0; k < 16; ++k) x[k] = y[k];
-}
-
 // R-point DFT on each of the 16/R consecutive groups of x[0..15].
 template <int R, bool INV, class C>
 __device__ __forceinline__ void dft_groups(C *x) {

@@ -38,41 +38,33 @@ void spectral_order(int log2N, int32_t *nu) {
     }
 }
 
-// The plan's twiddle table: the forward twiddles of every pass (pp.twn
-// entries), then the folded factors of the TMEM-twiddle kernels (pp.tw8n).
-static std::vector<float2> twiddle_tables(const PassPlan &pp) {
-    // pass p < np-1: entry (k-1) s + n' = W_{16 s}^{n' k}, k in [1, 16), n' in [0, s)
-    std::vector<float2> tw((size_t)(pp.twn + pp.tw8n));
+// Twiddles of the forward passes, pp.twn entries: pass p < np-1, entry (k-1) s + n'
+// = W_{16 s}^{n' k}, k in [1, 16), n' in [0, s).
+static void append_twiddles(std::vector<float2> &tw, const PassPlan &pp) {
     for (int p = 0; p + 1 < pp.np; ++p) {
         const int s = pp.stride[p], B = 16 * s;
         for (int k = 1; k < 16; ++k)
             for (int n = 0; n < s; ++n) {
                 const long long e = ((long long)n * k) % B;
                 const double a = -2.0 * M_PI * (double)e / (double)B;
-                tw[(size_t)pp.tw_off[p] + (size_t)(k - 1) * s + n] =
-                    make_float2((float)std::cos(a), (float)std::sin(a));
+                tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
             }
     }
-    // N = 8192 runs as two 4096-point transforms (and one twiddle, below)
-    const PassPlan fp = pp.log2N == 13 ? make_pass_plan(12) : pp;
-    // folded factors (inverse sign): w^8; w^4; w^2, w^2 e(2); w, w e(1), w e(2),
-    // w e(3) with w = exp(2 pi i n' / (16 s)), e(m) = exp(2 pi i m / 16); row i
-    // of pass p at tw8_off[p] + i s + n'
-    static const int kPow[8] = {8, 4, 2, 2, 1, 1, 1, 1}, kRot[8] = {0, 0, 0, 2, 0, 1, 2, 3};
-    for (int p = 0; p + 1 < fp.np; ++p) {
-        const int s = fp.stride[p], B = 16 * s;
-        for (int i = 0; i < 8; ++i)
-            for (int n = 0; n < s; ++n) {
-                const double a = 2.0 * M_PI * (double)(kPow[i] * n + kRot[i] * s) / (double)B;
-                tw[(size_t)pp.twn + (size_t)fp.tw8_off[p] + (size_t)i * s + n] =
-                    make_float2((float)std::cos(a), (float)std::sin(a));
-            }
-    }
-    if (pp.log2N == 13)
-        for (int t = 0; t < 256; ++t) {
-            const double a = 2.0 * M_PI * (double)t / 8192.0;
-            tw[(size_t)(pp.twn + fp.tw8n + t)] = make_float2((float)std::cos(a), (float)std::sin(a));
+}
+
+// The plan's twiddle table: its own passes' and, at N = 8192, which the bank and
+// batch kernels run as two 4096-point transforms, those of N = 4096 and the odd
+// half's W_8192^n, n < 2048.
+static std::vector<float2> twiddle_tables(const PassPlan &pp) {
+    std::vector<float2> tw;
+    append_twiddles(tw, pp);
+    if (pp.log2N == 13) {
+        append_twiddles(tw, make_pass_plan(12));
+        for (int n = 0; n < 2048; ++n) {
+            const double a = -2.0 * M_PI * (double)n / 8192.0;
+            tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
         }
+    }
     return tw;
 }
 
@@ -317,7 +309,9 @@ int ols_plan(ols_plan_t *out, int64_t N, int32_t M, int32_t F, uint32_t flags) {
     if (e == cudaSuccess && !r2r) e = dev_alloc(&p->Htk, sizeof(float2) * (size_t)F * (size_t)N);
     if (e == cudaSuccess && r2r) e = dev_alloc(&p->hpack, sizeof(float2) * (size_t)Fc * (size_t)M);
     if (e == cudaSuccess && r2r) e = r2r_prepare(*p);
-    if (e == cudaSuccess) e = dev_alloc(&p->tw, sizeof(float2) * (size_t)(p->pp.twn + p->pp.tw8n + N / 2));
+    std::vector<float2> tw = twiddle_tables(p->pp);
+    const size_t ntw = (tw.size() + 1) & ~(size_t)1;         // the derivative's sines follow, read 16 bytes at a time
+    if (e == cudaSuccess) e = dev_alloc(&p->tw, sizeof(float2) * (ntw + (size_t)N));
     if (e == cudaSuccess) e = dev_alloc(&p->tw64, sizeof(double2) * (size_t)N);
     if (e == cudaSuccess) e = dev_alloc(&p->nu, sizeof(int32_t) * (size_t)N);
     if (e == cudaSuccess) e = dev_alloc(&p->d_status, sizeof(int));
@@ -341,16 +335,20 @@ int ols_plan(ols_plan_t *out, int64_t N, int32_t M, int32_t F, uint32_t flags) {
         if (e == cudaSuccess) e = tc_prepare(*p, bf16);
     }
     if (e == cudaSuccess) {
-        std::vector<float2> tw = twiddle_tables(p->pp);
-        p->tw8 = p->tw + p->pp.twn;
-        p->dsin = reinterpret_cast<const float *>(p->tw8 + p->pp.tw8n);
+        p->twb = l == 13 ? p->tw + p->pp.twn : p->tw;
+        p->dsin = reinterpret_cast<const float *>(p->tw + ntw);
+        tw.resize(ntw);
         std::vector<int32_t> nu((size_t)N);
         spectral_order(l, nu.data());
-        auto dsin = [&](int64_t q) {
+        // sin(2 pi nu / N) as hi + lo: one rounding in the product with the spectrum, not two
+        std::vector<float> sines((size_t)(2 * N));
+        for (int64_t q = 0; q < N; ++q) {
             const int f = p->layout == LAYOUT_STD ? nu[(size_t)q] : layout_freq(p->layout, (int)q);
-            return (float)std::sin(2.0 * M_PI * (double)f / (double)N);
-        };
-        for (int64_t q = 0; q < N; q += 2) tw.push_back(make_float2(dsin(q), dsin(q + 1)));
+            const double v = std::sin(2.0 * M_PI * (double)f / (double)N);
+            sines[(size_t)q] = (float)v;
+            sines[(size_t)(N + q)] = (float)(v - (double)(float)v);
+        }
+        for (int64_t q = 0; q < 2 * N; q += 2) tw.push_back(make_float2(sines[(size_t)q], sines[(size_t)(q + 1)]));
         e = cudaMemcpy(p->tw, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(p->nu, nu.data(), sizeof(int32_t) * nu.size(), cudaMemcpyHostToDevice);
     }

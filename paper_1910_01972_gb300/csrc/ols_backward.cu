@@ -127,8 +127,8 @@ ols_backward_kernel(const float2 *__restrict__ sig, long long Ns, const float2 *
     tmem::fence_before_sync();
     __syncthreads();
     tmem::fence_after_sync();
-    const TwPlain tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
-    tw_plain_fill<LOG2N>(twg, tw.base, t);
+    const TwTmem<LOG2N, XCHG_SMEM> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u};
+    tw_tmem_fill<LOG2N, XCHG_SMEM>(twg, tw.base, t);
     const uint32_t acol = tw.base + 96;
     const L2Hints l2 = L2Hints::make();
     const int lo = M - 1;

@@ -58,7 +58,7 @@ struct BankGeo {
 
 struct BankArgs {
     const float4 *Hk;       // [F][N] spectra in kernel layout
-    const float2 *tw8;      // folded twiddles
+    const float2 *tw;       // twiddles (N = 8192: of N = 4096)
     int F;                  // spectra per segment
     int n0;                 // circular position of a segment's first output
     long long step;         // outputs per segment
@@ -150,8 +150,8 @@ ols_bank_kernel(const BankArgs a, const EPI epi) {
     tmem::fence_before_sync();
     __syncthreads();
     tmem::fence_after_sync();
-    const TwTmemT<EPI::XCH> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(a.tw8, t)};
-    tw_tmem_fill<LOG2N, EPI::XCH>(a.tw8, tw.base, t);
+    const TwTmem<LOG2N, EPI::XCH> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(a.tw, t)};
+    tw_tmem_fill<LOG2N, EPI::XCH>(a.tw, tw.base, t);
     const uint32_t xcol = tw.base + 96;
 
     // this CTA's share of the steps

@@ -212,7 +212,7 @@ int measure_tiles(int32_t M, int32_t F, int64_t N, int block, int sm_count, int3
     if (e == cudaSuccess) e = cudaMemcpy(dp, &d, sizeof(d), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(ptrs, hp, sizeof(hp), cudaMemcpyHostToDevice);
     TwTables tw{};
-    tw.tw[l] = p->tw8;
+    tw.tw[l] = p->twb;
     double t_best = 1e300, t_of[4] = {0, 0, 0, 0};
     for (int c = 0; c < 4 && e == cudaSuccess; ++c) {
         const int R = kTileChoices[c];
@@ -418,7 +418,7 @@ int ols_batch_plan_tiles(ols_batch_t *out, int32_t B, const int64_t *Ns, const i
             d.index = b;
             d.log2N = l;
             d.status = bt->plans[b]->d_status;
-            bt->tw_all.tw[l] = bt->plans[b]->tw8;
+            bt->tw_all.tw[l] = bt->plans[b]->twb;
         }
         // tile schedule: tiles per item of each problem, given or tuned per
         // (M, F, N) for this block size; then, while the batch would have
@@ -531,7 +531,7 @@ int ols_batch_plan_tiles(ols_batch_t *out, int32_t B, const int64_t *Ns, const i
         }
         g.nitems = (long long)(items.size() - i0);
         g.grid = (int)std::min<long long>(g.nitems, cap);
-        g.tw = bt->plans[order[i]]->tw8;
+        g.tw = bt->plans[order[i]]->twb;
         bt->groups.push_back(g);
         ranges.push_back({p0, i0});
         i = j;

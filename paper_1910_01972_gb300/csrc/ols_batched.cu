@@ -35,7 +35,7 @@ ols_batched_kernel(const BatchProblemDev *__restrict__ probs, const int2 *__rest
     tmem::fence_before_sync();
     __syncthreads();
     tmem::fence_after_sync();
-    const TwTmem tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(twg, t)};
+    const TwTmem<LOG2N> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(twg, t)};
     tw_tmem_fill<LOG2N>(twg, tw.base, t);
     int xc = 0;
     for (;;) {
@@ -139,7 +139,7 @@ __device__ __noinline__ int batch_one_tile(const BatchProblemDev *__restrict__ p
         // the TMEM layout and exchange of the plain kernel, so results stay bitwise
         // those of per-problem calls; the twiddles are written on an item's first
         // tile only
-        const TwTmem twt{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(tw, t)};
+        const TwTmem<LOG2N> twt{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(tw, t)};
         if (fill) tw_tmem_fill<LOG2N>(tw, twt.base, t);
         ols_segment<LOG2N>(P, s_ptrs[P.index], y_ptrs[P.index], twt, seg, bufs, t, xc, bar);
     }

@@ -81,12 +81,6 @@ struct Geo {
     __host__ __device__ static constexpr int off(int k) {
         return LOG2N == 13 ? 256 * (k & 7) + 4096 * (k >> 3) : k * T;
     }
-    // folded-twiddle table (TMEM twiddles): 8 rows of stride(p) entries per pass
-    __host__ __device__ static constexpr int tw8_off(int p) {
-        int o = 0;
-        for (int i = 0; i < p; ++i) o += 8 * stride(i);
-        return o;
-    }
     // the exchange between the last two passes goes through TMEM (kernels
     // with TMEM twiddles; columns 64..95 of the thread's block are free)
     static constexpr bool TX = LOG2N >= 9 && LOG2N <= 12;
@@ -573,7 +567,7 @@ __device__ __forceinline__ void tx_inverse(float2 *x, uint32_t xb) {
 template <int LOG2N, int P, int XCH>
 __device__ __forceinline__ int tw_index(int t) {
     using G = Geo<LOG2N>;
-    if constexpr (XCH && G::TX && P == G::NP - 2) {   // the relabelled lanes holding p0 .. p(s-1)
+    if constexpr (XCH != XCHG_SMEM && G::TX && P == G::NP - 2) {   // the relabelled lanes holding p0 .. p(s-1)
         if constexpr (LOG2N == 11) return XCH == XCHG_SHFL ? ((t >> 3) & 3) + 4 * (t & 1) : (t >> 1) & 7;
         else if constexpr (LOG2N == 12) return (t & 3) + 4 * ((t >> 3) & 1) + 8 * ((t >> 4) & 1);
         else if constexpr (LOG2N == 10) return (t >> 3) & 3;
@@ -638,83 +632,76 @@ struct TwGlobal {
     }
 };
 
-// TwTmemT: the thread's own twiddles of every pass, preloaded into its TMEM
-// lane as the eight folded factors of stage_inv / stage_fwd (pass P at columns
-// 32 P .. 32 P + 31 of `base`, four columns each): no L1 traffic.  The last
-// stage's sixteen words are loaded while the other stages run.
-// XCH: the segment FFT also uses the TMEM exchange where Geo<>::TX allows it
-// (kernels whose epilogue needs the registers opt out).
-template <int XCH = XCHG_TMEM>
+// TwTmem: the thread's own 15 twiddles of every pass, preloaded into its TMEM
+// lane (pass P at columns 32 P .. 32 P + 29 of `base`): no L1 traffic.
+// XCH: the segment FFT also uses the TMEM exchange where Geo<>::TX allows it, and
+// N = 8192 runs as two halves (XCHG_SMEM: neither, the adjoint's form).
+// A pass takes its twiddles in one load, or (WORDS = 16) in two of eight, with 16
+// live registers instead of 30: at N = 512 and 8192 one load spills beside the next
+// filter's spectrum (plain form at 8192 52 bytes, 327 us against 324; the other lengths
+// 0.3 to 3% faster with one: power at 4096 188 / 194 us, plain at 2048 525.1 / 526.6).
+//
+// Tried and taken back: the twiddles folded into radix-2 butterflies s = a + W b,
+// d = 2 a - s, eight factors per pass and 192 FP32 lane operations per DFT-16 instead
+// of 220.  It was faster where the kernel is bound by FP32 issue (32 filters, 2^23
+// samples, N = 2048: 510 us against 525; real pairs 273 / 280; power at N = 4096 182 / 188;
+// N = 256, 512, 1024 and 8192 equal or slower), but d inherits the rounding of s and the
+// results' error against 64 bits grew by 4 to 8%; with d formed like s (256 operations,
+// more than the plain form) it still was up to 2% larger.
+template <int XCH, int WORDS>
 struct TwTmemT {
     static constexpr int xchg = XCH;
     uint32_t base;
-    float2 odd = {0.f, 0.f};         // N = 8192: exp(2 pi i (t mod 256) / 8192)
+    const float2 *odd = nullptr;     // N = 8192: W_8192^(256 j + t) at 256 j, t the thread of its half
     // columns 64..95: the staging area of the TMEM exchange
     __device__ __forceinline__ uint32_t xbase() const { return base + 64; }
     struct Fetched {
-        float v[16];
+        float v[WORDS];
+        uint32_t col;
     };
     template <int LOG2N, int P>
     __device__ __forceinline__ void fetch(Fetched &f, int) const {
-        tmem::ld16(base + 32 * P, f.v);
-    }
-    // inverse: twiddle and DFT-16 (f: fetched by fetch)
-    template <int LOG2N, int P>
-    __device__ __forceinline__ void dft_inv(float2 *x, Fetched &f) const {
-        float w1[16];
-        tmem::wait_ld16(f.v);
-        tmem::ld16(base + 32 * P + 16, w1);
-        stage_inv<8, LOG2N == 8>(x, f.v);
-        stage_inv<4, LOG2N == 8>(x, f.v + 4);
-        stage_inv<2, LOG2N == 8>(x, f.v + 8);
-        tmem::wait_ld16(w1);
-        stage_inv<1, LOG2N == 8>(x, w1);
-    }
-    // forward: DFT-16 and twiddle
-    template <int LOG2N, int P>
-    __device__ __forceinline__ void dft_fwd(float2 *x) const {
-        float w1[16], w8[16];
-        tmem::ld16(base + 32 * P + 16, w1);
-        tmem::wait_ld16(w1);
-        tmem::ld16(base + 32 * P, w8);
-        stage_fwd<1>(x, w1);
-        tmem::wait_ld16(w8);
-        stage_fwd<2>(x, w8 + 8);
-        stage_fwd<4>(x, w8 + 4);
-        stage_fwd<8>(x, w8);
-    }
-};
-
-// TwPlain: the thread's 15 twiddles of every pass in its TMEM lane (pass P at
-// columns 32 P .. 32 P + 29), applied by complex multiplies around a plain
-// DFT.  The adjoint's form: it transforms forward, where folding saves nothing
-// (a butterfly of (a - b) W is no multiply-add; folded 239 / 209 us for both
-// gradients / dh alone at N = 1024, plain 235 / 195; decimation in time with
-// folded butterflies 235 / 206, and it spills at N = 4096: 320 against 305).
-struct TwPlain {
-    uint32_t base;
-    struct Fetched {
-        float v[32];
-    };
-    template <int LOG2N, int P>
-    __device__ __forceinline__ void fetch(Fetched &f, int) const {
-        tmem::ld32(base + 32 * P, f.v);
+        f.col = base + 32 * P;
+        if constexpr (WORDS == 16) tmem::ld16(f.col, f.v);
+        else tmem::ld32(f.col, f.v);
     }
     template <bool INV>
-    __device__ __forceinline__ void apply(float2 *x, const Fetched &f) const {
-        tmem::wait_ld();
+    __device__ __forceinline__ void apply(float2 *x, Fetched &f) const {
+        if constexpr (WORDS == 16) {
+            float u[16];
+            tmem::wait_ld16(f.v);
+            tmem::ld16(f.col + 16, u);
 #pragma unroll
-        for (int k = 1; k < 16; ++k) x[k] = ctw<INV>(x[k], make_float2(f.v[2 * k - 2], f.v[2 * k - 1]));
+            for (int k = 1; k < 9; ++k) x[k] = ctw<INV>(x[k], make_float2(f.v[2 * k - 2], f.v[2 * k - 1]));
+            tmem::wait_ld16(u);
+#pragma unroll
+            for (int k = 9; k < 16; ++k) x[k] = ctw<INV>(x[k], make_float2(u[2 * k - 18], u[2 * k - 17]));
+        } else {
+            tmem::wait_ld();
+#pragma unroll
+            for (int k = 1; k < 16; ++k) x[k] = ctw<INV>(x[k], make_float2(f.v[2 * k - 2], f.v[2 * k - 1]));
+        }
     }
 };
+template <int LOG2N, int XCH = XCHG_TMEM>
+using TwTmem = TwTmemT<XCH, LOG2N == 9 || LOG2N == 13 ? 16 : 32>;
 
-// Fill a TwPlain for thread t from the plan's twiddle table.
-template <int LOG2N, int P = 0>
-__device__ __forceinline__ void tw_plain_fill(const float2 *tw, uint32_t base, int t) {
+// A kernel with the TMEM exchange (and N = 8192 as two halves)?
+template <class TW>
+struct tw_tx { static constexpr bool value = false; };
+template <int XCH, int WORDS>
+struct tw_tx<TwTmemT<XCH, WORDS>> { static constexpr bool value = XCH != XCHG_SMEM; };
+
+// Fill a TwTmem<LOG2N, XCH> for thread t from the plan's twiddle table (XCHG_SMEM: of
+// this N; else the bank kernels' table, which at N = 8192 is that of N = 4096).
+template <int LOG2N, int XCH = XCHG_TMEM, int P = 0>
+__device__ __forceinline__ void tw_tmem_fill(const float2 *tw, uint32_t base, int t) {
     using G = Geo<LOG2N>;
-    if constexpr (P < G::NP - 1) {
+    if constexpr (LOG2N == 13 && XCH != XCHG_SMEM) {
+        tw_tmem_fill<12, XCH>(tw, base, t & 255);       // two 4096-point transforms
+    } else if constexpr (P < G::NP - 1) {
         constexpr int s = G::stride(P);
-        const float2 *w = tw + G::tw_off(P) + t % s;
+        const float2 *w = tw + G::tw_off(P) + tw_index<LOG2N, P, XCH>(t);
         float v[32];
 #pragma unroll
         for (int k = 1; k < 16; ++k) {
@@ -724,54 +711,16 @@ __device__ __forceinline__ void tw_plain_fill(const float2 *tw, uint32_t base, i
         }
         v[30] = v[31] = 0.f;
         tmem::st32(base + 32 * P, v);
-        tw_plain_fill<LOG2N, P + 1>(tw, base, t);
+        tw_tmem_fill<LOG2N, XCH, P + 1>(tw, base, t);
     } else {
         tmem::wait_st();
     }
 }
 
-using TwTmem = TwTmemT<true>;
-template <class TW>
-struct is_tw_tmem : std::false_type {};
-template <int X>
-struct is_tw_tmem<TwTmemT<X>> : std::true_type {};
-template <class TW>
-__device__ __forceinline__ constexpr bool tw_xchg() {
-    if constexpr (is_tw_tmem<TW>::value) return TW::xchg != XCHG_SMEM;
-    else return false;
-}
-
-// Fill a TwTmemT<XCH> for thread t from the plan's folded-twiddle table (pass
-// P at offset tw8_off(P): eight rows of stride(P) entries, row i at n' holding
-// factor i of w = exp(2 pi i n' / (16 stride))).
-template <int LOG2N, int XCH = XCHG_TMEM, int P = 0>
-__device__ __forceinline__ void tw_tmem_fill(const float2 *tw8, uint32_t base, int t) {
-    using G = Geo<LOG2N>;
-    if constexpr (LOG2N == 13) {
-        tw_tmem_fill<12, XCH>(tw8, base, t & 255);      // two 4096-point transforms
-    } else if constexpr (P < G::NP - 1) {
-        constexpr int s = G::stride(P);
-        const float2 *w = tw8 + G::tw8_off(P) + tw_index<LOG2N, P, XCH>(t);
-        float v[32];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float2 wi = __ldg(w + i * s);
-            v[4 * i] = v[4 * i + 1] = wi.x;
-            v[4 * i + 2] = v[4 * i + 3] = -wi.y;
-        }
-        tmem::st32(base + 32 * P, v);
-        tw_tmem_fill<LOG2N, XCH, P + 1>(tw8, base, t);
-    } else {
-        tmem::wait_st();
-    }
-}
-
-// The twiddle that a thread keeps in registers (N = 8192; after the 4096-point
-// table of tw8).
+// The odd half's twiddles of thread t (N = 8192; they follow the 4096-point table).
 template <int LOG2N>
-__device__ __forceinline__ float2 tw_odd(const float2 *tw8, int t) {
-    if constexpr (LOG2N == 13) return __ldg(tw8 + Geo<12>::tw8_off(2) + (t & 255));
-    else return make_float2(0.f, 0.f);
+__device__ __forceinline__ const float2 *tw_odd(const float2 *tw, int t) {
+    return LOG2N == 13 ? tw + Geo<12>::TWN + (t & 255) : nullptr;
 }
 
 // One global-table twiddle step (fetch and apply back to back).
@@ -788,7 +737,7 @@ __device__ __forceinline__ void twiddle(float2 *x, const float2 *tw, int t) {
 // W_8192^n, n < 4096.  Threads 0..255 do the even half, 256..511 the odd one
 // (groups with barriers of their own), each with three radix-16 passes and the
 // TMEM exchange of N = 4096; four passes with three exchanges over 512 threads
-// took 358 us where this takes 319 (24 filters, 2^22 samples).  In the time domain a thread of group g holds
+// took 360 us where this takes 328 (24 filters, 2^22 samples).  In the time domain a thread of group g holds
 // n and n + 4096 for eight n = 256 (8 g + k) + t mod 256, so the butterfly is its
 // own, and half of its values go to the other group (swap_halves).
 // Shared memory: group g owns 8704 float2 at bufs + 8704 g: 4352 for the passes'
@@ -807,18 +756,21 @@ __device__ __forceinline__ void swap_halves(float2 *v, float2 *bufs, int t, int 
     for (int k = 0; k < 8; ++k) v[k] = hx[8704 * (g ^ 1) + 256 * k + tl];
     ++xc;
 }
-// x[j] *= (w e^{2 pi i j / 32})^(-1 forward, +1 inverse)
+// x[j] *= W_8192^n (inverse: its conjugate), n = 256 j + t; w + 256 j: from the table
+// (16 KB, L1), rounded once.  j + 8 is a quarter turn on from j, which is exact.  All
+// sixteen from the table took 340 us where this takes 328 (24 filters, 2^22 samples);
+// factors formed from W_8192^t and constants 324, but their rounding adds 5% to the
+// error of the results (2.04e-7 against 1.93e-7), and W_8192^t merged into the
+// twiddles of pass 0 took 348 with 2.01e-7.
 template <bool INV>
-__device__ __forceinline__ void odd_twiddle(float2 *x, float2 w) {
-    constexpr float c32[9] = {1.f, 0.98078528040323044f, 0.92387953251128674f, 0.83146961230254524f,
-                              0.70710678118654752f, 0.55557023301960218f, 0.38268343236508977f,
-                              0.19509032201612825f, 0.f};
+__device__ __forceinline__ void odd_twiddle(float2 *x, const float2 *w) {
+    float2 f[8];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {       // (each factor formed by itself: sharing those of j and j + 8 took 358 us
-        // where this takes 319, a longer live range each)
-        const float c = j <= 8 ? c32[j] : -c32[16 - j], s = j <= 8 ? c32[8 - j] : c32[j - 8];
-        const float2 wj = make_float2(fmaf(w.x, c, -w.y * s), fmaf(w.x, s, w.y * c));
-        x[j] = INV ? cmul(x[j], wj) : cmulc(x[j], wj);
+    for (int j = 0; j < 8; ++j) f[j] = __ldg(w + 256 * j);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        x[j] = ctw<INV>(x[j], f[j]);
+        x[j + 8] = ctw<INV>(rot_quarter<INV>(x[j + 8]), f[j]);
     }
 }
 template <int LOG2N, int P, class TW, class BAR = CtaBarrier>
@@ -885,18 +837,14 @@ template <int LOG2N, int P, class TW, class BAR>
 __device__ __forceinline__ void forward_passes(float2 *x, float2 *bufs, const TW &tw, int t, int &xc,
                                                const BAR &bar) {
     using G = Geo<LOG2N>;
-    if constexpr (LOG2N == 13 && is_tw_tmem<TW>::value) {
+    if constexpr (LOG2N == 13 && tw_tx<TW>::value) {
         forward13(x, bufs, tw, t, xc, bar);
     } else if constexpr (P < G::NP - 1) {
-        if constexpr (is_tw_tmem<TW>::value) {
-            tw.template dft_fwd<LOG2N, P>(x);
-        } else {
-            typename TW::Fetched f;
-            tw.template fetch<LOG2N, P>(f, t);        // in flight during the DFT
-            dft_groups<G::radix(P), false>(x);
-            tw.template apply<false>(x, f);
-        }
-        constexpr bool tx = G::TX && tw_xchg<TW>();
+        typename TW::Fetched f;
+        tw.template fetch<LOG2N, P>(f, t);            // in flight during the DFT
+        dft_groups<G::radix(P), false>(x);
+        tw.template apply<false>(x, f);
+        constexpr bool tx = G::TX && tw_tx<TW>::value;
         if constexpr (tx && P == G::NP - 2) {
             tx_forward<LOG2N, TW::xchg>(x, tw.xbase());
         } else {
@@ -921,15 +869,15 @@ template <int LOG2N, int P, class TW, class BAR>
 __device__ __forceinline__ void inverse_passes(float2 *x, float2 *bufs, const TW &tw, int t, int &xc,
                                                const BAR &bar) {
     using G = Geo<LOG2N>;
-    if constexpr (LOG2N == 13 && is_tw_tmem<TW>::value) {
+    if constexpr (LOG2N == 13 && tw_tx<TW>::value) {
         inverse13(x, bufs, tw, t, xc, bar);
-        return;
-    } else if constexpr (P < G::NP - 1) {
+    } else {
+    if constexpr (P < G::NP - 1) {
         typename TW::Fetched f;
         // in flight during the exchange, except TMEM twiddles before the TMEM
         // exchange (their registers then are not live across it: with them the
         // kernel spills)
-        constexpr bool tx = G::TX && tw_xchg<TW>();
+        constexpr bool tx = G::TX && tw_tx<TW>::value;
         constexpr bool late = tx && P == G::NP - 2;
         if constexpr (!late) tw.template fetch<LOG2N, P>(f, t);
         if constexpr (tx && P == G::NP - 2) {
@@ -941,16 +889,11 @@ __device__ __forceinline__ void inverse_passes(float2 *x, float2 *bufs, const TW
             ++xc;
         }
         if constexpr (late) tw.template fetch<LOG2N, P>(f, t);
-        if constexpr (is_tw_tmem<TW>::value) {
-            tw.template dft_inv<LOG2N, P>(x, f);
-        } else {
-            tw.template apply<true>(x, f);
-            dft_groups<G::radix(P), true>(x);
-        }
-    } else {
-        dft_groups<G::radix(P), true>(x);
+        tw.template apply<true>(x, f);
     }
-    if constexpr (P > 0 && !(LOG2N == 13 && is_tw_tmem<TW>::value)) inverse_passes<LOG2N, P - 1>(x, bufs, tw, t, xc, bar);
+    dft_groups<G::radix(P), true>(x);
+    if constexpr (P > 0) inverse_passes<LOG2N, P - 1>(x, bufs, tw, t, xc, bar);
+    }
 }
 template <int LOG2N, int P>
 __device__ __forceinline__ void inverse_passes(float2 *x, float2 *bufs, const float2 *tw, int t, int &xc) {

@@ -14,7 +14,7 @@ cudaError_t launch_forward(const ols_plan_s &p, const float2 *s, int64_t Ns, flo
                            int64_t nseg, int64_t Nout, cudaStream_t st, int *launches) {
     BankArgs a{};
     a.Hk = reinterpret_cast<const float4 *>(p.Hk);
-    a.tw8 = p.tw8;
+    a.tw = p.twb;
     a.F = p.F;
     a.n0 = p.M - 1;
     a.step = L;
@@ -35,19 +35,14 @@ PassPlan make_pass_plan(int log2N) {
     pp.T = pp.N / 16;
     pp.np = (log2N + 3) / 4;
     const int rl = (log2N % 4) ? (1 << (log2N % 4)) : 16;
-    int off = 0, off8 = 0;
+    int off = 0;
     for (int p = 0; p < pp.np; ++p) {
         pp.radix[p] = (p == pp.np - 1) ? rl : 16;
         pp.stride[p] = (p == pp.np - 1) ? 1 : (pp.N >> (4 * (p + 1)));
         pp.tw_off[p] = off;
-        pp.tw8_off[p] = off8;
-        if (p < pp.np - 1) {
-            off += 15 * pp.stride[p];
-            off8 += 8 * pp.stride[p];
-        }
+        if (p < pp.np - 1) off += 15 * pp.stride[p];
     }
     pp.twn = off;
-    pp.tw8n = log2N == 13 ? 8 * (256 + 16) + 256 : off8;   // N = 8192: two 4096-point transforms
     return pp;
 }
 

@@ -26,8 +26,6 @@ struct PassPlan {
     int stride[4];
     int tw_off[4];
     int twn;     // twiddle entries of passes 0 .. np-2
-    int tw8_off[4];
-    int tw8n;    // folded-twiddle entries (8 per stride position) of those passes
 };
 PassPlan make_pass_plan(int log2N);
 
@@ -127,9 +125,9 @@ struct ols_plan_s {
     ols::PassPlan pp{};
     float2 *Hk = nullptr;        // [F][N] spectra in kernel layout (FP32)
     float2 *Htk = nullptr;       // [F][N] spectra of conj(h_f[M-1-k]) (adjoint), kernel layout
-    float2 *tw = nullptr;        // forward twiddles (FP32), pp.twn entries, then the folded ones
-    const float *dsin = nullptr; // sin(2 pi nu / N) at each storage position (derivative): after tw8
-    const float2 *tw8 = nullptr; // folded twiddles of the TMEM-twiddle kernels: tw + pp.twn (pp.tw8n entries)
+    float2 *tw = nullptr;        // forward twiddles (FP32), pp.twn entries; N = 8192: then twb
+    const float *dsin = nullptr; // sin(2 pi nu / N) at each storage position (derivative): after the twiddles
+    const float2 *twb = nullptr; // twiddles of the bank and batch kernels: tw, or (N = 8192) those of N = 4096 and the odd half's
     double2 *tw64 = nullptr;     // W_N^m, m in [0, N) (FP64)
     int32_t *nu = nullptr;       // spectral order (device copy)
     int last_launches = 0;
@@ -169,7 +167,7 @@ struct BatchProblemDev {
     int *status;          // the problem's plan status word (bounds checks of OLS_CHECK builds)
 };
 
-// Folded-twiddle tables of every segment length, by log2 N (single-launch batches).
+// Twiddle tables (twb) of every segment length, by log2 N (single-launch batches).
 struct TwTables {
     const float2 *tw[kMaxLog2N + 1];
 };

@@ -119,7 +119,7 @@ struct EpiPost {
     ols_candidate *cand;
     unsigned long long *count;
     long long cap;
-    const float *dsin;              // DERIV: sin(2 pi nu / N) at each storage position
+    const float *dsin;              // DERIV: sin(2 pi nu / N) at each storage position, then its rounding errors
     __device__ __forceinline__ float2 sample(long long i) const { return __ldg(sig + i); }
     // DERIV: central differences of a circular sequence are the product of its
     // spectrum with i sin(2 pi nu / N).  The segment's spectrum is scaled once
@@ -138,13 +138,16 @@ struct EpiPost {
         if constexpr (MODE == POST_DERIV) {
             if (!at_end(sg)) {
                 const float4 *p = reinterpret_cast<const float4 *>(dsin) + 4 * t;
+                auto scale = [](float2 &x, float s, float r) {
+                    x = make_float2(fmaf(-s, x.y, -r * x.y), fmaf(s, x.x, r * x.x));
+                };
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const float4 s = __ldg(p + q);
-                    X[4 * q] = make_float2(-s.x * X[4 * q].y, s.x * X[4 * q].x);
-                    X[4 * q + 1] = make_float2(-s.y * X[4 * q + 1].y, s.y * X[4 * q + 1].x);
-                    X[4 * q + 2] = make_float2(-s.z * X[4 * q + 2].y, s.z * X[4 * q + 2].x);
-                    X[4 * q + 3] = make_float2(-s.w * X[4 * q + 3].y, s.w * X[4 * q + 3].x);
+                    const float4 s = __ldg(p + q), r = __ldg(p + q + Geo<LOG2N>::N / 4);
+                    scale(X[4 * q], s.x, r.x);
+                    scale(X[4 * q + 1], s.y, r.y);
+                    scale(X[4 * q + 2], s.z, r.z);
+                    scale(X[4 * q + 3], s.w, r.w);
                 }
             }
         }
@@ -267,7 +270,7 @@ static cudaError_t post_launch_mode(const ols_plan_s &p, const PostArgs &a, cuda
     constexpr bool NEIGH = MODE == POST_DERIV || MODE == POST_PEAK;
     BankArgs b{};
     b.Hk = reinterpret_cast<const float4 *>(p.Hk);
-    b.tw8 = p.tw8;
+    b.tw = p.twb;
     b.F = p.F;
     b.n0 = NEIGH ? p.M : p.M - 1;
     b.step = a.step;

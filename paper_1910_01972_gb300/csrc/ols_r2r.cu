@@ -89,7 +89,7 @@ cudaError_t r2r_launch(const ols_plan_s &p, const float *s, int64_t Ns, float *y
                        int64_t Nout, cudaStream_t st) {
     BankArgs a{};
     a.Hk = reinterpret_cast<const float4 *>(p.Hk);
-    a.tw8 = p.tw8;
+    a.tw = p.twb;
     a.F = (p.F + 1) / 2;
     a.n0 = p.M - 1;
     a.step = L;
