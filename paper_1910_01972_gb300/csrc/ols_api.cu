@@ -107,7 +107,7 @@ static std::vector<uint16_t> tc_dft16_tables(bool bf16) {
 // Tables of ols_tc64.cu: the inverse DFT-64 as the real 128 x 128 matrix [[C, S],
 // [-S, C]] (rows: Re, Im of the input; columns: Re, Im of the output), split in
 // 16-bit hi and lo parts (element (k, n) at byte (k/8) 2048 + (n/8) 128 + (n%8) 16
-// + (k%8) 2), then the twiddles e(n2 nu1 / 4096) / 8 as float2, points (n2 = 16 q +
+// + (k%8) 2), then the twiddles e(n2 nu1 / 4096) as float2, points (n2 = 16 q +
 // 2 i, + 1) of row nu1 at float4 index i 256 + 64 q + nu1.
 static std::vector<uint16_t> tc64_tables(bool bf16) {
     std::vector<uint16_t> out(2 * 128 * 128 + 4096 * 4);
@@ -135,7 +135,7 @@ static std::vector<uint16_t> tc64_tables(bool bf16) {
     for (int n2 = 0; n2 < 64; ++n2)
         for (int nu1 = 0; nu1 < 64; ++nu1) {
             const double th = 2.0 * M_PI * (double)(n2 * nu1) / 4096.0;
-            const float w[2] = {(float)(std::cos(th) / 8.0), (float)(std::sin(th) / 8.0)};
+            const float w[2] = {(float)std::cos(th), (float)std::sin(th)};
             const int q = n2 / 16, i = (n2 % 16) / 2;
             std::memcpy(&out[2 * 128 * 128 + ((i * 256 + 64 * q + nu1) * 4 + 2 * (n2 & 1)) * 2], w, sizeof(w));
         }

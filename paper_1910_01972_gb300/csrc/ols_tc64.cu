@@ -33,11 +33,16 @@
 // store, wait and exchange three times, and their threads' work bounds them:
 // 64 filters, 2^22 samples 1156 us there, 733 here (FP16; the FP32 kernel 620).
 // Spectra prefetched a filter ahead 761 us: their registers spill.
-// Scales (exact powers of two): spectra of the segment x 16 (|Y| <= 2.9 for |s| <=
-// 1.42, unit-L2 filters and M <= N), stage 2's operand x 2 (|Z| <= 23).  They give
-// FP16 operands the range of ols_tc.cu: a tone of |s| = 64 in its matched filter
-// comes through (x 512 it overflowed from |s| = 4 on, with the same error at
-// |s| <= 1.42: 6.8e-7).
+// Scale (an exact power of two): the segment's spectrum x 16, undone in the output.
+// Both inverse operands, Y and Z, are averages of phase-rotated outputs of the
+// segment's circular convolution, so |Y|, |Z| <= |s| sqrt(M) for a unit-L2 filter (a
+// tone in its matched filter reaches it): at most 16 x 1.42 x 64 = 1454 for |s| <= 1.42, and FP16's
+// 65504 from |s| sqrt(M) = 4094 on (x 512: from 128 on).  The forward transform's
+// second operand is at most 64 |s|.  At the other end FP16 runs out of bits below
+// 2^-14.  Errors (1e-6) of uniform signals of amplitude 2^-10, 2^-6, 2^-3 and 1 through random
+// filters: 130, 8, 1.2, 0.68 (stage 2's operands at an eighth of this: 180, 11, 1.5, 0.69; the
+// radix-16 form 210, 13, 2.1, 1.2); of a tone of 2^-10 in its matched filter (M = 512), against
+// the samples as split: 1.3 (2.2; 2.6).  The split itself costs that tone 2.5.
 // Waits are bounded as in ols_tc.cu.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -343,11 +348,11 @@ ols_tc64_kernel(const float2 *__restrict__ sig, const uint32_t *__restrict__ sig
                 ok = wait_done(bars, 1, phase, wait_limit, status);
                 if (!ok) break;
                 load_d(X, lane, 1, q);
-                // conjugate back; x 8 undoes the twiddles' 1/8, x 16 is the spectrum's scale
+                // conjugate back, x 16: the spectrum's scale
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
-                    xs[512 * i] = make_float4(X[2 * i].x * 128.f, X[2 * i].y * -128.f, X[2 * i + 1].x * 128.f,
-                                              X[2 * i + 1].y * -128.f);
+                    xs[512 * i] = make_float4(X[2 * i].x * 16.f, X[2 * i].y * -16.f, X[2 * i + 1].x * 16.f,
+                                              X[2 * i + 1].y * -16.f);
             }
             const long long rem = active ? Nout - start : 0;
             const int span = (int)(rem < L ? rem : L);
@@ -398,7 +403,7 @@ ols_tc64_kernel(const float2 *__restrict__ sig, const uint32_t *__restrict__ sig
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
                         if ((unsigned)(v0 + 64 * j) < (unsigned)span && in_bounds(start + v0 + 64 * j < Nout, status))
-                            __stcs(dst + 64 * j, make_float2(z[j].x * 0.5f, z[j].y * 0.5f));
+                            __stcs(dst + 64 * j, make_float2(z[j].x * 0.0625f, z[j].y * 0.0625f));
                 }
             }
         }

@@ -60,3 +60,30 @@ def test_range_of_a_matched_tone(M, amplitude):
     assert p.status() == 0
     assert oracle.rel_l2(y, oracle.conv(s, h)) <= BOUND[_native.OLS_FLAG_TC_FP16SPLIT]
     p.close()
+
+
+# relative error (1e-6) of the radix-16 form on the same tones
+FAINT = [(2.0 ** -10, 16, 9.32), (2.0 ** -10, 64, 4.95), (2.0 ** -10, 512, 2.62), (2.0 ** -10, 4000, 0.84),
+         (2.0 ** -8, 16, 2.31), (2.0 ** -8, 512, 0.90)]
+
+
+@pytest.mark.parametrize("amplitude,M,figure", FAINT)
+def test_faint_matched_tone(amplitude, M, figure):
+    """FP16 parts below 2^-14 lose bits: the operands between the stages must not lose more of a faint
+    signal than those of the radix-16 form did.  Against the samples as split, so that the rounding of
+    the split itself, the same for both, neither adds nor cancels."""
+    _build.build()
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    w = 2.0 * np.pi * 37 / 4096
+    s = (amplitude * np.exp(1j * w * np.arange(3 * 4096))).astype(np.complex64)
+    x = s.view(np.float32)
+    hi = x.astype(np.float16).astype(np.float32)
+    split = (hi + (x - hi).astype(np.float16).astype(np.float32)).view(np.complex64)
+    h = (np.exp(1j * w * np.arange(M)) / np.sqrt(M)).astype(np.complex64)[None]
+    p = Plan(M, 1, 4096, flags=_native.OLS_FLAG_TC_FP16SPLIT)
+    p.set_filters(dev(h))
+    y = p.convolve(dev(s)).cpu().numpy()
+    assert p.status() == 0
+    assert oracle.rel_l2(y, oracle.conv(split, h)) <= 1e-6 * figure
+    p.close()
