@@ -79,6 +79,8 @@ struct BankSegment {
 
 // y[f][j] written once, the aliased samples dropped.
 struct EpiPlain {
+    template <int LOG2N>
+    static constexpr bool narrow() { return false; }
     static constexpr int XCH = XCHG_TMEM;
     template <int LOG2N>
     static constexpr int edge() { return 0; }
@@ -150,7 +152,7 @@ ols_bank_kernel(const BankArgs a, const EPI epi) {
     tmem::fence_before_sync();
     __syncthreads();
     tmem::fence_after_sync();
-    const TwTmem<LOG2N, EPI::XCH> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(a.tw, t)};
+    const TwTmem<LOG2N, EPI::XCH, EPI::template narrow<LOG2N>()> tw{tbase + tmem::lane_bits() + (uint32_t)(threadIdx.x / 128) * 128u, tw_odd<LOG2N>(a.tw, t)};
     tw_tmem_fill<LOG2N, EPI::XCH>(a.tw, tw.base, t);
     const uint32_t xcol = tw.base + 96;
 

@@ -638,8 +638,10 @@ struct TwGlobal {
 // N = 8192 runs as two halves (XCHG_SMEM: neither, the adjoint's form).
 // A pass takes its twiddles in one load, or (WORDS = 16) in two of eight, with 16
 // live registers instead of 30: at N = 512 and 8192 one load spills beside the next
-// filter's spectrum (plain form at 8192 52 bytes, 327 us against 324; the other lengths
-// 0.3 to 3% faster with one: power at 4096 188 / 194 us, plain at 2048 525.1 / 526.6).
+// filter's spectrum (plain form at 8192 52 bytes, 327 us against 324), and so do some
+// epilogues elsewhere (NARROW: derivative at 4096, 8 filters, 2e6 samples, 58.7 / 51.9 us);
+// the others are 0.3 to 3% faster with one (power at 4096 194 / 188 us, plain at
+// 2048 526.6 / 525.1).
 //
 // Tried and taken back: the twiddles folded into radix-2 butterflies s = a + W b,
 // d = 2 a - s, eight factors per pass and 192 FP32 lane operations per DFT-16 instead
@@ -683,8 +685,8 @@ struct TwTmemT {
         }
     }
 };
-template <int LOG2N, int XCH = XCHG_TMEM>
-using TwTmem = TwTmemT<XCH, LOG2N == 9 || LOG2N == 13 ? 16 : 32>;
+template <int LOG2N, int XCH = XCHG_TMEM, bool NARROW = false>
+using TwTmem = TwTmemT<XCH, NARROW || LOG2N == 9 || LOG2N == 13 ? 16 : 32>;
 
 // A kernel with the TMEM exchange (and N = 8192 as two halves)?
 template <class TW>

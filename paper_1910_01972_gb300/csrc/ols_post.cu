@@ -104,8 +104,58 @@ __device__ __forceinline__ void append_candidates(bool hit, long long j, int f, 
     }
 }
 
+// DERIV, a segment at an end of the stream (called by its own threads): y in
+// circular order to the exchange buffer `buf`, padded q -> q + q/16; then each
+// output reads its two neighbours, the one-sided ends at j = 0 and j = Nout - 1.
+// drow: the filter's row of d.
+template <int LOG2N, class BAR>
+__device__ __forceinline__ void derivative_exchange(const float2 *x, float2 *drow, float2 *buf, int t,
+                                                    const BankSegment &sg, const BAR &bar) {
+    using G = Geo<LOG2N>;
+    if constexpr (LOG2N == 13) bar();             // the buffers of both halves, free between two barriers
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const int n = G::base(t) + G::off(k);
+        buf[n + (n >> 4)] = x[k];
+    }
+    bar();
+    float2 *dst = drow + (sg.j0 - sg.n0);
+    // circular positions of outputs j = 0 and j = Nout-1, if in this segment
+    const int n_first = sg.j0 == 0 ? sg.n0 : -2;
+    const int n_last = (sg.Nout - sg.j0 == (long long)sg.span) ? sg.span - 1 + sg.n0 : -2;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const int n = G::base(t) + G::off(k);
+        if ((unsigned)(n - sg.n0) < (unsigned)sg.span &&
+            in_bounds(sg.j0 - sg.n0 + n < sg.Nout && n >= 1 && n + 1 < G::N, sg.status)) {
+            const int lo = (n == n_first) ? n : n - 1;
+            const int hi = (n == n_last) ? n : n + 1;
+            const float sc = (lo == n || hi == n) ? 1.f : 0.5f;
+            const float2 a = buf[lo + (lo >> 4)], b = buf[hi + (hi >> 4)];
+            __stcs(dst + n, make_float2((b.x - a.x) * sc, (b.y - a.y) * sc));
+        }
+    }
+    if constexpr (LOG2N == 13) bar();
+}
+// The same as a call, which takes the two end segments' code and registers out of
+// the loop that all others run: at N = 512 .. 2048 the loop spills 90 to 110 bytes with
+// the code inline and nothing with the call (16 filters, 2^22 samples, N = 1024: 141
+// -> 132 us; 3 filters, 300,000 samples, N = 512 / 1024 / 2048: 9.4 / 9.9 / 9.8 -> 8.4 / 8.7 / 9.6).
+// At N = 256, 4096 and 8192 the call was slower (8 filters, 2e6 samples: 35.5 -> 36.1, 51.9 ->
+// 55.2, 75.2 -> 81.7).
+template <int LOG2N, class BAR>
+__device__ __noinline__ void derivative_exchange_call(const float2 *x, float2 *drow, float2 *buf, int t, BankSegment sg,
+                                                      BAR bar) {
+    derivative_exchange<LOG2N>(x, drow, buf, t, sg, bar);
+}
+
 template <int MODE>
 struct EpiPost {
+    // two loads of twiddles where one spills
+    template <int LOG2N>
+    static constexpr bool narrow() {
+        return (MODE == POST_DERIV && LOG2N >= 10) || (MODE == POST_PEAK && LOG2N == 12);
+    }
     // POWER: one of the exchange's three bits by shuffles (as the real form)
     static constexpr int XCH = MODE == POST_POWER ? XCHG_SHFL : XCHG_TMEM;
     // PEAK: warp-edge powers [2][T/32][16] floats per segment of several warps
@@ -222,35 +272,17 @@ struct EpiPost {
                 if ((unsigned)(v + G::off(k)) < (unsigned)sg.span && in_bounds(sg.j0 + v + G::off(k) < sg.Nout, sg.status))
                     __stcs(dst + G::off(k), x[k]);
         } else {
-            // y (circular order) to the exchange buffer not in use, padded q -> q + q/16;
-            // then each output reads its two neighbours
-            // (N = 8192: the buffers of both halves, free between two barriers)
-            float2 *dbuf = LOG2N == 13 ? bufs : bufs + (xc & 1) * G::PADN;
-            if constexpr (LOG2N == 13) bar();
-            else ++xc;
+            float2 *drow = static_cast<float2 *>(out) + (size_t)f * (size_t)sg.Nout;
+            float2 *buf = LOG2N == 13 ? bufs : bufs + (xc & 1) * G::PADN;      // not in use
+            if constexpr (LOG2N != 13) ++xc;
+            if constexpr (LOG2N >= 9 && LOG2N <= 11) {
+                float2 y[16];
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const int n = G::base(t) + G::off(k);
-                dbuf[n + (n >> 4)] = x[k];
+                for (int k = 0; k < 16; ++k) y[k] = x[k];
+                derivative_exchange_call<LOG2N>(y, drow, buf, t, sg, bar);
+            } else {
+                derivative_exchange<LOG2N>(x, drow, buf, t, sg, bar);
             }
-            bar();
-            float2 *dst = static_cast<float2 *>(out) + (size_t)f * (size_t)sg.Nout + (sg.j0 - sg.n0);
-            // circular positions of outputs j = 0 and j = Nout-1 (one-sided ends), if in this segment
-            const int n_first = sg.j0 == 0 ? sg.n0 : -2;
-            const int n_last = (sg.Nout - sg.j0 == (long long)sg.span) ? sg.span - 1 + sg.n0 : -2;
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const int n = G::base(t) + G::off(k);
-                if ((unsigned)(n - sg.n0) < (unsigned)sg.span &&
-                    in_bounds(sg.j0 - sg.n0 + n < sg.Nout && n >= 1 && n + 1 < G::N, sg.status)) {
-                    const int lo = (n == n_first) ? n : n - 1;
-                    const int hi = (n == n_last) ? n : n + 1;
-                    const float sc = (lo == n || hi == n) ? 1.f : 0.5f;
-                    const float2 a = dbuf[lo + (lo >> 4)], b = dbuf[hi + (hi >> 4)];
-                    __stcs(dst + n, make_float2((b.x - a.x) * sc, (b.y - a.y) * sc));
-                }
-            }
-            if constexpr (LOG2N == 13) bar();
         }
     }
 };

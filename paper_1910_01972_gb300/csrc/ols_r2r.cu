@@ -48,6 +48,8 @@ cudaError_t launch_pack_real_pairs(const float *h, int M, int F, float2 *g, cuda
 // Real samples in, one inverse FFT per filter pair, its real and imaginary
 // parts stored as the pair's two output rows.
 struct EpiReal {
+    template <int LOG2N>
+    static constexpr bool narrow() { return false; }
     static constexpr int XCH = XCHG_SHFL;
     template <int LOG2N>
     static constexpr int edge() { return 0; }
