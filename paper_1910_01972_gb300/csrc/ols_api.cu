@@ -690,7 +690,7 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 static void backward_layout(const ols_plan_s &p, int64_t nseg, bool want_ds, bool want_dh, size_t *edge_bytes,
                             size_t *part_bytes, size_t *sum_bytes, int *grid, int *block) {
-    *grid = backward_grid(p, nseg, block);
+    *grid = backward_grid(p, nseg, want_dh, block);
     *edge_bytes = want_ds ? align256(sizeof(float2) * (size_t)nseg * 2 * (size_t)(p.M - 1)) : 0;
     const size_t spec = sizeof(float2) * (size_t)p.F * (size_t)p.N;
     *part_bytes = want_dh ? align256(spec * (size_t)(*grid)) : 0;

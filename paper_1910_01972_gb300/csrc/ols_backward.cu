@@ -405,17 +405,31 @@ cudaError_t prepare_backward(ols_plan_s &p) {
 // stay within 16 MB: a block runs its windows' F + 2 transforms in a row, so
 // more blocks of fewer windows finish sooner (F = 8: 45 windows of N = 512 in
 // 12 blocks instead of 3 43 -> 27 us, 37 of N = 1024 in 19 instead of 10 31 ->
-// 27 us).  A small-block call whose whole workspace (both gradients) would not
+// 27 us).  With dh the finishing kernel has up to four times as many partial spectra to
+// sum, so the blocks per SM are limited by the filters, whose transforms have to
+// pay for it.  Time of both gradients with small blocks over that with large ones, by
+// small blocks (152 SMs), for 1 / 4 / 16 filters (2 filters at 228: .99, .95, 1.10, .89, 1.12):
+//   blocks        114                152                304                456
+//   N = 256   .90 / .77 / .59    .97 / .82 / .61   1.17 / .99 / .75   1.36 / 1.18 / .92
+//   N = 512   .86 / .72 / .55    .94 / .77 / .58   1.10 / .94 /  -    1.30 / 1.15 /  -
+//   N = 1024  .97 / .89 / .83   1.06 / .95 /  -    1.17 / 1.10 /  -   1.15 / 1.04 /  -
+//   N = 2048  .82 / .65 /  -     .89 / .69 /  -    1.05 /  -  /  -    1.25 /  -  /  -
+//   N = 4096  .84 / .83 /  -     .88 /  -  /  -    1.11 /  -  /  -      -
+// and dh alone is at most .05 above; ds alone gains at every size (.49 to .98).
+// A small-block call whose whole workspace (both gradients) would not
 // fit OLS_NOALLOC_SCRATCH_BYTES keeps the large blocks (filters nearly as long
 // as the segment have edges of up to 20 MB): the rule makes no call too large for
-// that scratch.  It looks neither at the gradients wanted nor at the entry point.
-int backward_grid(const ols_plan_s &p, int64_t nseg, int *block) {
+// that scratch.
+int backward_grid(const ols_plan_s &p, int64_t nseg, bool want_dh, int *block) {
     const int T = p.pp.T, large = p.log2N == 10 ? 256 : 512, small = T > 128 ? T : 128;
     const int64_t gs = (nseg + small / T - 1) / (small / T), gl = (nseg + large / T - 1) / (large / T);
     const int64_t spec = (int64_t)sizeof(float2) * p.F * p.N;
     const int64_t edges = (int64_t)sizeof(float2) * nseg * 2 * (p.M - 1);
     const int64_t need = edges + (gs + 1) * spec + 3 * 256;       // each part rounded up to 256 bytes
-    if (small < large && gs > gl && gs <= (int64_t)(512 / small) * p.sm_count && gs * spec <= (int64_t)16 << 20 &&
+    int quarters = 4 * (512 / small);                             // quarters of a block per SM
+    if (want_dh && large / small < 4) quarters = p.log2N == 10 && p.F == 1 ? 3 : 4;
+    else if (want_dh) quarters = p.F >= 16 ? 12 : p.F >= 4 ? 8 : p.F >= 2 && p.log2N > 8 ? 6 : 4;
+    if (small < large && gs > gl && 4 * gs <= (int64_t)quarters * p.sm_count && gs * spec <= (int64_t)16 << 20 &&
         need <= (int64_t)OLS_NOALLOC_SCRATCH_BYTES) {
         *block = small;
         return (int)gs;

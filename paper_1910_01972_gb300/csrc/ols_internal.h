@@ -247,7 +247,7 @@ int backward_validate(ols_plan_t plan, const float *s, int64_t Ns, const float *
 cudaError_t prepare_backward(ols_plan_s &p);
 cudaError_t launch_backward(const ols_plan_s &p, const BackwardArgs &a, cudaStream_t st, int *launches);
 // Block size and grid of the adjoints window kernel for nseg windows.
-int backward_grid(const ols_plan_s &p, int64_t nseg, int *block);
+int backward_grid(const ols_plan_s &p, int64_t nseg, bool want_dh, int *block);
 // FP64 precompute kernels.  Htk (may be null): the spectra of conj(h_f[M-1-k]),
 // always in the standard layout.
 cudaError_t launch_tw64(double2 *tw64, int N, cudaStream_t st);
