@@ -38,34 +38,63 @@ void spectral_order(int log2N, int32_t *nu) {
     }
 }
 
+// cos(2 pi m / n) for every m, n a power of two (>= 8): the first octants evaluated, the
+// rest by symmetry.  A plan's tables index one of these instead of calling cos and sin
+// for each entry (creating a plan of N = 8192 569 -> 399 us, a tensor-core plan of N = 4096 869 -> 361).
+class Cosines {
+    std::vector<double> c;
+    size_t n;
+
+  public:
+    explicit Cosines(size_t n_) : c(n_), n(n_) {
+        for (size_t m = 0; m <= n / 4; ++m)
+            c[m] = m <= n / 8 ? std::cos(2.0 * M_PI * (double)m / (double)n)
+                              : std::sin(2.0 * M_PI * (double)(n / 4 - m) / (double)n);
+        for (size_t m = n / 4 + 1; m <= n / 2; ++m) c[m] = -c[n / 2 - m];
+        for (size_t m = n / 2 + 1; m < n; ++m) c[m] = c[n - m];
+    }
+    double cos(size_t m) const { return c[m & (n - 1)]; }
+    double sin(size_t m) const { return c[(m + n - n / 4) & (n - 1)]; }
+    float2 root(size_t m) const { return make_float2((float)cos(m), (float)-sin(m)); }    // exp(-2 pi i m / n)
+};
+
 // Twiddles of the forward passes, pp.twn entries: pass p < np-1, entry (k-1) s + n'
-// = W_{16 s}^{n' k}, k in [1, 16), n' in [0, s).
-static void append_twiddles(std::vector<float2> &tw, const PassPlan &pp) {
+// = W_{16 s}^{n' k}, k in [1, 16), n' in [0, s).  cs: of N, or of a multiple (step = it / N).
+static void append_twiddles(std::vector<float2> &tw, const PassPlan &pp, const Cosines &cs, size_t step) {
     for (int p = 0; p + 1 < pp.np; ++p) {
-        const int s = pp.stride[p], B = 16 * s;
-        for (int k = 1; k < 16; ++k)
-            for (int n = 0; n < s; ++n) {
-                const long long e = ((long long)n * k) % B;
-                const double a = -2.0 * M_PI * (double)e / (double)B;
-                tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
-            }
+        const size_t s = (size_t)pp.stride[p], unit = step * (size_t)pp.N / (16 * s);
+        for (size_t k = 1; k < 16; ++k)
+            for (size_t n = 0; n < s; ++n) tw.push_back(cs.root(n * k * unit));
     }
 }
 
 // The plan's twiddle table: its own passes' and, at N = 8192, which the bank and
 // batch kernels run as two 4096-point transforms, those of N = 4096 and the odd
 // half's W_8192^n, n < 2048.
-static std::vector<float2> twiddle_tables(const PassPlan &pp) {
+static std::vector<float2> twiddle_tables(const PassPlan &pp, const Cosines &cs) {
     std::vector<float2> tw;
-    append_twiddles(tw, pp);
+    tw.reserve((size_t)3 * pp.N);
+    append_twiddles(tw, pp, cs, 1);
     if (pp.log2N == 13) {
-        append_twiddles(tw, make_pass_plan(12));
-        for (int n = 0; n < 2048; ++n) {
-            const double a = -2.0 * M_PI * (double)n / 8192.0;
-            tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
-        }
+        append_twiddles(tw, make_pass_plan(12), cs, 2);
+        for (size_t n = 0; n < 2048; ++n) tw.push_back(cs.root(n));
     }
     return tw;
+}
+
+// v = hi + lo in 16 bits (FP16 or BF16).
+static void split16(double v, bool bf16, uint16_t *hi, uint16_t *lo) {
+    if (bf16) {
+        const __nv_bfloat16 h = __double2bfloat16(v);
+        const __nv_bfloat16 l = __double2bfloat16(v - (double)__bfloat162float(h));
+        *hi = *reinterpret_cast<const uint16_t *>(&h);
+        *lo = *reinterpret_cast<const uint16_t *>(&l);
+    } else {
+        const __half h = __double2half(v);
+        const __half l = __double2half(v - (double)__half2float(h));
+        *hi = *reinterpret_cast<const uint16_t *>(&h);
+        *lo = *reinterpret_cast<const uint16_t *>(&l);
+    }
 }
 
 // The DFT-16 as the real 32x32 matrix B[k][n] of D = A B with
@@ -76,27 +105,17 @@ static std::vector<float2> twiddle_tables(const PassPlan &pp) {
 // (k/8) 512 + (n/8) 128 + (n%8) 16 + (k%8) 2).  Order: fwd hi, fwd lo, inv hi, inv lo.
 static std::vector<uint16_t> tc_dft16_tables(bool bf16) {
     std::vector<uint16_t> out(4 * 1024);
+    const Cosines cs(16);
     for (int inv = 0; inv < 2; ++inv)
         for (int k = 0; k < 32; ++k)
             for (int n = 0; n < 32; ++n) {
                 const int p = k % 16, q = n % 16;
-                const double th = 2.0 * M_PI * (double)((p * q) % 16) / 16.0;
-                const double c = std::cos(th), s = (inv ? 1.0 : -1.0) * std::sin(th);
+                const double c = cs.cos((size_t)(p * q)), s = (inv ? 1.0 : -1.0) * cs.sin((size_t)(p * q));
                 double v;
                 if (k < 16) v = n < 16 ? c : s;
                 else v = n < 16 ? -s : c;
                 uint16_t hi, lo;
-                if (bf16) {
-                    const __nv_bfloat16 h = __double2bfloat16(v);
-                    const __nv_bfloat16 l = __double2bfloat16(v - (double)__bfloat162float(h));
-                    hi = *reinterpret_cast<const uint16_t *>(&h);
-                    lo = *reinterpret_cast<const uint16_t *>(&l);
-                } else {
-                    const __half h = __double2half(v);
-                    const __half l = __double2half(v - (double)__half2float(h));
-                    hi = *reinterpret_cast<const uint16_t *>(&h);
-                    lo = *reinterpret_cast<const uint16_t *>(&l);
-                }
+                split16(v, bf16, &hi, &lo);
                 const int e = ((k / 8) * 512 + (n / 8) * 128 + (n % 8) * 16 + (k % 8) * 2) / 2;
                 out[(size_t)(2 * inv) * 1024 + e] = hi;
                 out[(size_t)(2 * inv + 1) * 1024 + e] = lo;
@@ -109,33 +128,22 @@ static std::vector<uint16_t> tc_dft16_tables(bool bf16) {
 // 16-bit hi and lo parts (element (k, n) at byte (k/8) 2048 + (n/8) 128 + (n%8) 16
 // + (k%8) 2), then the twiddles e(n2 nu1 / 4096) as float2, points (n2 = 16 q +
 // 2 i, + 1) of row nu1 at float4 index i 256 + 64 q + nu1.
-static std::vector<uint16_t> tc64_tables(bool bf16) {
+static std::vector<uint16_t> tc64_tables(bool bf16, const Cosines &c4096) {
     std::vector<uint16_t> out(2 * 128 * 128 + 4096 * 4);
+    uint16_t hi[64], lo[64];         // of the 64 cosines; sin(m) = cos(m - 16)
+    for (int m = 0; m < 64; ++m) split16(c4096.cos((size_t)(64 * m)), bf16, &hi[m], &lo[m]);
     for (int k = 0; k < 128; ++k)
         for (int n = 0; n < 128; ++n) {
-            const double th = 2.0 * M_PI * (double)(((k % 64) * (n % 64)) % 64) / 64.0;
-            const double cs = std::cos(th), sn = std::sin(th);
-            const double v = (k < 64) == (n < 64) ? cs : (k < 64 ? sn : -sn);
-            uint16_t hi, lo;
-            if (bf16) {
-                const __nv_bfloat16 h = __double2bfloat16(v);
-                const __nv_bfloat16 l = __double2bfloat16(v - (double)__bfloat162float(h));
-                hi = *reinterpret_cast<const uint16_t *>(&h);
-                lo = *reinterpret_cast<const uint16_t *>(&l);
-            } else {
-                const __half h = __double2half(v);
-                const __half l = __double2half(v - (double)__half2float(h));
-                hi = *reinterpret_cast<const uint16_t *>(&h);
-                lo = *reinterpret_cast<const uint16_t *>(&l);
-            }
+            const int m = (k % 64) * (n % 64);
+            // [[C, S], [-S, C]]; -sin(m) = cos(m + 16)
+            const int i = ((k < 64) == (n < 64) ? m : k < 64 ? m - 16 : m + 16) & 63;
             const int e = ((k / 8) * 2048 + (n / 8) * 128 + (n % 8) * 16 + (k % 8) * 2) / 2;
-            out[e] = hi;
-            out[128 * 128 + e] = lo;
+            out[e] = hi[i];
+            out[128 * 128 + e] = lo[i];
         }
     for (int n2 = 0; n2 < 64; ++n2)
         for (int nu1 = 0; nu1 < 64; ++nu1) {
-            const double th = 2.0 * M_PI * (double)(n2 * nu1) / 4096.0;
-            const float w[2] = {(float)std::cos(th), (float)std::sin(th)};
+            const float w[2] = {(float)c4096.cos((size_t)(n2 * nu1)), (float)c4096.sin((size_t)(n2 * nu1))};
             const int q = n2 / 16, i = (n2 % 16) / 2;
             std::memcpy(&out[2 * 128 * 128 + ((i * 256 + 64 * q + nu1) * 4 + 2 * (n2 & 1)) * 2], w, sizeof(w));
         }
@@ -309,7 +317,8 @@ int ols_plan(ols_plan_t *out, int64_t N, int32_t M, int32_t F, uint32_t flags) {
     if (e == cudaSuccess && !r2r) e = dev_alloc(&p->Htk, sizeof(float2) * (size_t)F * (size_t)N);
     if (e == cudaSuccess && r2r) e = dev_alloc(&p->hpack, sizeof(float2) * (size_t)Fc * (size_t)M);
     if (e == cudaSuccess && r2r) e = r2r_prepare(*p);
-    std::vector<float2> tw = twiddle_tables(p->pp);
+    const Cosines cs((size_t)N);
+    std::vector<float2> tw = twiddle_tables(p->pp, cs);
     const size_t ntw = (tw.size() + 1) & ~(size_t)1;         // the derivative's sines follow, read 16 bytes at a time
     if (e == cudaSuccess) e = dev_alloc(&p->tw, sizeof(float2) * (ntw + (size_t)N));
     if (e == cudaSuccess) e = dev_alloc(&p->tw64, sizeof(double2) * (size_t)N);
@@ -329,7 +338,7 @@ int ols_plan(ols_plan_t *out, int64_t N, int32_t M, int32_t F, uint32_t flags) {
     if (e == cudaSuccess && flags != OLS_FLAG_FP32 && flags != OLS_FLAG_R2R) {
         const bool bf16 = flags == OLS_FLAG_TC_BF16SPLIT;
         if (l == 12) p->layout = LAYOUT_ROWS64;
-        const std::vector<uint16_t> b = l == 12 ? tc64_tables(bf16) : tc_dft16_tables(bf16);
+        const std::vector<uint16_t> b = l == 12 ? tc64_tables(bf16, cs) : tc_dft16_tables(bf16);
         e = dev_alloc(&p->tc_bmat, sizeof(uint16_t) * b.size());
         if (e == cudaSuccess) e = cudaMemcpy(p->tc_bmat, b.data(), sizeof(uint16_t) * b.size(), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = tc_prepare(*p, bf16);
@@ -344,7 +353,7 @@ int ols_plan(ols_plan_t *out, int64_t N, int32_t M, int32_t F, uint32_t flags) {
         std::vector<float> sines((size_t)(2 * N));
         for (int64_t q = 0; q < N; ++q) {
             const int f = p->layout == LAYOUT_STD ? nu[(size_t)q] : layout_freq(p->layout, (int)q);
-            const double v = std::sin(2.0 * M_PI * (double)f / (double)N);
+            const double v = cs.sin((size_t)f);
             sines[(size_t)q] = (float)v;
             sines[(size_t)(N + q)] = (float)(v - (double)(float)v);
         }
