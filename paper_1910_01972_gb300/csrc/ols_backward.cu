@@ -103,7 +103,6 @@ struct BwdGeo {
     static constexpr size_t CLAIM = (228u * 1024u) / (MINB + 1) + 1024u;
     static constexpr size_t SMEM = USED > CLAIM ? USED : CLAIM;
     static constexpr uint32_t TMEM_COLS = (uint32_t)(BLOCK / 128) * 128u;   // a 128-column lane range per 128 threads
-    static_assert(G::XBUFS == 2, "the product buffer is the exchange buffer not in use");
 };
 
 template <int LOG2N, int BLOCK, bool WANT_DS, bool WANT_DH>

@@ -26,9 +26,6 @@
 #include "tmem.cuh"
 
 // Tuning knobs (compile-time; defaults are the measured best on GB300).
-#ifndef OLS_XBUFS
-#define OLS_XBUFS 2          // exchange buffers per segment (2: one barrier per exchange)
-#endif
 #ifndef OLS_WARPS_PER_SM
 #define OLS_WARPS_PER_SM 16  // resident warps per SM the register budget must allow
 #endif
@@ -84,7 +81,7 @@ struct Geo {
     // the exchange between the last two passes goes through TMEM (kernels
     // with TMEM twiddles; columns 64..95 of the thread's block are free)
     static constexpr bool TX = LOG2N >= 9 && LOG2N <= 12;
-    static constexpr int XBUFS = OLS_XBUFS;
+    static constexpr int XBUFS = 2;      // exchange buffers per segment: one barrier per exchange
     static constexpr size_t SMEM = sizeof(float2) * (size_t)(SEGS * XBUFS * PADN);
     // TMEM twiddles: 128 columns per 128 threads (a thread's lane, 32 columns per pass)
     static constexpr uint32_t TMEM_COLS = (uint32_t)(BLOCK / 128) * 128u;
@@ -140,7 +137,6 @@ struct SegmentBarrier {
 // Write x in the layout of pass PW, barrier, read it back in the layout of PR.
 template <int LOG2N, int PW, int PR, class BAR = CtaBarrier>
 __device__ __forceinline__ void exchange(float2 *x, float2 *buf, int t, const BAR &bar = BAR{}) {
-    if constexpr (Geo<LOG2N>::XBUFS == 1) bar();   // previous readers of buf are done
     const int bw = pad_base<LOG2N, PW>(t);
 #pragma unroll
     for (int k = 0; k < 16; ++k) buf[bw + pad_off<LOG2N, PW>(k)] = x[k];
@@ -215,7 +211,6 @@ __device__ __forceinline__ int tx_addr(int t, int k) {
 // The shared-memory exchange of passes 0 and 1 when pass 1 is relabelled.
 template <int LOG2N, int PW, int PR, int XCH, class BAR>
 __device__ __forceinline__ void exchange_tx(float2 *x, float2 *buf, int t, const BAR &bar) {
-    if constexpr (Geo<LOG2N>::XBUFS == 1) bar();
 #pragma unroll
     for (int k = 0; k < 16; ++k) buf[tx_addr<LOG2N, PW, XCH>(t, k)] = x[k];
     bar();
@@ -850,7 +845,7 @@ __device__ __forceinline__ void forward_passes(float2 *x, float2 *bufs, const TW
         if constexpr (tx && P == G::NP - 2) {
             tx_forward<LOG2N, TW::xchg>(x, tw.xbase());
         } else {
-            float2 *buf = bufs + (G::XBUFS == 2 ? (xc & 1) * G::PADN : 0);
+            float2 *buf = bufs + (xc & 1) * G::PADN;
             if constexpr (tx && P + 1 == G::NP - 2) exchange_tx<LOG2N, P, P + 1, TW::xchg>(x, buf, t, bar);
             else exchange<LOG2N, P, P + 1>(x, buf, t, bar);
             ++xc;
@@ -885,7 +880,7 @@ __device__ __forceinline__ void inverse_passes(float2 *x, float2 *bufs, const TW
         if constexpr (tx && P == G::NP - 2) {
             tx_inverse<LOG2N, TW::xchg>(x, tw.xbase());
         } else {
-            float2 *buf = bufs + (G::XBUFS == 2 ? (xc & 1) * G::PADN : 0);
+            float2 *buf = bufs + (xc & 1) * G::PADN;
             if constexpr (tx && P + 1 == G::NP - 2) exchange_tx<LOG2N, P + 1, P, TW::xchg>(x, buf, t, bar);
             else exchange<LOG2N, P + 1, P>(x, buf, t, bar);
             ++xc;

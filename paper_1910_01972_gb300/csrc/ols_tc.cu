@@ -217,7 +217,7 @@ __device__ __forceinline__ void tc_forward_passes(float2 *x, float2 *bufs, const
     }
     if constexpr (P < G::NP - 1) {
         twiddle<LOG2N, P, false>(x, tw, t);
-        exchange<LOG2N, P, P + 1>(x, bufs + (G::XBUFS == 2 ? (xc & 1) * G::PADN : 0), t);
+        exchange<LOG2N, P, P + 1>(x, bufs + (xc & 1) * G::PADN, t);
         ++xc;
         tc_forward_passes<LOG2N, P + 1, BF16>(x, bufs, tw, t, xc, c);
     }
@@ -237,7 +237,7 @@ __device__ __forceinline__ void tc_inverse_pair(float2 *xa, float2 *xb, float2 *
     constexpr float scale = P == G::NP - 1 ? 1.0f : 0.25f;
     // a: enter pass P
     if constexpr (P < G::NP - 1) {
-        exchange<LOG2N, P + 1, P>(xa, bufs + (G::XBUFS == 2 ? (xc & 1) * G::PADN : 0), t);
+        exchange<LOG2N, P + 1, P>(xa, bufs + (xc & 1) * G::PADN, t);
         ++xc;
         twiddle<LOG2N, P, true>(xa, tw, t);
     }
@@ -250,7 +250,7 @@ __device__ __forceinline__ void tc_inverse_pair(float2 *xa, float2 *xb, float2 *
     // b: finish pass P+1, enter pass P
     if constexpr (B_IN_FLIGHT) wait_load(xb, c, 1);
     if constexpr (P < G::NP - 1) {
-        exchange<LOG2N, P + 1, P>(xb, bufs + (G::XBUFS == 2 ? (xc & 1) * G::PADN : 0), t);
+        exchange<LOG2N, P + 1, P>(xb, bufs + (xc & 1) * G::PADN, t);
         ++xc;
         twiddle<LOG2N, P, true>(xb, tw, t);
     }
