@@ -79,6 +79,7 @@ struct BankSegment {
 
 // y[f][j] written once, the aliased samples dropped.
 struct EpiPlain {
+    static constexpr bool WIDE = true;      // 512-thread CTAs at N = 4096 (see bank_launch)
     template <int LOG2N>
     static constexpr bool narrow() { return false; }
     static constexpr int XCH = XCHG_TMEM;
@@ -227,21 +228,21 @@ cudaError_t bank_launch_block(BankArgs a, const EPI &epi, int sm_count, cudaStre
     return cudaGetLastError();
 }
 
-// Block size of a call.  Up to N = 2048 one CTA of 512 threads per SM shares
-// the spectra's L1 lines among the most segments (32 filters, 2^21 samples,
-// blocks of 512 / 256: N = 256 94 / 97 us, 1024 113 / 120, 2048 133 / 141); with fewer
-// than four steps per SM two CTAs of 256 start and end sooner (32 filters,
-// 2^15 samples, N = 2048: 12.5 / 11.0 us; from 2^17 samples on the two are
-// equal).  While CTAs of 128 threads, four per SM, leave at most one step each,
-// they set up sooner and reach more SMs (one filter, 2^16 samples, 256 / 128:
-// N = 256 6.4 / 5.2 us, 512 6.6 / 5.2, 2048 6.6 / 5.4; 32 filters, 2^15 samples, N = 512
-// 9.7 / 8.6, 1024 9.8 / 8.6).  At N = 4096 a 512-thread CTA holds only two segments and 256
-// threads, one segment, were faster throughout (166 / 159 us; one filter, 2^23
-// samples: 52 / 48 us).  N = 8192 needs 512 threads for its one segment.
+// Block size of a call.  One CTA of 512 threads per SM shares the spectra's L1
+// lines among the most segments (32 filters, 2^21 samples, blocks of 512 / 256 / 128: N = 512
+// 107 / 112 / 110 us, 1024 109 / 117 / 115, 2048 135 / 145 / 137; N = 256 93 / 92 / 93).  With fewer
+// than four steps per SM two CTAs of 256 start and end sooner (32 filters, 2^15 samples: N = 256
+// 7.0 / 6.4 us, 1024 8.9 / 7.7, 2048 10.1 / 8.7; from 2^17 samples on the two are within 2%).  While CTAs of
+// 128 threads, four per SM, leave at most one step each, they set up sooner and reach
+// more SMs (one filter, 2^16 samples, 256 / 128: N = 256 4.3 / 3.5 us, 512 5.0 / 3.9, 2048 5.4 / 4.3; 32 filters,
+// 2^15 samples, N = 512 7.4 / 7.2, 2048 8.7 / 7.9).  At N = 4096 a 512-thread CTA holds only two
+// segments: it pays from four spectra per segment on, and not for the derivative and
+// the peaks, whose epilogues spill or stay longer at its barriers (2^22 samples, 512 / 256: 32 filters plain 284 /
+// 310 us, power 282 / 301, derivative 357 / 335, peaks 320 / 315; 8 filters plain 84 / 89; 2 filters 32.5 / 31.6; one
+// filter 23.6 / 21.8).  N = 8192 needs 512 threads for its one segment.
 template <int LOG2N, class EPI>
 cudaError_t bank_prepare() {
-    cudaError_t e = cudaSuccess;
-    if constexpr (LOG2N != 12) e = bank_prepare_block<LOG2N, 512, EPI>();
+    cudaError_t e = bank_prepare_block<LOG2N, 512, EPI>();
     if constexpr (LOG2N != 13) {
         if (e == cudaSuccess) e = bank_prepare_block<LOG2N, 256, EPI>();
     }
@@ -252,15 +253,18 @@ cudaError_t bank_prepare() {
 }
 template <int LOG2N, class EPI>
 cudaError_t bank_launch(const BankArgs &a, const EPI &epi, int sm_count, cudaStream_t st) {
-    if constexpr (LOG2N == 12) {
-        return bank_launch_block<LOG2N, 256>(a, epi, sm_count, st);
-    } else if constexpr (LOG2N == 13) {
+    if constexpr (LOG2N == 13) {
         return bank_launch_block<LOG2N, 512>(a, epi, sm_count, st);
     } else {
         constexpr int SL = 512 / Geo<LOG2N>::T;
         const long long steps = (a.nseg + SL - 1) / SL * a.F;
-        constexpr int SL1 = 128 / Geo<LOG2N>::T;
-        if ((a.nseg + SL1 - 1) / SL1 * a.F <= 4ll * sm_count) return bank_launch_block<LOG2N, 128>(a, epi, sm_count, st);
+        if constexpr (LOG2N == 12) {
+            if (!EPI::WIDE || a.F < 4) return bank_launch_block<LOG2N, 256>(a, epi, sm_count, st);
+        } else {
+            constexpr int SL1 = 128 / Geo<LOG2N>::T;
+            if ((a.nseg + SL1 - 1) / SL1 * a.F <= 4ll * sm_count)
+                return bank_launch_block<LOG2N, 128>(a, epi, sm_count, st);
+        }
         if (steps < 4ll * sm_count) return bank_launch_block<LOG2N, 256>(a, epi, sm_count, st);
         return bank_launch_block<LOG2N, 512>(a, epi, sm_count, st);
     }

@@ -297,9 +297,9 @@ __device__ __forceinline__ void tx11_inverse(float2 *x, uint32_t xb) {
 // a pair sends half of its registers, v[2 (p4 + 2 p5 + 4 p2 + 8 p3) + re/im] with
 // lane bit 0 = p6 <-> x[p3 + 2 p4 + 4 p5 + 8 p6] with lane bit 0 = p2.  Sixteen
 // shuffles and 48 selects take the place of a round trip and its register
-// moves; which is faster depends on the epilogue (32 filters, 2^23 samples:
-// plain store 533 us against 508, real pairs 271 against 274; 16 filters:
-// power 268 against 276, derivative 326 against 316).
+// moves; which is faster depends on the epilogue (2^23 samples, shuffles / two round
+// trips: 32 filters plain 521 / 522 us, real 275 / 274; 16 filters power 259 / 268, detection 262 /
+// 275, derivative 301 / 287, peaks 299 / 291).
 __device__ __forceinline__ void tx11s_forward(float2 *x, uint32_t xb) {
     const bool odd = threadIdx.x & 1;
     float v[32];

@@ -151,13 +151,14 @@ __device__ __noinline__ void derivative_exchange_call(const float2 *x, float2 *d
 
 template <int MODE>
 struct EpiPost {
+    static constexpr bool WIDE = MODE == POST_POWER || MODE == POST_DETECT;
     // two loads of twiddles where one spills
     template <int LOG2N>
     static constexpr bool narrow() {
         return (MODE == POST_DERIV && LOG2N >= 10) || (MODE == POST_PEAK && LOG2N == 12);
     }
-    // POWER: one of the exchange's three bits by shuffles (as the real form)
-    static constexpr int XCH = MODE == POST_POWER ? XCHG_SHFL : XCHG_TMEM;
+    // one of the exchange's three bits by shuffles (as the real form)
+    static constexpr int XCH = WIDE ? XCHG_SHFL : XCHG_TMEM;
     // PEAK: warp-edge powers [2][T/32][16] floats per segment of several warps
     template <int LOG2N>
     static constexpr int edge() {

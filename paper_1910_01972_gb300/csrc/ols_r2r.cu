@@ -48,6 +48,7 @@ cudaError_t launch_pack_real_pairs(const float *h, int M, int F, float2 *g, cuda
 // Real samples in, one inverse FFT per filter pair, its real and imaginary
 // parts stored as the pair's two output rows.
 struct EpiReal {
+    static constexpr bool WIDE = true;
     template <int LOG2N>
     static constexpr bool narrow() { return false; }
     static constexpr int XCH = XCHG_SHFL;

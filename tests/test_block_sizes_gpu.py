@@ -48,3 +48,27 @@ def test_three_block_sizes(N, M):
             ref = oracle.conv(s[:n + M - 1], h[f:f + 1])
             assert oracle.max_stream_rel_l2(y[f:f + 1].cpu().numpy(), ref) <= 2e-6
     plan.close()
+
+
+@pytest.mark.parametrize("M,F", [(513, 4), (513, 9), (4096, 4)])
+def test_block_sizes_at_4096(M, F):
+    """N = 4096: 512-thread CTAs from four steps per SM and four spectra on, else 256."""
+    _build.build()
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    N, L = 4096, 4096 - M + 1
+    short, long = 2 * ((4 * sms - 1) // F), 2 * -(-4 * sms // F) + 1        # segments; steps = ceil(n / 2) F
+    assert -(-short // 2) * F < 4 * sms <= -(-long // 2) * F
+    g = np.random.Generator(np.random.PCG64(M + F))
+    s, h = synth.signal(g, long * L + M - 1), synth.filters(g, F, M)
+    plan = Plan(M, F, N)
+    plan.set_filters(torch.from_numpy(h).cuda())
+    sd = torch.from_numpy(s).cuda()
+    part = sd[:short * L + M - 1].contiguous()
+    for call in (plan.convolve, plan.convolve_power):
+        a, b = call(part), call(sd)
+        assert torch.equal(a, b[:, :a.shape[1]])
+    y = plan.convolve(sd)[F - 1:].cpu().numpy()
+    assert oracle.max_stream_rel_l2(y, oracle.conv(s, h[F - 1:])) <= 2e-6
+    plan.close()
