@@ -9,15 +9,15 @@
 //   BLOCK / (N/16) segments in slots that exchange under barriers of their
 //   own.  What bounds it: FP32 issue and the latency of the exchanges
 //   between the passes, with the 16 resident warps that 128 registers allow;
-//   no unit is saturated (filter bank, N = 2048: FMA pipe 54% of cycles, L1
-//   data path 49%, HBM 64%).
+//   no unit is saturated (filter bank, N = 2048: issue 64% and FMA pipe 57% of cycles, L1
+//   data path 48%; 521 us against an HBM floor of 326).
 // * Spectra of filter f + 1 are loaded into registers while filter f is
 //   transformed.  The slots of a CTA run through the filters side by side, so
 //   those loads hit L1 for most of them: one CTA of 512 threads per SM instead
 //   of four of 128 took L1 hits from 11% to 35% of sectors and L2 reads down
 //   by 31%.  (Spectra copied to shared memory by bulk copies and read from
-//   there at the head of each filter, without registers held: 627 us against
-//   536; the load latency is then exposed 32 times per segment.)
+//   there at the head of each filter, without registers held, were 17% slower;
+//   the load latency is then exposed 32 times per segment.)
 // * Work is shared out in steps (block of segments, filter): the grid is at
 //   most the resident CTAs, each takes the same number of consecutive steps
 //   (give or take one) and transforms a segment again where its share begins
@@ -26,11 +26,10 @@
 //   fills the chip.
 // * Output stores carry the streaming hint, so that they do not push the
 //   spectra out of L1 (2% on the filter bank).
-// Measured before (a CTA of 128 threads per segment group, all filters of it)
-// and after, 32- / 16-filter banks of 2^23 samples: N = 256 170 -> 141 us
-// (3e6 samples), N = 512 247 -> 228, N = 1024 251 -> 224, N = 2048 530 -> 507,
-// N = 4096 358 -> 314; 24 filters, 2^22 samples, N = 8192 360 -> 322 us; 65521
-// samples of 32 filters at N = 2048: 35 -> 12 us.
+// Device time (us) before (a CTA of 128 threads per segment group, all filters of it)
+// and after, plain form, 32 filters of 2^22 samples: N = 256 (3e6 samples) 166 -> 142, 512
+// 253 -> 208, 1024 257 -> 212, 2048 279 -> 262, 4096 333 -> 285, 8192 (24 filters) 340 -> 312;
+// 65521 samples of 32 filters at N = 2048: 33 -> 10.
 #pragma once
 
 #include <cstdint>

@@ -641,7 +641,8 @@ struct TwGlobal {
 // Tried and taken back: the twiddles folded into radix-2 butterflies s = a + W b,
 // d = 2 a - s, eight factors per pass and 192 FP32 lane operations per DFT-16 instead
 // of 220.  It was faster where the kernel is bound by FP32 issue (32 filters, 2^23
-// samples, N = 2048: 510 us against 525; real pairs 273 / 280; power at N = 4096 182 / 188;
+// samples, N = 2048: 510 us against 525; real pairs 273 / 280; power at N = 4096, 256-thread
+// CTAs, 182 / 188;
 // N = 256, 512, 1024 and 8192 equal or slower), but d inherits the rounding of s and the
 // results' error against 64 bits grew by 4 to 8%; with d formed like s (256 operations,
 // more than the plain form) it still was up to 2% larger.

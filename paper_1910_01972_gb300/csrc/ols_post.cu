@@ -177,10 +177,10 @@ struct EpiPost {
     // for all its filters, so the inverse FFT yields the derivative itself and
     // no output needs its neighbours.  A segment holding the first or the last
     // output of the stream, whose differences are one-sided, keeps its plain
-    // spectrum and goes through the neighbour exchange below.  16- / 32-filter
-    // banks of 2^23 samples (N = 1024 / 2048): the exchange for every segment
-    // took 212 / 404 us (one CTA of 128 threads per segment group, one fewer
-    // per SM for its registers), this 142 / 317.
+// spectrum and goes through the neighbour exchange below.  Device time of the
+    // exchange for every segment (one CTA of 128 threads per segment group, one fewer per SM
+    // for its registers) and of this, 16 filters: N = 1024, 2^22 samples 210 -> 125 us; N = 2048,
+    // 2^23 samples 402 -> 286.
     __device__ __forceinline__ static bool at_end(const BankSegment &sg) {
         return sg.j0 == 0 || sg.Nout - sg.j0 == (long long)sg.span;
     }

@@ -31,8 +31,8 @@
 // threads about 2900 issue cycles beside them, of 5700 that a step takes.
 // Three radix-16 stages (ols_tc.cu) need a third of the multiply-adds but split,
 // store, wait and exchange three times, and their threads' work bounds them:
-// 64 filters, 2^22 samples 1156 us there, 733 here (FP16; the FP32 kernel 620).
-// Spectra prefetched a filter ahead 761 us: their registers spill.
+// 64 filters, 2^22 samples 1146 us there, 734 here (FP16; the FP32 kernel 569).
+// Spectra prefetched a filter ahead were 4% slower: their registers spill.
 // Scale (an exact power of two): the segment's spectrum x 16, undone in the output.
 // Both inverse operands, Y and Z, are averages of phase-rotated outputs of the
 // segment's circular convolution, so |Y|, |Z| <= |s| sqrt(M) for a unit-L2 filter (a
