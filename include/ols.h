@@ -85,7 +85,8 @@ typedef struct ols_batch_s *ols_batch_t;
  * significant bits per operand; BF16 split: ~16 bits.  Input range: the
  * FP16 form assumes |s| <= 1.42 and unit-L2 filters (larger inputs should be
  * scaled by a power of two; outside that range 16-bit operands can
- * overflow).  Forward convolution only (ols_convolve, ols_convolve_host). */
+ * overflow; below about 2^-3 its operands lose bits, so that fainter inputs
+ * should be scaled up).  Forward convolution only (ols_convolve, ols_convolve_host). */
 #define OLS_FLAG_TC_FP16SPLIT 1u
 #define OLS_FLAG_TC_BF16SPLIT 2u
 /* Real-to-real convolution (Sec. 3.4's R2R variant and Algorithm 2 with
